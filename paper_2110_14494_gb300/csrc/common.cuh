@@ -14,7 +14,12 @@ constexpr double kQ = 1.602176634e-19;     // elementary charge, C
 constexpr double kMe = 9.1093837015e-31;   // electron mass, kg
 constexpr double kEps0 = 8.8541878128e-12; // vacuum permittivity, F/m
 constexpr int kMaxProc = PIC_MAX_PROC;
-constexpr int kTableStride = 8;            // processes per table row (7 used + total)
+// A rate table of n_bins nodes: n_bins rows of kTableRow reals (the rates of
+// seven processes, then 0), then for each node the total rate and its
+// difference to the next node's.  Every draw reads one pair of the totals
+// (8 KB of single precision for 1000 nodes, all of it in L1), only a draw that
+// may collide the two rows around its energy, 64 consecutive bytes.
+constexpr int kTableRow = 8, kTableStride = kTableRow + 2;  // kTableStride: reals per node in all
 constexpr int kNMom = PIC_SWARM_NMOM;
 constexpr unsigned kFull = 0xffffffffu;
 constexpr double kPi = 3.14159265358979323846;
@@ -96,9 +101,16 @@ inline Keys make_keys(uint64_t seed) {
     return k;
 }
 
-// Top 23 bits of a word, centred in their bin: exact in binary32 and binary64.
-template <class T> __device__ __forceinline__ T unif(uint32_t w) {
-    return ((T)(w >> 9) + (T)0.5) * (T)(1.0 / 8388608.0);
+// Top 23 bits of a word, centred in their bin: exact in binary32 and binary64
+// (there by placing the 24 bits 2 (w >> 9) + 1 below the leading bit of 1: one
+// subtraction on the narrow double pipe instead of a conversion and two operations).
+template <class T> __device__ __forceinline__ T unif(uint32_t w);
+template <> __device__ __forceinline__ float unif<float>(uint32_t w) {
+    return ((float)(w >> 9) + 0.5f) * (float)(1.0 / 8388608.0);
+}
+template <> __device__ __forceinline__ double unif<double>(uint32_t w) {
+    const unsigned long long m = (unsigned long long)((w >> 8) | 1u) << 28;
+    return __longlong_as_double((long long)(0x3ff0000000000000ull | m)) - 1.0;
 }
 
 __device__ __forceinline__ u32x4 draw_words(const Keys& K, uint64_t id, uint32_t step, uint32_t k) {

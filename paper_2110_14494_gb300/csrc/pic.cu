@@ -121,25 +121,36 @@ static int grid_n(long long n, int cap_blocks = 0) {
 
 // ================================================================== kernels
 // Rate table (Sec. 2.1.1 / 2.1.5): nu_k(eps_j) = N_k sigma_k(eps_j) v(eps_j) with
-// v = sqrt(2 e eps / m_e), evaluated in float64; row j holds the n_proc rates
-// and, in column 7, their sum; nu_max = max_j of the sum.
+// v = sqrt(2 e eps / m_e), evaluated in float64; row j holds the n_proc rates,
+// the pair of node j their sum and its difference to node j + 1 (both rounded
+// to T first; 0 at the last node); nu_max = max_j of the sum.  A block of y
+// index s builds the table of gas s (densities at dens + s n_proc): the 256
+// gases of a batched run take one launch instead of 4 us each.
 template <class T>
 __global__ void k_rate_table(const double* __restrict__ eps, const double* __restrict__ sigma,
                              const double* __restrict__ dens, int n_proc, int n_bins, T* __restrict__ tab,
-                             double* __restrict__ tab64, unsigned long long* numax_bits) {
+                             unsigned long long* numax_bits) {
     const int j = blockIdx.x * blockDim.x + threadIdx.x;
     if (j >= n_bins) return;
-    const double v = sqrt(2.0 * kQ * eps[j] / kMe);
-    double tot = 0.0;
-    for (int k = 0; k < kTableStride; ++k) {
-        double r = 0.0;
-        if (k < n_proc) r = dens[k] * sigma[k * n_bins + j] * v;
-        if (k < 7) { tab[j * kTableStride + k] = (T)r; tab64[j * kTableStride + k] = r; }
+    dens += (size_t)blockIdx.y * n_proc;
+    tab += (size_t)blockIdx.y * n_bins * kTableStride;
+    const int j1 = j + 1 < n_bins ? j + 1 : j;
+    const double v = sqrt(2.0 * kQ * eps[j] / kMe), v1 = sqrt(2.0 * kQ * eps[j1] / kMe);
+    double tot = 0.0, tot1 = 0.0;
+    for (int k = 0; k < kTableRow; ++k) {
+        double r = 0.0, r1 = 0.0;
+        if (k < n_proc) {
+            r = dens[k] * sigma[k * n_bins + j] * v;
+            r1 = dens[k] * sigma[k * n_bins + j1] * v1;
+        }
+        tab[j * kTableRow + k] = (T)r;
         tot += r;
+        tot1 += r1;
     }
-    tab[j * kTableStride + 7] = (T)tot;
-    tab64[j * kTableStride + 7] = tot;
-    atomicMax(numax_bits, (unsigned long long)__double_as_longlong(tot));
+    T* pair = tab + (size_t)n_bins * kTableRow + 2 * j;
+    pair[0] = (T)tot;
+    pair[1] = (T)tot1 - (T)tot;
+    atomicMax(numax_bits + blockIdx.y, (unsigned long long)__double_as_longlong(tot));
 }
 
 // Initial seeding (Sec. 2.3, Eq. 7 read with a negative exponent): per cell
@@ -929,7 +940,7 @@ static size_t al256(size_t x) { return (x + 255) & ~(size_t)255; }
 
 struct Layout {
     size_t total = 0;
-    size_t buf[2], cq[2], table, table64, E4, E4b, qe, qp, qn, st, cnt, start, sums, key, rank, msc, gas, rho, phi,
+    size_t buf[2], cq[2], table, E4, E4b, qe, qp, qn, st, cnt, start, sums, key, rank, msc, gas, rho, phi,
         phi_prev, phi_x, phi_y, mg, photo, hostio;
 };
 
@@ -957,7 +968,6 @@ static Layout make_layout(const pic_config* c) {
     }
     const int nb = c->gas.n_bins > 0 ? c->gas.n_bins : 2;
     L.table = take((size_t)nb * kTableStride * R);
-    L.table64 = take((size_t)nb * kTableStride * 8);
     L.E4 = take(ncell * 4 * R);
     // float32 Cartesian coupled contexts alternate between two packed fields
     // (the solve writes the one the current push does not read)
@@ -1261,12 +1271,10 @@ static int build_table(pic_ctx* c) {
     cudaMemsetAsync(nmx, 0, 8, c->s);
     if (c->prec == 32)
         k_rate_table<float><<<(nb + 127) / 128, 128, 0, c->s>>>(d, d + nb, d + (size_t)nb * (np + 1), np, nb,
-                                                                (float*)(c->ws + c->L.table),
-                                                                (double*)(c->ws + c->L.table64), nmx);
+                                                                (float*)(c->ws + c->L.table), nmx);
     else
         k_rate_table<double><<<(nb + 127) / 128, 128, 0, c->s>>>(d, d + nb, d + (size_t)nb * (np + 1), np, nb,
-                                                                 (double*)(c->ws + c->L.table),
-                                                                 (double*)(c->ws + c->L.table64), nmx);
+                                                                 (double*)(c->ws + c->L.table), nmx);
     unsigned long long bits = 0;
     e = cudaMemcpyAsync(&bits, nmx, 8, cudaMemcpyDeviceToHost, c->s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(c->s);
@@ -1319,8 +1327,11 @@ extern "C" int pic_init(const pic_config* cfg, void* d_ws, size_t ws_bytes, cons
     int dev = 0, sms = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    const int bps = c->prec == 32 ? PushLaunch<float>::blocks_per_sm(MODE_PIC, c->n_bins)
-                                  : PushLaunch<double>::blocks_per_sm(MODE_PIC, c->n_bins);
+    // Double precision: two blocks of four warps an SM fill the double pipe, and a warp that takes many
+    // electrons in turn keeps its lanes busy (2e5 electrons: two blocks 7.9 ms a step, four 8.15, one 8.3).
+    int bps = c->prec == 32 ? PushLaunch<float>::blocks_per_sm(MODE_PIC, c->n_bins)
+                            : PushLaunch<double>::blocks_per_sm(MODE_PIC, c->n_bins);
+    if (c->prec == 64 && bps > 2) bps = 2;
     c->grid_push = sms * bps;
     if (cfg->coupled) {
         if (c->g.axi) {
@@ -1347,6 +1358,7 @@ template <class T> static PushArgs<T> make_args(pic_ctx* c, int mode) {
     A.cq = c->childq<T>(0);
     A.cq2 = c->childq<T>(1);
     A.gen = 0;
+    A.sms = device_sms();
     A.st = c->st();
     A.table = (const T*)(c->ws + c->L.table);
     A.n_bins = c->n_bins;
@@ -1357,7 +1369,7 @@ template <class T> static PushArgs<T> make_args(pic_ctx* c, int mode) {
     A.eps_lo = (T)c->cfg.gas.eps[0];
     A.eps_hi = (T)c->cfg.gas.eps[c->n_bins - 1];
     A.nu_max = (T)c->nu_max;
-    A.tau_scale = (T)(-0.69314718055994530942 / c->nu_max);
+    A.tau_scale = flight_scale<T>(c->nu_max);
     A.inv_dl2 = (T)(0.69314718055994530942 * c->inv_dl);
     A.l0t = (T)(c->l0 * c->inv_dl);
     A.dt = (T)c->dt_cur;
@@ -2362,7 +2374,7 @@ static size_t swarm_extra(const swarm_config* sc) {
 
 struct BatchLayout {
     size_t total, ctx, ctx_bytes, buf[2], cq[2], csw[2], cnt_in, cnt_out, prefix, bd, Ez, mom, counts, zref, zhist;
-    size_t tabs, numax, tau, dens, nmx, tab64;  // per-swarm rate tables
+    size_t tabs, numax, tau, dens, nmx;  // per-swarm rate tables
     long long segs, cap_child;
 };
 
@@ -2404,7 +2416,6 @@ static BatchLayout batch_layout(const swarm_config* sc, int n) {
     L.tau = take((size_t)n * R);
     L.dens = take((size_t)n * np * 8);
     L.nmx = take((size_t)n * 8);
-    L.tab64 = take((size_t)nb * kTableStride * 8);
     L.total = o;
     return L;
 }
@@ -2577,10 +2588,8 @@ template <class T> struct BatchRunner {
         T* tabs = (T*)(ws + L.tabs);
         cudaError_t e = cudaMemcpyAsync(d_dens, dens.data(), dens.size() * 8, cudaMemcpyHostToDevice, s);
         if (e == cudaSuccess) e = cudaMemsetAsync(d_nmx, 0, (size_t)n * 8, s);
-        for (int i = 0; i < n && e == cudaSuccess; ++i) {
-            k_rate_table<T><<<(nb + 127) / 128, 128, 0, s>>>(d_gas, d_gas + nb, d_dens + (size_t)i * np, np, nb,
-                                                             tabs + (size_t)i * nb * kTableStride,
-                                                             (double*)(ws + L.tab64), d_nmx + i);
+        if (e == cudaSuccess) {
+            k_rate_table<T><<<dim3((nb + 127) / 128, n), 128, 0, s>>>(d_gas, d_gas + nb, d_dens, np, nb, tabs, d_nmx);
             e = cudaGetLastError();
         }
         std::vector<unsigned long long> bits((size_t)n);
@@ -2593,7 +2602,7 @@ template <class T> struct BatchRunner {
             memcpy(&v, &bits[i], 8);
             if (!(v > 0.0)) return PIC_ERR_ARG;
             numax[i] = (T)v;
-            tau[i] = (T)(-0.69314718055994530942 / v);
+            tau[i] = flight_scale<T>(v);
         }
         e = cudaMemcpyAsync(ws + L.numax, numax.data(), (size_t)n * sizeof(T), cudaMemcpyHostToDevice, s);
         if (e == cudaSuccess) e = cudaMemcpyAsync(ws + L.tau, tau.data(), (size_t)n * sizeof(T), cudaMemcpyHostToDevice, s);

@@ -27,8 +27,9 @@ template <class T> struct PushArgs {
     ChildQ<T> cq, cq2;         // product queues: parents fill cq; children generation g reads
                                // (g even ? cq : cq2) and spills into the other one
     int gen;
+    int sms;                   // multiprocessors of the device (work distribution)
     DevState* st;
-    const T* table;            // [n_bins][8]: nu_0..nu_{n_proc-1}, zeros, total
+    const T* table;            // rate table (see kTableRow)
     int n_bins, n_proc;
     int kind[8];
     T thr[8];                  // eV
@@ -36,7 +37,7 @@ template <class T> struct PushArgs {
     T l0, inv_dl;              // ln(eps_0), (n_bins-1) / (ln eps_last - ln eps_0), in T
     T eps_lo, eps_hi;          // eV
     T nu_max;
-    T tau_scale;               // -ln 2 / nu_max: single-precision flight times from base-2 logarithms
+    T tau_scale;               // flight-time factor (flight_scale)
     T inv_dl2, l0t;            // ln 2 * inv_dl and l0 * inv_dl: table coordinate from a base-2 logarithm
     T dt;                      // duration of this step
     T dt_kick;                 // duration of the previous step (the half-kick completes its Eq. 2)
@@ -80,12 +81,33 @@ template <class T> struct ProcSmem {
 };
 
 // ------------------------------------------------------------------ arithmetic
+// Double-precision arithmetic runs on two lanes a clock per multiprocessor,
+// so a double operation costs a warp sixteen clocks whatever its lanes do; the
+// helpers below give the values of the plain expressions with fewer of them.
+// x / c for a constant c with rc = 1 / c rounded to nearest: the quotient's
+// estimate is corrected to within one unit in the last place, and the last
+// correction by its exact remainder then rounds correctly (Markstein, IBM J.
+// Res. Dev. 34, 1990, theorem on division by a correctly rounded reciprocal).
+__device__ __forceinline__ double div_const(double x, double c, double rc) {
+    double q = __dmul_rn(x, rc);
+    q = __fma_rn(__fma_rn(-c, q, x), rc, q);
+    return __fma_rn(__fma_rn(-c, q, x), rc, q);
+}
+// max(x, 0) with dmax's choice for NaN (0): not negative and not NaN as integers.
+__device__ __forceinline__ float max0(float x) { return dmax(x, 0.0f); }
+__device__ __forceinline__ double max0(double x) {
+    return (unsigned long long)__double_as_longlong(x) <= 0x7ff0000000000000ull ? x : 0.0;
+}
+// a >= b of positive values.
+__device__ __forceinline__ bool ge_pos(float a, float b) { return a >= b; }
+__device__ __forceinline__ bool ge_pos(double a, double b) { return __double_as_longlong(a) >= __double_as_longlong(b); }
+
 // Double precision follows the oracle's operation order (no FMA contraction in
 // that translation unit); single precision uses precomputed factors.
 template <class T> struct Arith;
 template <> struct Arith<double> {
-    static __device__ __forceinline__ double energy(double v2) { return 0.5 * kMe * v2 / kQ; }
-    static __device__ __forceinline__ double speed(double e) { return sqrt(2.0 * kQ * e / kMe); }
+    static __device__ __forceinline__ double energy(double v2) { return div_const(0.5 * kMe * v2, kQ, 1.0 / kQ); }
+    static __device__ __forceinline__ double speed(double e) { return sqrt(div_const(2.0 * kQ * e, kMe, 1.0 / kMe)); }
     static __device__ __forceinline__ double lg(double u) { return log(u); }
     static __device__ __forceinline__ double tau(double u0, double nu_max) { return -log(u0) / nu_max; }
     static __device__ __forceinline__ void sc2pi(double u, double* s, double* c) { sincospi(2.0 * u, s, c); }
@@ -98,9 +120,21 @@ template <> struct Arith<float> {
     static __device__ __forceinline__ void sc2pi(float u, float* s, float* c) { sincospif(2.0f * u, s, c); }
 };
 
+// cos and sin of the polar angle, cos = 1 - 2 u2.  In double precision 2 u2
+// and ct^2 are exact (u2 has 24 bits), so each fused operation rounds as the
+// two it replaces, and 1 - ct^2 is at least 2^-23.
+__device__ __forceinline__ void polar(float u2, float& ct, float& st) {
+    ct = 1.0f - 2.0f * u2;
+    st = sqrtf(dmax(0.0f, 1.0f - ct * ct));
+}
+__device__ __forceinline__ void polar(double u2, double& ct, double& st) {
+    ct = __fma_rn(-2.0, u2, 1.0);
+    st = sqrt(__fma_rn(-ct, ct, 1.0));
+}
+
 template <class T> __device__ __forceinline__ void iso_dir(T u2, T u3, T n[3]) {
-    T ct = (T)1 - (T)2 * u2;
-    T st = sqrt(dmax((T)0, (T)1 - ct * ct));
+    T ct, st;
+    polar(u2, ct, st);
     T s, c;
     Arith<T>::sc2pi(u3, &s, &c);
     n[0] = st * c;
@@ -111,6 +145,11 @@ template <class T> __device__ __forceinline__ void iso_dir(T u2, T u3, T n[3]) {
 template <class T> __device__ __forceinline__ void fly(T x[3], T v[3], const T a[3], T tau) {
 #pragma unroll
     for (int d = 0; d < 3; ++d) {
+        // a field along one axis (swarms): the other two only drift
+        if (sizeof(T) == 8 && (__double_as_longlong((double)a[d]) << 1) == 0) {
+            x[d] = x[d] + tau * v[d];
+            continue;
+        }
         x[d] = x[d] + tau * (v[d] + (T)0.5 * tau * a[d]);
         v[d] = v[d] + tau * a[d];
     }
@@ -349,9 +388,13 @@ __device__ __forceinline__ void deposit_at(const PushArgs<T>& A, T x0, T x1, T x
 // (far below a cell crossing), a table coordinate one near 1e-5 of a bin, and
 // the scattering cosine a reciprocal square root.
 // The collision rates a candidate event is tested against: the table
-// ([n_bins][8]: the rates, zeros, their total), its maximum total nu_max and
-// -ln 2 / nu_max.  One gas for a PIC context; batched swarms of different
+// (see kTableRow), its maximum total nu_max and the flight_scale of that.  One gas for a PIC context; batched swarms of different
 // compositions each have their own.
+// Factor of the flight times: -ln 2 / nu_max in single precision (times a
+// base-2 logarithm), 1 / nu_max in double (div_const).
+template <class T> inline T flight_scale(double nu_max) {
+    return (T)((sizeof(T) == 4 ? -0.69314718055994530942 : 1.0) / nu_max);
+}
 template <class T> struct Rates {
     const T* tab;
     T nu_max, tau_scale;
@@ -360,7 +403,7 @@ template <class T> struct Rates {
 template <class T> struct EvArith;
 template <> struct EvArith<double> {
     static __device__ __forceinline__ double flight(const Rates<double>& R, double u0) {
-        return -log(u0) / R.nu_max;
+        return div_const(-log(u0), R.nu_max, R.tau_scale);
     }
     static __device__ __forceinline__ double coord(const PushArgs<double>& A, double e) {
         return (log(e) - A.l0) * A.inv_dl;
@@ -372,7 +415,7 @@ template <> struct EvArith<double> {
 };
 template <> struct EvArith<float> {
     static __device__ __forceinline__ float flight(const Rates<float>& R, float u0) {
-        return __log2f(u0) * R.tau_scale;
+        return __fmul_rn(__log2f(u0), R.tau_scale);
     }
     static __device__ __forceinline__ float coord(const PushArgs<float>& A, float e) {
         return fmaf(__log2f(e), A.inv_dl2, -A.l0t);
@@ -380,52 +423,90 @@ template <> struct EvArith<float> {
     static __device__ __forceinline__ float cosine(float dot, float v2) { return v2 > 0.0f ? dot * rsqrtf(v2) : 0.0f; }
 };
 
-// Index and fraction in the table, linear in ln(eps), clamped at both ends.
-template <class T>
-__device__ __forceinline__ void table_pos(const PushArgs<T>& A, T e, int& j, T& f, LStats& ls) {
+// Coordinate in the table, linear in ln(eps), clamped at both ends.
+template <class T> __device__ __forceinline__ T table_pos(const PushArgs<T>& A, T e, LStats& ls) {
     if (e <= A.eps_lo) {
-        j = 0; f = (T)0;
         if (e < A.eps_lo) ++ls.clamped;
-    } else if (e >= A.eps_hi) {
-        j = A.n_bins - 2; f = (T)1;
-        if (e > A.eps_hi) ++ls.clamped;
-    } else {
-        T t = EvArith<T>::coord(A, e);
-        int jj = (int)floor(t);
-        if (jj > A.n_bins - 2) jj = A.n_bins - 2;
-        if (jj < 0) jj = 0;
-        j = jj;
-        f = t - (T)jj;
+        return (T)0;
     }
+    if (e >= A.eps_hi) {
+        if (e > A.eps_hi) ++ls.clamped;
+        return (T)(A.n_bins - 1);
+    }
+    return EvArith<T>::coord(A, e);
+}
+// Its node and the fraction towards the next one.
+template <class T> __device__ __forceinline__ void table_split(const PushArgs<T>& A, T t, int& j, T& f) {
+    if (sizeof(T) == 8) {
+        // floor by adding 1.5 2^52 rounded down: the integer stands in the low word
+        const double big = 6755399441055744.0, r = __dadd_rd((double)t, big);
+        const int j0 = __double2loint(r);
+        j = j0 > A.n_bins - 2 ? A.n_bins - 2 : (j0 < 0 ? 0 : j0);
+        f = t - (j == j0 ? (T)(r - big) : (T)j);
+        return;
+    }
+    int jj = (int)floor(t);
+    if (jj > A.n_bins - 2) jj = A.n_bins - 2;
+    if (jj < 0) jj = 0;
+    j = jj;
+    f = t - (T)jj;
 }
 
-// Chooses the process for a candidate collision: the smallest k with
-// u1 nu_max < sum_{i<=k} nu_i(eps); -1 = null collision.
-template <class T, bool FAST>
-__device__ __forceinline__ int select_process(const PushArgs<T>& A, const Rates<T>& R, T e, T u1, LStats& ls) {
-    int j;
-    T f;
-    table_pos(A, e, j, f, ls);
-    const T* r0 = R.tab + j * kTableStride;
-    const T* r1 = r0 + kTableStride;
-    const T target = u1 * R.nu_max;
-    if (FAST) {
-        const T t0 = __ldg(r0 + 7), t1 = __ldg(r1 + 7);
-        const T tot = t0 + f * (t1 - t0);
-        if (target >= tot) return -1;
+// Two consecutive rows of a table, and one pair of its totals.
+template <class T> struct LdTab;
+template <> struct LdTab<float> {
+    static __device__ __forceinline__ void rows(const float* p, float a[8], float b[8]) {
+        const float4* q = reinterpret_cast<const float4*>(p);
+        const float4 v0 = __ldg(q), v1 = __ldg(q + 1), v2 = __ldg(q + 2), v3 = __ldg(q + 3);
+        a[0] = v0.x; a[1] = v0.y; a[2] = v0.z; a[3] = v0.w; a[4] = v1.x; a[5] = v1.y; a[6] = v1.z; a[7] = v1.w;
+        b[0] = v2.x; b[1] = v2.y; b[2] = v2.z; b[3] = v2.w; b[4] = v3.x; b[5] = v3.y; b[6] = v3.z; b[7] = v3.w;
     }
-    // the first k with target < sum_{i<=k} nu_i: every process is visited by
-    // every lane (the same sums in the same order), so the lanes of a warp
-    // stay together whichever process they pick
+    static __device__ __forceinline__ void pair(const float* p, float& a, float& d) {
+        const float2 v = __ldg(reinterpret_cast<const float2*>(p));
+        a = v.x; d = v.y;
+    }
+};
+template <> struct LdTab<double> {
+    static __device__ __forceinline__ void rows(const double* p, double a[8], double b[8]) {
+        const double2* q = reinterpret_cast<const double2*>(p);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const double2 u = __ldg(q + i), v = __ldg(q + 4 + i);
+            a[2 * i] = u.x; a[2 * i + 1] = u.y;
+            b[2 * i] = v.x; b[2 * i + 1] = v.y;
+        }
+    }
+    static __device__ __forceinline__ void pair(const double* p, double& a, double& d) {
+        const double2 v = __ldg(reinterpret_cast<const double2*>(p));
+        a = v.x; d = v.y;
+    }
+};
+
+// A candidate collision that may be real: the table coordinate of the energy
+// before it, the rate u1 nu_max to compare with, and the words of the
+// scattering direction (few values: they are held through the draws of the
+// warp's other lanes).
+template <class T> struct Hit {
+    T t, target;
+    uint32_t z, w;
+};
+
+// Chooses the process of a candidate collision: the smallest k with
+// u1 nu_max < sum_{i<=k} nu_i(eps); -1 = null collision.  Every process is
+// visited by every lane (the same sums in the same order; rows of fewer than
+// seven processes end in zeros, which change no sum), so the lanes of a warp
+// stay together whichever process they pick.
+template <class T> __device__ __forceinline__ int select_process(const PushArgs<T>& A, const Rates<T>& R, const Hit<T>& h) {
+    int j;
+    T f, a[kTableRow], b[kTableRow];
+    table_split(A, h.t, j, f);
+    LdTab<T>::rows(R.tab + j * kTableRow, a, b);
     T cum = (T)0;
     int sel = -1;
 #pragma unroll
-    for (int k = 0; k < kTableStride - 1; ++k) {
-        if (k < A.n_proc) {
-            const T a = __ldg(r0 + k), b = __ldg(r1 + k);
-            cum += a + f * (b - a);
-            sel = (sel < 0 && target < cum) ? k : sel;
-        }
+    for (int k = 0; k < kTableRow - 1; ++k) {
+        cum += a[k] + f * (b[k] - a[k]);
+        sel = (sel < 0 && h.target < cum) ? k : sel;
     }
     return sel;
 }
@@ -462,7 +543,7 @@ template <class T> struct Lane {
     uint32_t k;
 };
 
-enum { EV_CONTINUE = 0, EV_DONE = 1, EV_ATTACHED = 2, EV_IONIZED = 3 };
+enum { EV_CONTINUE = 0, EV_DONE = 1, EV_ATTACHED = 2, EV_IONIZED = 3, EV_HIT = 4 };
 
 // Electrode mask of the cell containing x (cell index by correctly rounded
 // (x - origin) / dx, folded into the grid).
@@ -506,28 +587,47 @@ __device__ __forceinline__ void photo_test(const PushArgs<T>& A, const Keys& K, 
     A.pe_k[slot] = k;
 }
 
-// One candidate collision of the null-collision method (Sec. 2.1.1): flight
-// time tau = -ln(u0) / nu_max; if it ends the step, fly to the end; else fly
-// tau, pick the process with u1 nu_max against the cumulative rates at the
-// electron's energy (none = null collision) and scatter isotropically with
-// u2, u3.  Ionization returns EV_IONIZED with the product's speed in sp (the
-// caller queues the product, which flies the remaining time, and its
-// positive-ion event); attachment returns EV_ATTACHED (the caller records the
-// negative-ion event at the electron's position) and ends the electron.
-template <class T, int MODE, bool FAST, bool STATS>
-__device__ __forceinline__ int event(const PushArgs<T>& A, const Rates<T>& R, const Keys& K, uint32_t step,
-                                     const ProcSmem<T>* ps, Lane<T>& L, LStats& ls, T& sp) {
+// One draw of the null-collision method (Sec. 2.1.1): flight time tau =
+// -ln(u0) / nu_max; if it ends the step, fly to the end (EV_DONE); else fly
+// tau and compare u1 nu_max with the total rate at the electron's energy:
+// EV_CONTINUE for a null collision, EV_HIT when a process may take it (h;
+// without FAST always: select_process then decides).
+template <class T, bool FAST>
+__device__ __forceinline__ int candidate(const PushArgs<T>& A, const Rates<T>& R, const Keys& K, uint32_t step,
+                                         Lane<T>& L, LStats& ls, Hit<T>& h) {
     const u32x4 r = draw_words(K, L.id, step, L.k);
     ++L.k;
     const T tau = EvArith<T>::flight(R, unif<T>(r.x));
-    if (tau >= L.t_left) { fly(L.d, L.v, L.a, L.t_left); return EV_DONE; }
+    if (ge_pos(tau, L.t_left)) { fly(L.d, L.v, L.a, L.t_left); return EV_DONE; }
     fly(L.d, L.v, L.a, tau);
-    L.t_left -= tau;
+    L.t_left = sub_rn(L.t_left, tau);
     ++ls.events;
-    T* v = L.v;
+    const T* v = L.v;
     const T v2 = v[0] * v[0] + v[1] * v[1] + v[2] * v[2];
-    const T e = Arith<T>::energy(v2);
-    const int p = select_process<T, FAST>(A, R, e, unif<T>(r.y), ls);
+    h.t = table_pos(A, Arith<T>::energy(v2), ls);
+    h.target = unif<T>(r.y) * R.nu_max;
+    h.z = r.z;
+    h.w = r.w;
+    if (FAST) {
+        // single precision: the interpolated total decides null collisions
+        int j;
+        T f, t0, dt;
+        table_split(A, h.t, j, f);
+        LdTab<T>::pair(R.tab + A.n_bins * kTableRow + 2 * j, t0, dt);
+        if (h.target >= t0 + f * dt) { ++ls.nulls; return EV_CONTINUE; }
+    }
+    return EV_HIT;
+}
+
+// The collision of a hit: the process, then isotropic scattering with u2, u3.
+// Ionization returns EV_IONIZED with the product's speed in sp (the caller
+// queues the product, which flies the remaining time, and its positive-ion
+// event); attachment returns EV_ATTACHED (the caller records the negative-ion
+// event at the electron's position) and ends the electron.
+template <class T, int MODE, bool STATS>
+__device__ __forceinline__ int collide(const PushArgs<T>& A, const Rates<T>& R, const ProcSmem<T>* ps, const Hit<T>& h,
+                                       Lane<T>& L, LStats& ls, T& sp) {
+    const int p = select_process<T>(A, R, h);
     if (p < 0) { ++ls.nulls; return EV_CONTINUE; }
     if (STATS) ++ls.coll[p & 7];
     const int kind = ps->kind[p];
@@ -536,14 +636,16 @@ __device__ __forceinline__ int event(const PushArgs<T>& A, const Rates<T>& R, co
         ++ls.attached;
         return EV_ATTACHED;
     }
+    T* v = L.v;
+    const T v2 = v[0] * v[0] + v[1] * v[1] + v[2] * v[2], e = Arith<T>::energy(v2);
     T n[3];
-    iso_dir(unif<T>(r.z), unif<T>(r.w), n);
+    iso_dir(unif<T>(h.z), unif<T>(h.w), n);
     // energy after the collision: elastic recoil with cos(chi) = n_old . n_new,
     // excitation loss, or half of what ionization leaves (all three formed,
     // one kept: no branch on the process kind)
     const T cchi = EvArith<T>::cosine(v[0] * n[0] + v[1] * n[1] + v[2] * n[2], v2);
-    const T e_el = dmax(e * ((T)1 - (T)2 * ps->mratio[p] * ((T)1 - cchi)), (T)0);
-    const T e_in = dmax(e - ps->thr[p], (T)0);
+    const T e_el = max0(e * ((T)1 - (T)2 * ps->mratio[p] * ((T)1 - cchi)));
+    const T e_in = max0(e - ps->thr[p]);
     const T e2 = kind == PIC_PROC_ELASTIC ? e_el : (kind == PIC_PROC_EXCITATION ? e_in : (T)0.5 * e_in);
     const T sp2 = Arith<T>::speed(e2);
     v[0] = sp2 * n[0]; v[1] = sp2 * n[1]; v[2] = sp2 * n[2];
@@ -553,6 +655,33 @@ __device__ __forceinline__ int event(const PushArgs<T>& A, const Rates<T>& R, co
         return EV_IONIZED;
     }
     return EV_CONTINUE;
+}
+
+// The next draws of a warp's electrons (all lanes call; `active` ones have an
+// electron).  Single precision: two draws, the second by the lanes whose first
+// was a null collision, then the collisions of all hits together: six of ten
+// draws are null, and a warp pays for a collision whatever its lanes.  Double
+// precision: two rounds of a draw and its collision (both cost the same on the
+// narrow double pipe, so a draw with fewer lanes gains nothing).  Measured per
+// pass, 1e6 electrons, float: two draws 330 us, three 355, two rounds 390;
+// 1.4e4 electrons, double: two rounds 579 us a step, two draws 610.
+template <class T, int MODE, bool FAST, bool STATS>
+__device__ __forceinline__ int advance(const PushArgs<T>& A, const Rates<T>& R, const Keys& K, uint32_t step,
+                                       const ProcSmem<T>* ps, bool active, Lane<T>& L, LStats& ls, T& sp) {
+    constexpr int kRounds = FAST ? 1 : 2, kDraws = FAST ? 2 : 1;
+    int r = EV_CONTINUE;
+#pragma unroll
+    for (int q = 0; q < kRounds; ++q) {
+        Hit<T> h;
+#pragma unroll
+        for (int d = 0; d < kDraws; ++d) {
+            if (active && r == EV_CONTINUE) r = candidate<T, FAST>(A, R, K, step, L, ls, h);
+            __syncwarp();
+        }
+        if (r == EV_HIT) r = collide<T, MODE, STATS>(A, R, ps, h, L, ls, sp);
+        __syncwarp();
+    }
+    return r;
 }
 
 // Domain faces (specular reflection or absorption) and electrode cells.
@@ -756,8 +885,8 @@ static __global__ void k_resample_commit(DevState* st) {
 
 // ------------------------------------------------------------------ collisions
 // Lanes refill from per-warp shared-memory stages.  Every lane owns one
-// electron at a time and advances it by up to two candidate collisions per
-// loop iteration; a lane whose electron has finished the step takes the next
+// electron at a time and advances it by up to two draws per loop iteration
+// (advance); a lane whose electron has finished the step takes the next
 // electron from the warp's input stage at once, so the warp stays converged
 // while electrons need different numbers of events.  All per-electron memory
 // work is done by the whole warp, 32 electrons at a time: the input stage is
@@ -775,6 +904,7 @@ static __global__ void k_resample_commit(DevState* st) {
 // CHILD = false: work item = one electron of the input buffer (already kicked
 // by k_field_kick), flying dt.  CHILD = true: work item = one queued
 // ionization product, built when it is staged.
+constexpr int kTripLimit = 1 << 24;  // of a warp in one launch (a minute): an error instead of an endless kernel
 constexpr int kRow = 11;    // padded row of a stage entry: x y z vx vy vz ax ay az w t
 constexpr int kOut = 64;    // output stage capacity (flushed at 32)
 constexpr int kCh = 64;     // product stage capacity of the batched swarm kernel (flushed at 32)
@@ -890,22 +1020,21 @@ template <class T, int MODE, bool FAST, bool STATS, bool CHILD>
 __device__ __forceinline__ void collide_loop(const PushArgs<T>& A, const ProcSmem<T>* ps, Stage<T>* sg) {
     const int lane = threadIdx.x & 31;
     const unsigned lt = (1u << lane) - 1u;
-    long long n_items;
-    unsigned long long* cursor;
+    unsigned long long* cursor = CHILD ? &A.st->n_fetch_c : &A.st->n_fetch;
     const ChildQ<T>& src = (A.gen & 1) ? A.cq2 : A.cq;
     // products the warp queue cannot take: the parents' go to the queue of the
     // first children launch, a children launch's to the other queue
     const ChildQ<T>& dst = CHILD ? ((A.gen & 1) ? A.cq : A.cq2) : A.cq;
     unsigned long long* dst_cnt = CHILD ? ((A.gen & 1) ? &A.st->n_child : &A.st->n_spill) : &A.st->n_child;
+    // work items of the launch (fixed while it runs; read again at each refill rather than held in registers)
+    auto items = [&]() -> long long {
+        if (!CHILD) return (long long)A.st->n_in;
+        const long long n = (long long)((A.gen & 1) ? A.st->n_spill : A.st->n_child);
+        return n < A.cap_child ? n : A.cap_child;
+    };
     if (CHILD) {
-        n_items = (long long)((A.gen & 1) ? A.st->n_spill : A.st->n_child);
-        if (n_items > A.cap_child) n_items = A.cap_child;
-        if (n_items == 0) return;  // the warp queues took every product
-        cursor = &A.st->n_fetch_c;
-        if (blockIdx.x == 0 && threadIdx.x == 0) atomicAdd(&A.st->n_updates, (unsigned long long)n_items);
-    } else {
-        n_items = (long long)A.st->n_in;
-        cursor = &A.st->n_fetch;
+        if (items() == 0) return;  // the warp queues took every product
+        if (blockIdx.x == 0 && threadIdx.x == 0) atomicAdd(&A.st->n_updates, (unsigned long long)items());
     }
     LStats ls;
     ls.zero();
@@ -913,12 +1042,12 @@ __device__ __forceinline__ void collide_loop(const PushArgs<T>& A, const ProcSme
     if (MODE == MODE_SWARM) M.zero();
     const Rates<T> rates{A.table, A.nu_max, A.tau_scale};
     Lane<T> L;
-    bool active = false, dry = false;
+    bool active = false, dry = false, first = true;
     // warp-uniform counters: input stage head and size, output stage size,
     // queued products, buffered negative-ion events
-    int in_head = 0, in_count = 0, n_out = 0, n_pq = 0, n_att = 0;
-    unsigned built = 0;  // products this lane built from the warp queue (counted as updates)
+    int in_head = 0, in_count = 0, n_out = 0, n_pq = 0, n_att = 0, trips = 0;
     for (;;) {
+        if (++trips > kTripLimit) { atomicOr(&A.st->err, kErrStack); break; }
         // 1. idle lanes take staged work items
         const bool want = !active;
         const unsigned need = __ballot_sync(kFull, want);
@@ -951,18 +1080,35 @@ __device__ __forceinline__ void collide_loop(const PushArgs<T>& A, const ProcSme
                     const int j = n_pq - cnt + lane;
                     build_product<T, MODE>(A, sg->pq + j * kPQRow, sg->pq_id[j], sg->pq_k[j], sg->in + lane * kRow,
                                            &sg->in_id[lane]);
-                    ++built;
                 }
+                if (lane == 0) atomicAdd(&A.st->n_updates, (unsigned long long)cnt);
                 n_pq -= cnt;
             } else {
-                unsigned long long b = 0;
-                if (lane == 0) b = atomicAdd(cursor, 32ull);
-                b = __shfl_sync(kFull, b, 0);
-                if ((long long)b >= n_items) {
+                // A warp's first items follow from its place, in an order that
+                // fills the SMs and their four schedulers evenly; later ones
+                // come from the cursor.  With few items a warp of single
+                // precision takes fewer at a time, so that more schedulers work
+                // (a lane's chain of draws, not the issue rate, takes the time
+                // then); double precision fills its warps, whose cost is the
+                // same for any number of lanes.  (Capacities are below 2^31.)
+                const unsigned warps = gridDim.x * (blockDim.x >> 5), n_items = (unsigned)items();
+                unsigned chunk = 32;
+                if (FAST && n_items <= 24u * warps) chunk = (n_items / warps + 8u) & ~7u;
+                unsigned b = 0;
+                if (first) {
+                    b = ((((threadIdx.x >> 5) - blockIdx.x / (unsigned)A.sms) & 3u) * gridDim.x + blockIdx.x) * chunk;
+                } else {
+                    unsigned long long c = 0;
+                    if (lane == 0) c = atomicAdd(cursor, (unsigned long long)chunk);
+                    c = __shfl_sync(kFull, c, 0) + (unsigned long long)warps * chunk;
+                    b = c < n_items ? (unsigned)c : n_items;
+                }
+                first = false;
+                const int left = b < n_items ? (int)(n_items - b) : 0;
+                if (left <= 0) {
                     dry = true;
                 } else {
-                    const long long left = n_items - (long long)b;
-                    cnt = left < 32 ? (int)left : 32;
+                    cnt = left < (int)chunk ? left : (int)chunk;
                     if (lane < cnt) {
                         const long long it = (long long)b + lane;
                         T* r = sg->in + lane * kRow;
@@ -991,16 +1137,9 @@ __device__ __forceinline__ void collide_loop(const PushArgs<T>& A, const ProcSme
             if (dry && in_head >= in_count && n_pq == 0) break;
             continue;
         }
-        // 4. up to two candidate collisions: the second only when the first
-        //    needs nothing from the warp (a null, elastic or excitation
-        //    collision), which halves the warp bookkeeping per draw (three
-        //    per trip measured slower: more lanes idle behind the others)
-        int r = EV_CONTINUE;
+        // 4. up to two draws, which halves the warp bookkeeping per draw
         T sp = (T)0;
-        if (active) {
-            r = event<T, MODE, FAST, STATS>(A, rates, A.K, A.step, ps, L, ls, sp);
-            if (r == EV_CONTINUE) r = event<T, MODE, FAST, STATS>(A, rates, A.K, A.step, ps, L, ls, sp);
-        }
+        const int r = advance<T, MODE, FAST, STATS>(A, rates, A.K, A.step, ps, active, L, ls, sp);
         const bool done = r == EV_DONE, ion = r == EV_IONIZED, att = r == EV_ATTACHED;
         if (done || att) active = false;
         // 5. ionization products wait in the warp queue as compact entries (the
@@ -1067,11 +1206,6 @@ __device__ __forceinline__ void collide_loop(const PushArgs<T>& A, const ProcSme
     }
     if (n_out > 0) flush_out<T, MODE>(A, sg, n_out, n_out, ls, M);
     if (MODE == MODE_PIC && n_att > 0) flush_att(A, sg, n_att);
-    {
-        unsigned pw = built;
-        for (int o = 16; o > 0; o >>= 1) pw += __shfl_xor_sync(kFull, pw, o);
-        if (lane == 0 && pw) atomicAdd(&A.st->n_updates, (unsigned long long)pw);
-    }
     if (STATS) flush_stats(A, ls, A.n_proc);
     if (MODE == MODE_SWARM) {
         M.m[14] += ls.w_ion;
@@ -1097,9 +1231,11 @@ template <class T> __device__ __forceinline__ Stage<T>* warp_stage(unsigned char
 }
 
 constexpr int kCollideThreads = 128;
-// Resident blocks per SM the collision kernels are compiled for: seven (28
-// warps, 72 registers) in single precision, four in double precision.
-template <class T> constexpr int collide_min_blocks() { return sizeof(T) == 4 ? 7 : 4; }
+// Resident blocks per SM the collision kernels are compiled for: six (24
+// warps, 80 registers, 76 KB of L1 left beside their stages for the 40 KB of
+// tables) in single precision, four in double precision.  1e6 electrons in
+// float: six 330 us, seven 356 (72 registers, 47 KB of L1), five 346.
+template <class T> constexpr int collide_min_blocks() { return sizeof(T) == 4 ? 6 : 4; }
 
 template <class T, int MODE, bool FAST, bool STATS>
 __global__ void __launch_bounds__(kCollideThreads, collide_min_blocks<T>()) k_push(const PushArgs<T> A) {

@@ -53,7 +53,7 @@ template <class T> struct BatchArgs {
     long long n_lo, n_hi;
     int gen;
     // collision rates of each swarm's gas: table of swarm s at tab_s + s *
-    // tab_stride (stride 0: one gas for all), nu_max and -ln 2 / nu_max
+    // tab_stride (stride 0: one gas for all), nu_max and its flight_scale
     const T* tab_s;
     long long tab_stride;
     const T* numax_s;
@@ -448,7 +448,9 @@ __device__ void batch_phase(const BatchArgs<T>& B, const ProcSmem<T>& ps, BatchS
     bool active = false, dry = false;
     int in_head = 0, in_count = 0, n_out = 0, n_ch = 0;
     StackSink<T> stk;
+    int trips = 0;
     for (;;) {
+        if (++trips > kTripLimit) { atomicOr(&B.bd->err, kErrStack); break; }
         bool want = !active;
         if (CHILD && want && stk.n > 0) {
             --stk.n;
@@ -552,13 +554,8 @@ __device__ void batch_phase(const BatchArgs<T>& B, const ProcSmem<T>& ps, BatchS
             if (dry && in_head >= in_count) break;
             continue;
         }
-        int r = EV_CONTINUE;
         T sp = (T)0;
-        if (active) {
-            // up to two candidate collisions per trip, as in the collision kernel
-            r = event<T, MODE_SWARM, FAST, false>(B.P, R, K, step, &ps, L, ls, sp);
-            if (r == EV_CONTINUE) r = event<T, MODE_SWARM, FAST, false>(B.P, R, K, step, &ps, L, ls, sp);
-        }
+        const int r = advance<T, MODE_SWARM, FAST, false>(B.P, R, K, step, &ps, active, L, ls, sp);
         const bool done = r == EV_DONE, ion = r == EV_IONIZED;
         if (r == EV_DONE || r == EV_ATTACHED) active = false;
         if (CHILD && ion) {
@@ -737,9 +734,10 @@ __device__ bool batch_run_step(const BatchArgs<T>& B, const ProcSmem<T>& ps, Bat
     return grid_barrier(bd);
 }
 
-// Every step of every swarm in one launch (cooperative: all blocks resident).
+// Every step of every swarm in one launch (cooperative: all blocks resident;
+// registers capped so that two blocks fit an SM in single precision).
 template <class T, bool FAST>
-__global__ void __launch_bounds__(256) k_batch_run(const BatchArgs<T> B, int n_steps) {
+__global__ void __launch_bounds__(256, sizeof(T) == 4 ? 2 : 1) k_batch_run(const BatchArgs<T> B, int n_steps) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ ProcSmem<T> ps;
     stage_proc_batch(ps, B);
