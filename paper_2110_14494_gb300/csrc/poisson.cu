@@ -353,6 +353,7 @@ __global__ void __launch_bounds__(BX * BY) k_sweep_first(float* __restrict__ e, 
 __global__ void k_resid_restrict(const float* __restrict__ e, const float* __restrict__ g,
                                  const uint8_t* __restrict__ mask, int nx, int ny, int nz, float* __restrict__ gc,
                                  const uint8_t* __restrict__ maskc, int black_zero) {
+    cudaTriggerProgrammaticLaunchCompletion();  // the tail may load its tables meanwhile
     pdl_wait();
     const int cx = nx / 2, cy = ny / 2;
     const int I = blockIdx.x * BX + threadIdx.x, J = blockIdx.y * BY + threadIdx.y, K = blockIdx.z;
@@ -676,6 +677,7 @@ __global__ void k_grad(const double* __restrict__ phi, int nx, int ny, int nz, d
     if (E4) { E4[4 * c] = (T)ex; E4[4 * c + 1] = (T)ey; E4[4 * c + 2] = (T)ez; E4[4 * c + 3] = (T)0; }
 }
 
+#include "poisson_tail.cuh"
 #include "poisson_mixed.cuh"
 
 dim3 grid3(int nx, int ny, int nz) { return dim3((nx + BX - 1) / BX, (ny + BY - 1) / BY, nz); }
@@ -699,6 +701,8 @@ dim3 grid3_red(int nx, int ny, int nz) { return dim3((nx + BX - 1) / BX, (ny + B
 
 // ------------------------------------------------------------------ host side
 static size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
+
+static TailPlan tail_plan(const MG& mg);
 
 void MG::plan(int nx_, int ny_, int nz_) {
     levels = 0;
@@ -765,6 +769,7 @@ size_t MG::carve(void* base, int nx_, int ny_, int nz_, bool mixed_, bool pair_c
         g[l] = (float*)take(n * sizeof(float));
         m[l] = (uint8_t*)take(n);
     }
+    tail_tab = tail_tables() ? (uint4*)take((size_t)tail_plan(*this).cells * sizeof(uint4)) : nullptr;
     return (size_t)(p - p0);
 }
 
@@ -783,6 +788,30 @@ int MG::tail_level() const {
 }
 
 
+// The tail's levels, their places in shared memory and their threads.
+static TailPlan tail_plan(const MG& mg) {
+    TailPlan T = {};
+    const int t = mg.tail_level();
+    for (int l = t; l < mg.levels && l - t < kTailMaxLevels; ++l)
+        T.L[T.levels++] = tail_geometry(mg.lx[l], mg.ly[l], mg.lz[l]);
+    tail_place(T);
+    return T;
+}
+
+// Hierarchies whose tail fits the kernel of poisson_tail.cuh: at most four
+// cells of a colour a thread on the first level, one on the others, and their
+// arrays in shared memory (every hierarchy of 8192 cells or fewer without an
+// extreme aspect); a single level of more cells keeps the plain kernel.
+bool MG::tail_tables() const {
+    const int t = tail_level();
+    if (omega != 1.0f || levels - t > kTailMaxLevels) return false;
+    const TailPlan T = tail_plan(*this);
+    if ((size_t)T.words * 4 > kTailSmem || T.L[0].ca > 0xffff || T.L[0].h > kTailPerThread * kTailThreads) return false;
+    for (int l = 1; l < T.levels; ++l)
+        if (T.L[l].h > kTailThreads) return false;
+    return true;
+}
+
 cudaError_t MG::build_masks(const uint8_t* mask, cudaStream_t s) {
     const long long n0 = (long long)lx[0] * ly[0] * lz[0];
     launches += levels;
@@ -790,7 +819,61 @@ cudaError_t MG::build_masks(const uint8_t* mask, cudaStream_t s) {
     for (int l = 1; l < levels; ++l)
         k_restrict_mask<<<grid3(lx[l], ly[l], lz[l]), kBlk, 0, s>>>(m[l - 1], lx[l - 1], ly[l - 1], lz[l - 1], m[l],
                                                                     mask_min_children);
+    if (tail_tables()) {
+        const TailPlan T = tail_plan(*this);
+        for (int l = 0; l < T.levels; ++l) {
+            k_tail_table<<<(2 * T.L[l].h + 127) / 128, 128, 0, s>>>(m[tail_level() + l], T.L[l], T.L[l > 0 ? l - 1 : 0],
+                                                                   tail_tab + T.L[l].w);
+            ++launches;
+        }
+    }
     return cudaGetLastError();
+}
+
+// The levels from tail_level() down in one launch.
+void MG::tail(cudaStream_t s, int pre, int post) {
+    const int t = tail_level();
+    if (tail_tab && pre > 0 && post > 0) {
+        TailPlan T = tail_plan(*this);
+        T.e_first = e[t];
+        T.g_first = g[t];
+        T.tab = tail_tab;
+        T.pre = pre;
+        T.post = post;
+        T.coarse = coarse_sweeps;
+        const size_t smem = (size_t)T.words * 4;
+        auto go = [&](void (*k)(TailPlan)) {
+            if (smem > 48 * 1024) cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+            launch_pdl(k, dim3(1), dim3(T.L[0].act), smem, s, T);
+        };
+        const int per = (T.L[0].h + T.L[0].act - 1) / T.L[0].act;
+        if (per == 1) go(k_tail_cycle<1>);
+        else if (per == 2) go(k_tail_cycle<2>);
+        else go(k_tail_cycle<4>);
+        return;
+    }
+    TailLevels T;
+    int off = 0;
+    for (int l = 0; l < levels; ++l) {
+        T.m[l] = m[l];
+        T.nx[l] = lx[l]; T.ny[l] = ly[l]; T.nz[l] = lz[l];
+        T.off[l] = off;
+        if (l >= t) off += lx[l] * ly[l] * lz[l];
+    }
+    T.e_first = e[t];
+    T.g_first = g[t];
+    T.first = t;
+    T.last = levels - 1;
+    T.warp_from = levels;
+    for (int l = levels - 1; l >= t && (long long)lx[l] * ly[l] * lz[l] <= kWarpCells; --l) T.warp_from = l;
+    T.pre = pre;
+    T.post = post;
+    T.coarse = coarse_sweeps;
+    T.omega = omega;
+    T.total = off;
+    const size_t smem = tail_smem_bytes(off);
+    if (smem > 48 * 1024) cudaFuncSetAttribute(k_tail_vcycle, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    launch_pdl(k_tail_vcycle, dim3(1), dim3(1024), smem, s, T);
 }
 
 // One V(pre, post)-cycle on A e0 = g0 (light: V(light_pre, light_post)); e0 is overwritten.  Levels above the
@@ -817,28 +900,7 @@ void MG::vcycle(cudaStream_t s, bool light) {
                    (const float*)g[l], (const uint8_t*)m[l], lx[l], ly[l], lz[l], g[l + 1], (const uint8_t*)m[l + 1],
                    pre > 0 ? 1 : 0);
     }
-    TailLevels T;
-    int off = 0;
-    for (int l = 0; l < levels; ++l) {
-        T.m[l] = m[l];
-        T.nx[l] = lx[l]; T.ny[l] = ly[l]; T.nz[l] = lz[l];
-        T.off[l] = off;
-        if (l >= t) off += lx[l] * ly[l] * lz[l];
-    }
-    T.e_first = e[t];
-    T.g_first = g[t];
-    T.first = t;
-    T.last = levels - 1;
-    T.warp_from = levels;
-    for (int l = levels - 1; l >= t && (long long)lx[l] * ly[l] * lz[l] <= kWarpCells; --l) T.warp_from = l;
-    T.pre = pre;
-    T.post = post;
-    T.coarse = coarse_sweeps;
-    T.omega = omega;
-    T.total = off;
-    const size_t smem = tail_smem_bytes(off);
-    if (smem > 48 * 1024) cudaFuncSetAttribute(k_tail_vcycle, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    launch_pdl(k_tail_vcycle, dim3(1), dim3(1024), smem, s, T);
+    tail(s, pre, post);
     for (int l = t - 1; l >= 0; --l) {
         launch_pdl(k_prolong_add, grid3(lx[l + 1], ly[l + 1], lz[l + 1]), kBlk, 0, s, (const float*)e[l + 1], e[l],
                    (const uint8_t*)m[l], lx[l], ly[l], lz[l]);

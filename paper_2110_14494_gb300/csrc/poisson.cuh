@@ -28,6 +28,7 @@ struct MG {
     float* e[kMaxLevels];
     float* g[kMaxLevels];
     uint8_t* m[kMaxLevels];
+    uint4* tail_tab = nullptr;  // cells of the tail's levels (poisson_tail.cuh)
     double* norms = nullptr;  // CG scalars: ||b||^2, ||r||^2, rho, gamma, z.r, z.q, alpha, beta
     double *r64 = nullptr, *p64 = nullptr, *q64 = nullptr;  // CG vectors (float64)
     int pre = 2, post = 2, coarse_sweeps = 4;  // coarse: red-black sweeps on the coarsest level
@@ -114,6 +115,8 @@ struct MG {
     cudaError_t build_masks(const uint8_t* mask, cudaStream_t s);
     void vcycle(cudaStream_t s, bool light);
     int tail_level() const;
+    bool tail_tables() const;  // the tail's levels fit the kernel of poisson_tail.cuh
+    void tail(cudaStream_t s, int pre, int post);
     // Returns PIC_OK, PIC_ERR_TIMEOUT or PIC_ERR_CUDA.  packed_prec selects the
     // element type (32: float, 64: double) of the optional packed field E4.
     int solve(const double* rho, const uint8_t* mask, double* phi, double h, double v_lo, double v_hi, double v_mask,
