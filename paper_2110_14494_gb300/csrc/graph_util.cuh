@@ -1,9 +1,35 @@
 // Helpers for recording device-driven loops into CUDA graphs (conditional
-// nodes added at the capture point of a stream).
+// nodes added at the capture point of a stream), and for launches that overlap
+// the end of the kernel before them.
 #pragma once
 #include <cuda_runtime.h>
 
 namespace pic {
+
+// Kernels of the solvers' cycles are launched with programmatic dependent
+// launch: their blocks may be scheduled while the previous kernel's last
+// blocks still run, and each waits here for that grid (and its memory) before
+// its first access.  Without the launch attribute the wait returns at once.
+__device__ __forceinline__ void pdl_wait() { cudaGridDependencySynchronize(); }
+
+template <class... P, class... A>
+void launch_pdl(void (*k)(P...), dim3 g, dim3 b, size_t smem, cudaStream_t s, A... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = g;
+    cfg.blockDim = b;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    cudaLaunchKernelEx(&cfg, k, args...);
+}
+
+__device__ __forceinline__ void bar_named(int id, int threads) {
+    asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(threads) : "memory");
+}
 
 // Adds a conditional node with handle h at the capture point of stream cs
 // (which must be capturing) and makes it the stream's only dependency;

@@ -1750,8 +1750,15 @@ static int solve_field_pair(pic_ctx* c) {
     return PIC_OK;
 }
 
-// The steady-state axisymmetric field solve as one graph launch: ring-cell
-// charge density, extrapolated warm start and the device-driven (r, z) solve
+// Right-hand side (i + 1/2) h^2 rho / eps0 of the ring cells from the
+// fixed-point charges: the volume pi (2 i + 1) h^3 leaves e / (2 pi h eps0) a charge.
+static AxiCharge axi_charge(pic_ctx* c) {
+    return AxiCharge{nullptr, (const long long*)c->qe(), (const long long*)c->qp(), (const long long*)c->qn(),
+                     kQ / (4294967296.0 * 2.0 * kPi * c->g.dx * kEps0)};
+}
+
+// The steady-state axisymmetric field solve as one graph launch: extrapolated
+// warm start and the device-driven (r, z) solve
 // reporting into DevState.  Returns PIC_ERR_STATE when the graph cannot be
 // recorded.
 static int solve_field_axi_graph(pic_ctx* c) {
@@ -1766,14 +1773,10 @@ static int solve_field_axi_graph(pic_ctx* c) {
             cudaGetLastError();
             return PIC_ERR_STATE;
         }
-        const double dV = c->g.dx * c->g.dx * c->g.dx * kPi;
-        k_fixed_to_rho<<<grid_n(n), 256, 0, c->fcap>>>((const long long*)c->qe(), (const long long*)c->qp(),
-                                                        (const long long*)c->qn(), n, 1.0 / (4294967296.0 * dV),
-                                                        c->rho(), c->g.nx);
         k_extrapolate<<<grid_n(n), 256, 0, c->fcap>>>(c->phi(), (double*)(c->ws + c->L.phi_prev), n, 1);
         DevState* st = c->st();
         long long fixed = 0;
-        const int rc = c->amg.capture_solve(c->fcap, c->rho(), c->phi(), c->g.dx, c->cfg.v_lo, c->cfg.v_hi,
+        const int rc = c->amg.capture_solve(c->fcap, axi_charge(c), c->phi(), c->g.dx, c->cfg.v_lo, c->cfg.v_hi,
                                             c->cfg.v_mask, c->cfg.poisson_rtol, c->cfg.poisson_max_cycles, c->prec,
                                             c->ws + c->L.E4, &st->poisson_cycles, &st->poisson_rel, &st->err,
                                             kErrPoissonLimit, &st->dev_kernels, &fixed);
@@ -1787,7 +1790,7 @@ static int solve_field_axi_graph(pic_ctx* c) {
         }
         cudaGraphDestroy(gr);
         c->agraph = gx;
-        c->agraph_kernels = fixed + 2;
+        c->agraph_kernels = fixed + 1;
     }
     const cudaError_t e = cudaGraphLaunch(c->agraph, c->s);
     if (e != cudaSuccess) return c->cuda_fail(e, "axisymmetric field solve graph");
@@ -1809,14 +1812,13 @@ static int solve_field_axi(pic_ctx* c) {
         c->fgraph_off = true;
     }
     c->last_on_device = false;
-    fixed_to_rho(c, c->rho());
     k_extrapolate<<<grid_n(c->g.ncell()), 256, 0, c->s>>>(c->phi(), (double*)(c->ws + c->L.phi_prev), c->g.ncell(),
                                                            c->n_solves >= 2 ? 1 : 0);
     c->n_solves++;
-    c->launches += 2;
+    c->launches += 1;
     const long long l0 = c->amg.launches;
     double hn[2];
-    int rc = c->amg.solve(c->rho(), c->mask, c->phi(), c->g.dx, c->cfg.v_lo, c->cfg.v_hi, c->cfg.v_mask,
+    int rc = c->amg.solve(axi_charge(c), c->mask, c->phi(), c->g.dx, c->cfg.v_lo, c->cfg.v_hi, c->cfg.v_mask,
                           c->cfg.poisson_rtol, c->cfg.poisson_max_cycles, c->prec, c->ws + c->L.E4, nullptr,
                           nullptr, c->s, &c->last_cycles, &c->last_rel, hn);
     if (rc == PIC_ERR_CUDA) return c->fail(rc, "axisymmetric poisson solve: CUDA error");

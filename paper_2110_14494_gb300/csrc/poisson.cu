@@ -27,28 +27,6 @@ namespace {
 
 constexpr int BX = 32, BY = 4;
 
-// Kernels of the V-cycle and of the CG iteration are launched with
-// programmatic dependent launch: their blocks may be scheduled while the
-// previous kernel's last blocks still run, and each waits here for that grid
-// (and its memory) before its first access.  Without the launch attribute
-// the wait returns at once.
-__device__ __forceinline__ void pdl_wait() { cudaGridDependencySynchronize(); }
-
-template <class... P, class... A>
-void launch_pdl(void (*k)(P...), dim3 g, dim3 b, size_t smem, cudaStream_t s, A... args) {
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = g;
-    cfg.blockDim = b;
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = s;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = at;
-    cfg.numAttrs = 1;
-    cudaLaunchKernelEx(&cfg, k, args...);
-}
-
 __device__ __forceinline__ int lin(int i, int j, int k, int nx, int ny) { return (k * ny + j) * nx + i; }
 
 // Block sum of a double into one atomicAdd (all threads of the block call).

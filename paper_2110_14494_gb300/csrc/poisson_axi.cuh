@@ -5,6 +5,15 @@
 
 namespace pic {
 
+// Right-hand side of a solve: rho in C/m^3, or (rho null) the fixed-point
+// charges of the grid, b = scale (q_pos - q_neg - q_e) with the ring volumes
+// cancelled against the ring cells' factor.
+struct AxiCharge {
+    const double* rho;
+    const long long *qe, *qp, *qn;
+    double scale;
+};
+
 // Loop state of a device-driven axisymmetric solve (device memory).
 struct AxiLoop {
     int cyc, trips, timeout, pad;
@@ -19,28 +28,26 @@ struct AxiMG {
     double* e[kMaxLevels];
     double* g[kMaxLevels];
     uint8_t* m[kMaxLevels];
-    double *norms = nullptr, *r = nullptr, *p = nullptr, *q = nullptr;
+    double* rd[kMaxLevels];  // reciprocal diagonals by column: [nr] inside, [nr] at the z faces
+    double *norms = nullptr, *r = nullptr, *p = nullptr, *q = nullptr, *w = nullptr;
+    double* part = nullptr;   // per-block partial sums
+    unsigned* ctr = nullptr;  // arrivals of their blocks
     int pre = 2, post = 2, coarse_sweeps = 64;
     long long launches = 0;
     bool persistent = false, masks_ready = false;
     AxiLoop* loop = nullptr;
-    // CG iterations run before the first convergence test (0 to 2, at most
-    // max_cycles).  0 for every caller: the coupled axisymmetric solves often
-    // converge in fewer than two, where a forced pair costs more than the
-    // loop trips it saves.
-    int min_cycles = 0;
-    int min_cycles_for(int max_cycles) const;
-    cudaStream_t cap_body[2] = {nullptr, nullptr};
+    cudaStream_t cap_body[3] = {nullptr, nullptr, nullptr};
     // Streams for recording loop bodies (call before the caller's capture).
     int prepare_capture();
     void release();
-    // Records the solve on the capturing stream cs: residual, a device-side
-    // while loop (decision, then a switch over the first and the later CG
-    // iterations), the gradient and a report of cycles, relative residual,
-    // cycle-limit flag (err_bit into *err_dst) and the loop's kernels (added
-    // to *kernels_dst).  No host synchronisation.  Returns PIC_OK or
+    // Records the solve on the capturing stream cs: residual, an if node with
+    // the first CG iteration, in it another with a device-side while loop over
+    // the later ones (most coupled solves need one iteration), the gradient
+    // and a report of cycles, relative residual, cycle-limit flag (err_bit
+    // into *err_dst) and the kernels run in the nodes (added to
+    // *kernels_dst).  No host synchronisation.  Returns PIC_OK or
     // PIC_ERR_CUDA / PIC_ERR_STATE (callers then use solve).
-    int capture_solve(cudaStream_t cs, const double* rho, double* phi, double h, double v_lo, double v_hi,
+    int capture_solve(cudaStream_t cs, const AxiCharge& rho, double* phi, double h, double v_lo, double v_hi,
                       double v_mask, double rtol, int max_cycles, int packed_prec, void* E4, int* cycles_dst,
                       double* rel_dst, unsigned* err_dst, unsigned err_bit, unsigned long long* kernels_dst,
                       long long* fixed_kernels);
@@ -51,12 +58,14 @@ struct AxiMG {
     static size_t bytes(int nr, int nz);
     size_t carve(void* base, int nr, int nz);
     cudaError_t build_masks(const uint8_t* mask, cudaStream_t s);
+    int tail_level() const;  // first level of the one-block kernel (levels: none)
     void vcycle(cudaStream_t s);
-    // rho: charge density (C/m^3) [nz][nr]; phi: initial guess and solution;
+    void iteration(cudaStream_t s, double* phi, bool first);
+    // rho: charge [nz][nr]; phi: initial guess and solution;
     // E4 (optional): packed [nz][nr][4] (E_r, 0, E_z, 0) in float (packed_prec
     // 32) or double (64); Er, Ez: optional float planes.  Returns PIC_OK,
     // PIC_ERR_TIMEOUT or PIC_ERR_CUDA.
-    int solve(const double* rho, const uint8_t* mask, double* phi, double h, double v_lo, double v_hi,
+    int solve(const AxiCharge& rho, const uint8_t* mask, double* phi, double h, double v_lo, double v_hi,
               double v_mask, double rtol, int max_cycles, int packed_prec, void* E4, float* Er, float* Ez,
               cudaStream_t s, int* cycles_out, double* rel_out, double* host_norms);
 };

@@ -105,10 +105,6 @@ __global__ void k_tail_table(const uint8_t* __restrict__ m, TailLevel L, TailLev
     tab[p] = c;
 }
 
-__device__ __forceinline__ void bar_named(int id, int threads) {
-    asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(threads) : "memory");
-}
-
 // A thread's cells of a level, colour by colour.
 template <int C> struct TailCells {
     uint32_t w[2][C];
