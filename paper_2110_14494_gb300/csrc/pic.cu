@@ -941,7 +941,7 @@ static size_t al256(size_t x) { return (x + 255) & ~(size_t)255; }
 struct Layout {
     size_t total = 0;
     size_t buf[2], cq[2], table, E4, E4b, qe, qp, qn, st, cnt, start, sums, key, rank, msc, gas, rho, phi,
-        phi_prev, phi_x, phi_y, mg, photo, hostio;
+        phi_prev, phi_x, phi_y, slot, mg, photo, hostio;  // slot: bytes of one potential
 };
 
 static size_t real_size(int prec) { return prec == 64 ? 8 : 4; }
@@ -988,11 +988,11 @@ static Layout make_layout(const pic_config* c) {
     L.rho = take(ncell * 8);
     // a potential slot holds ncell doubles, or a float pair: hi, then lo at
     // the next 256-byte boundary (the pair kernels use 16-byte accesses)
-    const size_t slot = 2 * al256(ncell * 4);
-    L.phi = take(slot);
-    L.phi_prev = take(slot);
-    L.phi_x = take(slot);
-    L.phi_y = pair ? take(slot) : L.phi_x;
+    L.slot = 2 * al256(ncell * 4);
+    L.phi = take(L.slot);
+    L.phi_prev = take(L.slot);
+    L.phi_x = take(L.slot);
+    L.phi_y = pair ? take(L.slot) : L.phi_x;
     L.mg = take(c->geometry == 1 ? AxiMG::bytes(c->nx, c->nz) : MG::bytes(c->nx, c->ny, c->nz, c->precision == 32, false));
     {
         const size_t np = (size_t)photo_cap(c);
@@ -1317,10 +1317,10 @@ extern "C" int pic_init(const pic_config* cfg, void* d_ws, size_t ws_bytes, cons
     if (e == cudaSuccess) e = cudaMemsetAsync(c->ws + L.qe, 0, ncell * 8, c->s);
     if (e == cudaSuccess) e = cudaMemsetAsync(c->ws + L.qp, 0, ncell * 8, c->s);
     if (e == cudaSuccess) e = cudaMemsetAsync(c->ws + L.qn, 0, ncell * 8, c->s);
-    if (e == cudaSuccess) e = cudaMemsetAsync(c->ws + L.phi, 0, ncell * 8, c->s);
-    if (e == cudaSuccess) e = cudaMemsetAsync(c->ws + L.phi_prev, 0, ncell * 8, c->s);
-    if (e == cudaSuccess) e = cudaMemsetAsync(c->ws + L.phi_x, 0, ncell * 8, c->s);
-    if (e == cudaSuccess) e = cudaMemsetAsync(c->ws + L.phi_y, 0, ncell * 8, c->s);
+    if (e == cudaSuccess) e = cudaMemsetAsync(c->ws + L.phi, 0, L.slot, c->s);
+    if (e == cudaSuccess) e = cudaMemsetAsync(c->ws + L.phi_prev, 0, L.slot, c->s);
+    if (e == cudaSuccess) e = cudaMemsetAsync(c->ws + L.phi_x, 0, L.slot, c->s);
+    if (e == cudaSuccess) e = cudaMemsetAsync(c->ws + L.phi_y, 0, L.slot, c->s);
     if (e != cudaSuccess) { rc = c->cuda_fail(e, "pic_init"); delete c; return rc; }
     rc = build_table(c);
     if (rc) { delete c; return rc; }
