@@ -29,41 +29,8 @@ constexpr int BX = 32, BY = 4;
 
 __device__ __forceinline__ int lin(int i, int j, int k, int nx, int ny) { return (k * ny + j) * nx + i; }
 
-// Block sum of a double into one atomicAdd (all threads of the block call).
-__device__ __forceinline__ void block_add(double v, double* dst) {
-    __shared__ double red[32];
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(kFull, v, o);
-    const int t = threadIdx.x + threadIdx.y * blockDim.x;
-    const int lane = t & 31, w = t >> 5, nw = (blockDim.x * blockDim.y) >> 5;
-    if (lane == 0) red[w] = v;
-    __syncthreads();
-    if (t == 0) {
-        double s = 0.0;
-        for (int q = 0; q < nw; ++q) s += red[q];
-        if (s != 0.0) atomicAdd(dst, s);
-    }
-    __syncthreads();  // red[] is reused by the next call in the same kernel
-}
-
 // Scalars of the flexible CG, in device memory.
-enum { S_B2 = 0, S_R2, S_RHO, S_GAM, S_T1, S_T2, S_ALPHA, S_BETA, S_N };
-
-// Stencil sum of the neighbours of interior cell c (x, y Neumann mirror and
-// z Dirichlet are folded into the diagonal; masked neighbours contribute 0).
-template <class V>
-__device__ __forceinline__ V nb_sum(const V* e, const uint8_t* m, int i, int j, int k, int nx, int ny, int nz, int c,
-                                    V& diag) {
-    const int pl = nx * ny;
-    V s = (V)0;
-    diag = (V)6;
-    if (i > 0) { if (!m[c - 1]) s += e[c - 1]; } else diag -= (V)1;
-    if (i < nx - 1) { if (!m[c + 1]) s += e[c + 1]; } else diag -= (V)1;
-    if (j > 0) { if (!m[c - nx]) s += e[c - nx]; } else diag -= (V)1;
-    if (j < ny - 1) { if (!m[c + nx]) s += e[c + nx]; } else diag -= (V)1;
-    if (k > 0) { if (!m[c - pl]) s += e[c - pl]; } else diag += (V)1;
-    if (k < nz - 1) { if (!m[c + pl]) s += e[c + pl]; } else diag += (V)1;
-    return s;
-}
+enum { S_B2 = 0, S_R2, S_RHO, S_GAM, S_ALPHA, S_BETA, S_N };
 
 #define CELL3D                                                   \
     const int i = blockIdx.x * BX + threadIdx.x;                 \
@@ -71,140 +38,6 @@ __device__ __forceinline__ V nb_sum(const V* e, const uint8_t* m, int i, int j, 
     const int k = blockIdx.z;                                    \
     const bool in = i < nx && j < ny;                            \
     const int c = in ? lin(i, j, k, nx, ny) : 0;
-
-// Reducing kernels run a bounded grid (z extent kZRed) and loop over z.
-constexpr int kZRed = 8;
-#define CELL3D_LOOP_BEGIN                                        \
-    const int i = blockIdx.x * BX + threadIdx.x;                 \
-    const int j = blockIdx.y * BY + threadIdx.y;                 \
-    const bool in = i < nx && j < ny;                            \
-    double acc = 0.0;                                            \
-    for (int k = blockIdx.z; k < nz; k += gridDim.z) {           \
-        const int c = in ? lin(i, j, k, nx, ny) : 0;
-#define CELL3D_LOOP_END }
-
-// b = h^2 rho / eps0 + plate terms + electrode neighbours; accumulates ||b||^2.
-__global__ void k_rhs_norm(const double* __restrict__ rho, const uint8_t* __restrict__ mask, int nx, int ny, int nz,
-                           double h2e, double v_lo, double v_hi, double v_mask, double* sc) {
-    CELL3D_LOOP_BEGIN
-    if (in && !mask[c]) {
-        const int pl = nx * ny;
-        double s = h2e * rho[c];
-        if (k == 0) s += 2.0 * v_lo;
-        if (k == nz - 1) s += 2.0 * v_hi;
-        if (i > 0 && mask[c - 1]) s += v_mask;
-        if (i < nx - 1 && mask[c + 1]) s += v_mask;
-        if (j > 0 && mask[c - nx]) s += v_mask;
-        if (j < ny - 1 && mask[c + nx]) s += v_mask;
-        if (k > 0 && mask[c - pl]) s += v_mask;
-        if (k < nz - 1 && mask[c + pl]) s += v_mask;
-        acc += s * s;
-    }
-    CELL3D_LOOP_END
-    block_add(acc, sc + S_B2);
-}
-
-// r = b - A phi with the true boundary values (float64) and its float32 copy
-// for the preconditioner; accumulates ||r||^2; electrode cells get phi = v_mask.
-__global__ void k_resid64(double* __restrict__ phi, const double* __restrict__ rho, const uint8_t* __restrict__ mask,
-                          int nx, int ny, int nz, double h2e, double v_lo, double v_hi, double v_mask,
-                          double* __restrict__ r, float* __restrict__ g0, double* sc) {
-    CELL3D_LOOP_BEGIN
-    if (in) {
-        if (mask[c]) {
-            phi[c] = v_mask;
-            r[c] = 0.0;
-            g0[c] = 0.0f;
-        } else {
-            const int pl = nx * ny;
-            const double pc = phi[c];
-            auto val = [&](int q, bool inside, double ghost) -> double {
-                if (!inside) return ghost;
-                if (mask[q]) return v_mask;
-                return phi[q];
-            };
-            const double sum = val(c - 1, i > 0, pc) + val(c + 1, i < nx - 1, pc) + val(c - nx, j > 0, pc) +
-                               val(c + nx, j < ny - 1, pc) + val(c - pl, k > 0, 2.0 * v_lo - pc) +
-                               val(c + pl, k < nz - 1, 2.0 * v_hi - pc);
-            const double rr = h2e * rho[c] + sum - 6.0 * pc;
-            r[c] = rr;
-            g0[c] = (float)rr;
-            acc += rr * rr;
-        }
-    }
-    CELL3D_LOOP_END
-    block_add(acc, sc + S_R2);
-}
-
-// q = A p (homogeneous boundary values) and p.q.
-__global__ void k_apply(const double* __restrict__ p, const uint8_t* __restrict__ mask, int nx, int ny, int nz,
-                        double* __restrict__ q, double* sc) {
-    CELL3D_LOOP_BEGIN
-    if (in) {
-        if (mask[c]) {
-            q[c] = 0.0;
-        } else {
-            double diag;
-            const double s = nb_sum(p, mask, i, j, k, nx, ny, nz, c, diag);
-            const double v = diag * p[c] - s;
-            q[c] = v;
-            acc += p[c] * v;
-        }
-    }
-    CELL3D_LOOP_END
-    block_add(acc, sc + S_GAM);
-}
-
-__global__ void k_alpha(double* sc) {
-    sc[S_ALPHA] = sc[S_RHO] / sc[S_GAM];
-    sc[S_R2] = 0.0;
-    sc[S_T1] = 0.0;
-    sc[S_T2] = 0.0;
-}
-
-// phi += alpha p; r -= alpha q; float32 copy of r; ||r||^2.
-__global__ void k_update_xr(double* __restrict__ phi, double* __restrict__ r, const double* __restrict__ p,
-                            const double* __restrict__ q, float* __restrict__ g0, int n, double* sc) {
-    const double a = sc[S_ALPHA];
-    double acc = 0.0;
-    const int stride = gridDim.x * blockDim.x * blockDim.y;
-    for (int c = (blockIdx.x * blockDim.y + threadIdx.y) * blockDim.x + threadIdx.x; c < n; c += stride) {
-        phi[c] += a * p[c];
-        const double rr = r[c] - a * q[c];
-        r[c] = rr;
-        g0[c] = (float)rr;
-        acc += rr * rr;
-    }
-    block_add(acc, sc + S_R2);
-}
-
-// t1 = z.r, t2 = z.q with z the preconditioned residual (float32).
-__global__ void k_dot2(const float* __restrict__ z, const double* __restrict__ r, const double* __restrict__ q, int n,
-                       double* sc, int with_q) {
-    const int stride = gridDim.x * blockDim.x * blockDim.y;
-    double a = 0.0, b = 0.0;
-    for (int c = (blockIdx.x * blockDim.y + threadIdx.y) * blockDim.x + threadIdx.x; c < n; c += stride) {
-        const double zz = (double)z[c];
-        a += zz * r[c];
-        if (with_q) b += zz * q[c];
-    }
-    block_add(a, sc + S_T1);
-    if (with_q) block_add(b, sc + S_T2);
-}
-
-// Flexible CG direction: beta = -alpha (z.q) / rho (equivalently
-// z.(r_new - r_old) / rho), rho <- z.r.
-__global__ void k_beta(double* sc, int first) {
-    sc[S_BETA] = first ? 0.0 : -sc[S_ALPHA] * sc[S_T2] / sc[S_RHO];
-    sc[S_RHO] = sc[S_T1];
-    sc[S_GAM] = 0.0;
-}
-
-__global__ void k_update_p(double* __restrict__ p, const float* __restrict__ z, int n, const double* sc) {
-    const double b = sc[S_BETA];
-    const int c = (blockIdx.x * blockDim.y + threadIdx.y) * blockDim.x + threadIdx.x;
-    if (c < n) p[c] = b != 0.0 ? (double)z[c] + b * p[c] : (double)z[c];
-}
 
 // Neighbour sum of the correction e, which is zero on electrode cells at
 // every level (they are never updated, and prolongation writes 0 there), so
@@ -657,6 +490,7 @@ __global__ void k_grad(const double* __restrict__ phi, int nx, int ny, int nz, d
 
 #include "poisson_tail.cuh"
 #include "poisson_mixed.cuh"
+#include "poisson_cg64.cuh"
 
 dim3 grid3(int nx, int ny, int nz) { return dim3((nx + BX - 1) / BX, (ny + BY - 1) / BY, nz); }
 const dim3 kBlk(BX, BY, 1);
@@ -668,12 +502,7 @@ void smooth_half(float* e, const float* g, const uint8_t* m, int nx, int ny, int
     if (zs == 4) launch_pdl(k_smooth<4>, gr, kBlk, 0, s, e, g, m, nx, ny, nz, color, omega);
     else launch_pdl(k_smooth<1>, gr, kBlk, 0, s, e, g, m, nx, ny, nz, color, omega);
 }
-dim3 grid_flat(long long n) { return dim3((unsigned)((n + BX * BY - 1) / (BX * BY))); }
-dim3 grid_red(long long n) {
-    long long b = (n + BX * BY - 1) / (BX * BY);
-    return dim3((unsigned)(b < 1216 ? b : 1216));
-}
-dim3 grid3_red(int nx, int ny, int nz) { return dim3((nx + BX - 1) / BX, (ny + BY - 1) / BY, nz < kZRed ? nz : kZRed); }
+dim3 grid_mx3(int nx, int ny, int nz) { return dim3((nx + BX - 1) / BX, (ny + BY - 1) / BY, (nz + ZC - 1) / ZC); }
 
 }  // namespace
 
@@ -704,13 +533,13 @@ bool MG::supported(int nx_, int ny_, int nz_) {
     return (long long)m.lx[L] * m.ly[L] * m.lz[L] * 9 <= 200 * 1024;
 }
 
-size_t MG::bytes(int nx_, int ny_, int nz_, bool mixed_, bool pair_copy) {
+size_t MG::bytes(int nx_, int ny_, int nz_, bool mixed_, bool pair_copy, bool lean) {
     MG m;
-    return m.carve(nullptr, nx_, ny_, nz_, mixed_, pair_copy);
+    return m.carve(nullptr, nx_, ny_, nz_, mixed_, pair_copy, lean);
 }
 
 // Lays the buffers out from base (base null: sizes only); returns the bytes.
-size_t MG::carve(void* base, int nx_, int ny_, int nz_, bool mixed_, bool pair_copy) {
+size_t MG::carve(void* base, int nx_, int ny_, int nz_, bool mixed_, bool pair_copy, bool lean) {
     plan(nx_, ny_, nz_);
     mixed = mixed_;
     uintptr_t p = (uintptr_t)base;
@@ -740,6 +569,10 @@ size_t MG::carve(void* base, int nx_, int ny_, int nz_, bool mixed_, bool pair_c
         r64 = (double*)take(n0 * 8);
         p64 = (double*)take(n0 * 8);
         q64 = (double*)take(n0 * 8);
+        w64 = lean ? nullptr : (double*)take(n0 * 8);
+        ctr = (unsigned*)(norms + 16);  // within the scalars' 256 bytes
+        const size_t b3 = (size_t)((nx_ + BX - 1) / BX) * ((ny_ + BY - 1) / BY) * ((nz_ + ZC - 1) / ZC);
+        part = lean && levels > 1 ? nullptr : (double*)take(3 * 8 * b3);
     }
     for (int l = 0; l < levels; ++l) {
         const size_t n = (size_t)lx[l] * ly[l] * lz[l];
@@ -747,7 +580,10 @@ size_t MG::carve(void* base, int nx_, int ny_, int nz_, bool mixed_, bool pair_c
         g[l] = (float*)take(n * sizeof(float));
         m[l] = (uint8_t*)take(n);
     }
-    tail_tab = tail_tables() ? (uint4*)take((size_t)tail_plan(*this).cells * sizeof(uint4)) : nullptr;
+    // lean: the partial sums share the second level's e and g (8 bytes a coarse cell, at least twice their size),
+    // which only the V-cycle uses
+    if (!mixed_ && lean && levels > 1) part = (double*)e[1];
+    tail_tab = tail_tables() && !lean ? (uint4*)take((size_t)tail_plan(*this).cells * sizeof(uint4)) : nullptr;
     return (size_t)(p - p0);
 }
 
@@ -797,7 +633,7 @@ cudaError_t MG::build_masks(const uint8_t* mask, cudaStream_t s) {
     for (int l = 1; l < levels; ++l)
         k_restrict_mask<<<grid3(lx[l], ly[l], lz[l]), kBlk, 0, s>>>(m[l - 1], lx[l - 1], ly[l - 1], lz[l - 1], m[l],
                                                                     mask_min_children);
-    if (tail_tables()) {
+    if (tail_tab) {
         const TailPlan T = tail_plan(*this);
         for (int l = 0; l < T.levels; ++l) {
             k_tail_table<<<(2 * T.L[l].h + 127) / 128, 128, 0, s>>>(m[tail_level() + l], T.L[l], T.L[l > 0 ? l - 1 : 0],
@@ -889,18 +725,17 @@ void MG::vcycle(cudaStream_t s, bool light) {
     }
 }
 
-// One flexible-CG iteration: z = M r, direction, q = A p, alpha, updates.
+// One flexible-CG iteration: z = M r, w = A z with the iteration's scalars,
+// then the direction and the updates.
 void MG::iteration(cudaStream_t s, double* phi, const uint8_t* mk, bool first) {
     const int nx = lx[0], ny = ly[0], nz = lz[0];
-    const int n = nx * ny * nz;
+    const int f = first ? 1 : 0;
     vcycle(s, false);
-    k_dot2<<<grid_red(n), kBlk, 0, s>>>(e[0], r64, q64, n, norms, first ? 0 : 1);
-    k_beta<<<1, 1, 0, s>>>(norms, first ? 1 : 0);
-    k_update_p<<<grid_flat(n), kBlk, 0, s>>>(p64, e[0], n, norms);
-    k_apply<<<grid3_red(nx, ny, nz), kBlk, 0, s>>>(p64, mk, nx, ny, nz, q64, norms);
-    k_alpha<<<1, 1, 0, s>>>(norms);
-    k_update_xr<<<grid_red(n), kBlk, 0, s>>>(phi, r64, p64, q64, g[0], n, norms);
-    launches += 6;
+    launch_pdl(k_apply64, grid_mx3(nx, ny, nz), kBlk, 0, s, (const float*)e[0], (const double*)r64, (const double*)q64,
+               w64, mk, nx, ny, nz, f, part, ctr + 1, norms);
+    launch_pdl(k_step64, grid_mx3(nx, ny, nz), kBlk, 0, s, (const float*)e[0], (const double*)w64, mk, p64, q64, phi,
+               r64, g[0], nx, ny, nz, f, part, ctr + 2, norms);
+    launches += 2;
 }
 
 void MG::release() {
@@ -929,10 +764,10 @@ int MG::solve(const double* rho, const uint8_t* mask, double* phi, double h, dou
             if (g_iter[q]) { cudaGraphExecDestroy(g_iter[q]); g_iter[q] = nullptr; }
         g_key[0] = phi; g_key[1] = rho; g_key[2] = mask;
     }
-    cudaMemsetAsync(norms, 0, S_N * 8, s);
-    k_rhs_norm<<<grid3_red(nx, ny, nz), kBlk, 0, s>>>(rho, mk, nx, ny, nz, h2e, v_lo, v_hi, v_mask, norms);
-    k_resid64<<<grid3_red(nx, ny, nz), kBlk, 0, s>>>(phi, rho, mk, nx, ny, nz, h2e, v_lo, v_hi, v_mask, r64, g[0], norms);
-    launches += 2;
+    if (cudaMemsetAsync(ctr, 0, 8 * sizeof(unsigned), s) != cudaSuccess) return PIC_ERR_CUDA;
+    k_resid64<<<grid_mx3(nx, ny, nz), kBlk, 0, s>>>(phi, rho, mk, nx, ny, nz, h2e, v_lo, v_hi, v_mask, r64, g[0], part,
+                                                    ctr, norms);
+    launches += 1;
     int cyc = 0, rc = PIC_OK;
     double bn = 1.0, rn = 0.0;
     for (;;) {
@@ -982,7 +817,6 @@ int MG::solve(const double* rho, const uint8_t* mask, double* phi, double h, dou
 
 // ------------------------------------------------------------------ mixed precision
 namespace {
-dim3 grid_mx3(int nx, int ny, int nz) { return dim3((nx + BX - 1) / BX, (ny + BY - 1) / BY, (nz + ZC - 1) / ZC); }
 // the float4 stencil kernels: four x cells per thread (nx % 4 == 0)
 dim3 grid_mx3v(int nx, int ny, int nz) {
     return dim3((nx / 4 + BX - 1) / BX, (ny + BY - 1) / BY, (nz + ZC - 1) / ZC);
@@ -1237,14 +1071,16 @@ bool poisson_args_ok(const poisson_config* pc, const double* rho, const double* 
     return MG::supported(pc->nx, pc->ny, pc->nz);
 }
 
-size_t poisson_bytes(const poisson_config* pc) { return MG::bytes(pc->nx, pc->ny, pc->nz, pc->precision == 32, true); }
+size_t poisson_bytes(const poisson_config* pc, bool lean) {
+    return MG::bytes(pc->nx, pc->ny, pc->nz, pc->precision == 32, true, lean);
+}
 
-// The solve behind both entry points, on a workspace of poisson_bytes(pc).
+// The solve behind both entry points, on a workspace of poisson_bytes(pc, lean).
 int poisson_run(const poisson_config* pc, const double* rho, const uint8_t* mask, double* phi, float* Ex, float* Ey,
-                float* Ez, double rtol, int max_cycles, void* ws, poisson_stats* st, cudaStream_t s) {
+                float* Ez, double rtol, int max_cycles, void* ws, bool lean, poisson_stats* st, cudaStream_t s) {
     MG mg;
     const bool mixed = pc->precision == 32;
-    mg.carve(ws, pc->nx, pc->ny, pc->nz, mixed, true);
+    mg.carve(ws, pc->nx, pc->ny, pc->nz, mixed, true, lean);
     double hn[2];
     int cycles = 0;
     double rel = 0.0;
@@ -1271,15 +1107,15 @@ extern "C" size_t poisson_workspace_bytes(const poisson_config* pc) {
     if (!pc || (pc->precision != 0 && pc->precision != 32 && pc->precision != 64) ||
         !MG::supported(pc->nx, pc->ny, pc->nz))
         return 0;
-    return poisson_bytes(pc);
+    return poisson_bytes(pc, false);
 }
 
 extern "C" int poisson_solve(const poisson_config* pc, const double* rho, const uint8_t* mask, double* phi, float* Ex,
                              float* Ey, float* Ez, double rtol, int max_cycles, void* ws, size_t ws_bytes,
                              poisson_stats* st, pic_stream_t stream) {
     if (!ws || !poisson_args_ok(pc, rho, phi, Ex, Ey, Ez, rtol, max_cycles)) return PIC_ERR_ARG;
-    if (ws_bytes < poisson_bytes(pc) || ((uintptr_t)ws & 255)) return PIC_ERR_ARG;
-    return poisson_run(pc, rho, mask, phi, Ex, Ey, Ez, rtol, max_cycles, ws, st, (cudaStream_t)stream);
+    if (ws_bytes < poisson_bytes(pc, false) || ((uintptr_t)ws & 255)) return PIC_ERR_ARG;
+    return poisson_run(pc, rho, mask, phi, Ex, Ey, Ez, rtol, max_cycles, ws, false, st, (cudaStream_t)stream);
 }
 
 // ------------------------------------------------------------------ no-allocation variant
@@ -1321,9 +1157,9 @@ extern "C" int poisson_solve_noalloc(const poisson_config* pc, const double* rho
                                      float* Ex, float* Ey, float* Ez, double rtol, int max_cycles, poisson_stats* st,
                                      pic_stream_t stream) {
     if (!poisson_args_ok(pc, rho, phi, Ex, Ey, Ez, rtol, max_cycles)) return PIC_ERR_ARG;
-    if (poisson_bytes(pc) > kNoAllocScratchBytes) return PIC_ERR_CAPACITY;
+    if (poisson_bytes(pc, true) > kNoAllocScratchBytes) return PIC_ERR_CAPACITY;
     void* ws = nullptr;
     int rc = noalloc_scratch(&ws);
     if (rc) return rc;
-    return poisson_run(pc, rho, mask, phi, Ex, Ey, Ez, rtol, max_cycles, ws, st, (cudaStream_t)stream);
+    return poisson_run(pc, rho, mask, phi, Ex, Ey, Ez, rtol, max_cycles, ws, true, st, (cudaStream_t)stream);
 }

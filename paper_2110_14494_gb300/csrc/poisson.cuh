@@ -29,8 +29,8 @@ struct MG {
     float* g[kMaxLevels];
     uint8_t* m[kMaxLevels];
     uint4* tail_tab = nullptr;  // cells of the tail's levels (poisson_tail.cuh)
-    double* norms = nullptr;  // CG scalars: ||b||^2, ||r||^2, rho, gamma, z.r, z.q, alpha, beta
-    double *r64 = nullptr, *p64 = nullptr, *q64 = nullptr;  // CG vectors (float64)
+    double* norms = nullptr;  // CG scalars: ||b||^2, ||r||^2, rho, gamma, alpha, beta
+    double *r64 = nullptr, *p64 = nullptr, *q64 = nullptr, *w64 = nullptr;  // CG vectors (float64; w64 not if lean)
     int pre = 2, post = 2, coarse_sweeps = 4;  // coarse: red-black sweeps on the coarsest level
     // mixed solve: an iteration after the untested ones whose relative
     // residual is already within light_ratio x rtol uses a V(light_pre,
@@ -110,8 +110,10 @@ struct MG {
     static bool supported(int nx, int ny, int nz);
     // Workspace of the float64 solve (mixed false) or of the mixed one
     // (pair_copy: with room for the pair copy of a float64 potential).
-    static size_t bytes(int nx, int ny, int nz, bool mixed = false, bool pair_copy = false);
-    size_t carve(void* base, int nx, int ny, int nz, bool mixed = false, bool pair_copy = false);
+    // lean: no more than the solve cannot do without (no stored A z, no tail tables), for the fixed scratch
+    // of poisson_solve_noalloc.
+    static size_t bytes(int nx, int ny, int nz, bool mixed = false, bool pair_copy = false, bool lean = false);
+    size_t carve(void* base, int nx, int ny, int nz, bool mixed = false, bool pair_copy = false, bool lean = false);
     cudaError_t build_masks(const uint8_t* mask, cudaStream_t s);
     void vcycle(cudaStream_t s, bool light);
     int tail_level() const;
