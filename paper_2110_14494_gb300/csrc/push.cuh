@@ -524,14 +524,6 @@ __device__ __forceinline__ uint64_t make_child(const Keys& K, uint32_t step, uin
     return cid;
 }
 
-// Products of products (rare) are built at once and wait on the lane's stack.
-template <class T> struct StackSink {
-    static constexpr int kDepth = 8;
-    T x[kDepth][3], v[kDepth][3], w[kDepth], t[kDepth];
-    uint64_t id[kDepth];
-    int n = 0;
-};
-
 // One electron in flight on a lane: start position x, displacement d within
 // the step (x + d is the position; single precision keeps the resolution of
 // the short flights that way), velocity, acceleration, weight, remaining time
@@ -907,7 +899,6 @@ static __global__ void k_resample_commit(DevState* st) {
 constexpr int kTripLimit = 1 << 24;  // of a warp in one launch (a minute): an error instead of an endless kernel
 constexpr int kRow = 11;    // padded row of a stage entry: x y z vx vy vz ax ay az w t
 constexpr int kOut = 64;    // output stage capacity (flushed at 32)
-constexpr int kCh = 64;     // product stage capacity of the batched swarm kernel (flushed at 32)
 constexpr int kPQ = 40;     // warp queue of ionization products (built 32 at a time)
 constexpr int kPQRow = 9;   // x y z, product speed, ax ay az of the ionizing electron, w, remaining time
 constexpr int kAtt = 32;    // warp buffer of attachment events awaiting their deposit

@@ -97,26 +97,34 @@ __device__ __forceinline__ int swarm_of(const long long* pre, int n, long long i
 }
 
 // Resampling per swarm, in place (see k_resample): thinning above n_hi,
-// duplication below n_lo.  Grid-stride over the step's items.
+// duplication below n_lo.  A block takes a contiguous part of the step's items
+// and passes over the swarms that need neither (most steps all of them: 57 us
+// with a search for every item, 26 us).
 template <class T, bool FLIP> __device__ void batch_resample(const BatchArgs<T>& B, uint32_t step) {
-    const long long total = B.prefix[B.n_swarms];
-    for (long long it = (long long)blockIdx.x * blockDim.x + threadIdx.x; it < total;
-         it += (long long)gridDim.x * blockDim.x) {
-        const int s = swarm_of(B.prefix, B.n_swarms, it);
+    const long long total = B.prefix[B.n_swarms], per = (total + gridDim.x - 1) / gridDim.x;
+    long long lo = blockIdx.x * per;
+    const long long hi = lo + per < total ? lo + per : total;
+    if (lo >= hi) return;
+    for (int s = swarm_of(B.prefix, B.n_swarms, lo); lo < hi; ++s) {
+        const long long first = B.prefix[s], next = B.prefix[s + 1], end = next < hi ? next : hi;
         const long long n = B.cnt_in[s];
         const bool thin = n > B.n_hi, dup = n > 0 && n < B.n_lo && 2 * n <= B.cap_s;
-        if (!thin && !dup) continue;
-        const long long i = s * B.cap_s + (it - B.prefix[s]);
-        const Keys K = dev_keys(B.seed + (uint64_t)s);
-        const Soa<T>& p = src_buf<T, FLIP>(B);
-        if (thin) {
-            const u32x4 r = draw_words(K, p.id[i], step, 0xA0000000u);
-            if (!(unif<T>(r.x) < (T)0.5)) p.r[PW][i] = (T)0;
-        } else {
-            const long long j = i + n;
-            for (int f = 0; f < 10; ++f) p.r[f][j] = p.r[f][i];
-            p.id[j] = derived_id(K, p.id[i], step, 0xA0000000u);
+        if (thin || dup) {
+            const Keys K = dev_keys(B.seed + (uint64_t)s);
+            const Soa<T>& p = src_buf<T, FLIP>(B);
+            for (long long it = lo + threadIdx.x; it < end; it += blockDim.x) {
+                const long long i = s * B.cap_s + (it - first);
+                if (thin) {
+                    const u32x4 r = draw_words(K, p.id[i], step, 0xA0000000u);
+                    if (!(unif<T>(r.x) < (T)0.5)) p.r[PW][i] = (T)0;
+                } else {
+                    const long long j = i + n;
+                    for (int f = 0; f < 10; ++f) p.r[f][j] = p.r[f][i];
+                    p.id[j] = derived_id(K, p.id[i], step, 0xA0000000u);
+                }
+            }
         }
+        lo = end;
     }
 }
 template <class T> __global__ void k_batch_resample(const BatchArgs<T> B) { batch_resample<T, false>(B, B.bd->step); }
@@ -252,10 +260,11 @@ constexpr long long kWarpChunk = 1024;  // default largest warp-private item ran
 template <class T> struct BatchStage {
     T in[32 * kRow];
     T out[kOut * kRow];
-    T ch[kCh * kRow];
-    uint64_t in_id[32], out_id[kOut], ch_id[kCh];
-    uint32_t ch_k[kCh];
-    int in_s[32], out_s[kOut], ch_s[kCh];
+    uint64_t in_id[32], out_id[kOut];
+    T pq[kPQ * kPQRow];   // products waiting to be built, as in Stage
+    uint64_t pq_id[kPQ];
+    uint32_t pq_k[kPQ];
+    int in_s[32], out_s[kOut], pq_s[kPQ];
     double macc[14];   // the warp's running moment sums for swarm macc_s (step macc_t)
     int macc_s;
 };
@@ -302,6 +311,7 @@ __device__ __forceinline__ void swarm_moments(const BatchArgs<T>& B, BatchStage<
         const bool mine = live && s == sg_s;
         todo &= ~__ballot_sync(kFull, mine);
         T red[14];
+#pragma unroll
         for (int q = 0; q < 14; ++q) {
             T v2 = mine ? m[q] : (T)0;
             for (int o = 16; o > 0; o >>= 1) v2 += __shfl_xor_sync(kFull, v2, o);
@@ -314,9 +324,10 @@ __device__ __forceinline__ void swarm_moments(const BatchArgs<T>& B, BatchStage<
             __syncwarp();
         }
         const int lane = threadIdx.x & 31;
-        double add = 0.0;
-        for (int k = 0; k < 14; ++k)
-            if (k == lane) add = (double)red[k];
+        T mine_sum = (T)0;
+#pragma unroll
+        for (int k = 0; k < 14; ++k) mine_sum = k == lane ? red[k] : mine_sum;
+        const double add = (double)mine_sum;
         if (sg->macc_s == sg_s) {
             if (lane < 14) sg->macc[lane] += add;
         } else if (lane < 14 && add != 0.0) {
@@ -384,50 +395,15 @@ __device__ __forceinline__ void batch_flush_out(const BatchArgs<T>& B, BatchStag
     n = rest;
 }
 
-template <class T>
-__device__ __forceinline__ void batch_flush_children(const BatchArgs<T>& B, BatchStage<T>* sg, int& n, int cnt,
-                                                     int dst, unsigned long long* cnt_p) {
-    const int lane = threadIdx.x & 31;
-    __syncwarp();
-    unsigned long long s0 = 0;
-    if (lane == 0) s0 = atomicAdd(cnt_p, (unsigned long long)cnt);
-    s0 = __shfl_sync(kFull, s0, 0);
-    if (lane < cnt) {
-        const unsigned long long q = s0 + lane;
-        if ((long long)q < B.cap_child) {
-            const T* r = sg->ch + lane * kRow;
-            const ChildQ<T>& Q = B.cq[dst];
-            Q.p.r[PX][q] = r[0]; Q.p.r[PY][q] = r[1]; Q.p.r[PZ][q] = r[2];
-            Q.p.r[VX][q] = r[3];
-            Q.p.r[AX][q] = r[4]; Q.p.r[AY][q] = r[5]; Q.p.r[AZ][q] = r[6];
-            Q.p.r[PW][q] = r[7];
-            Q.t_left[q] = r[8];
-            Q.p.id[q] = sg->ch_id[lane];
-            Q.k[q] = sg->ch_k[lane];
-            B.csw[dst][q] = (uint32_t)sg->ch_s[lane];
-        } else {
-            atomicOr(&B.bd->err, kErrChildCapacity);
-        }
-    }
-    __syncwarp();
-    const int rest = n - cnt;
-    if (lane < rest) {
-        for (int f = 0; f < 9; ++f) sg->ch[lane * kRow + f] = sg->ch[(cnt + lane) * kRow + f];
-        sg->ch_id[lane] = sg->ch_id[cnt + lane];
-        sg->ch_k[lane] = sg->ch_k[cnt + lane];
-        sg->ch_s[lane] = sg->ch_s[cnt + lane];
-    }
-    __syncwarp();
-    n = rest;
-}
-
 // The lane-refill collision loop of collide_loop, for batched swarms: one
 // phase of a step.  CHILD = false: the work items are the swarms' electrons
-// (n_items of them); their products are staged per warp and queued in queue
-// dstq (append counter dst_cnt).  CHILD = true: the items are the products
-// queued in srcq; their own products stay on the lane's stack, and what it
-// cannot hold goes to queue dstq for the next generation.  Every warp takes
-// item ranges from `cursor` until the phase runs dry.
+// (n_items of them).  CHILD = true: the items are the products queued in srcq.
+// Products wait in the warp's queue and become work items of the same phase,
+// 32 at a time; what that queue cannot hold goes to queue dstq (append counter
+// dst_cnt) for the next generation.  Every warp takes item ranges from
+// `cursor` until the phase runs dry.  256 float swarms, 60 steps: with every
+// product in the global queue, built by launches of their own, 120 ms (children
+// 131 us a launch); with the warp queue 111 ms (children 19 us).
 template <class T, bool FAST, bool CHILD, bool FLIP>
 __device__ void batch_phase(const BatchArgs<T>& B, const ProcSmem<T>& ps, BatchStage<T>* sg, uint32_t step,
                             long long n_items, unsigned long long* cursor, int srcq, int dstq,
@@ -446,23 +422,10 @@ __device__ void batch_phase(const BatchArgs<T>& B, const ProcSmem<T>& ps, BatchS
     int s_cur = -1, s_cache = -1;
     long long w_next = 0, w_end = 0;
     bool active = false, dry = false;
-    int in_head = 0, in_count = 0, n_out = 0, n_ch = 0;
-    StackSink<T> stk;
-    int trips = 0;
+    int in_head = 0, in_count = 0, n_out = 0, n_pq = 0, trips = 0;
     for (;;) {
         if (++trips > kTripLimit) { atomicOr(&B.bd->err, kErrStack); break; }
-        bool want = !active;
-        if (CHILD && want && stk.n > 0) {
-            --stk.n;
-            const int t = stk.n;
-            for (int d = 0; d < 3; ++d) { L.x[d] = stk.x[t][d]; L.v[d] = stk.v[t][d]; L.d[d] = (T)0; }
-            L.w = stk.w[t];
-            L.id = stk.id[t];
-            L.t_left = stk.t[t];
-            L.k = 1;
-            active = true;
-            want = false;
-        }
+        const bool want = !active;
         const unsigned need = __ballot_sync(kFull, want);
         const int avail = in_count - in_head;
         if (need && avail > 0) {
@@ -489,7 +452,28 @@ __device__ void batch_phase(const BatchArgs<T>& B, const ProcSmem<T>& ps, BatchS
             }
             in_head += __popc(need) < avail ? __popc(need) : avail;
         }
-        if (in_head >= in_count && !dry) {
+        if (in_head >= in_count && n_pq > 0 && (dry || n_pq >= 32)) {
+            // products built as the next work items
+            const int cnt = n_pq < 32 ? n_pq : 32;
+            __syncwarp();
+            if (lane < cnt) {
+                const int j = n_pq - cnt + lane;
+                const T* q = sg->pq + j * kPQRow;
+                T* r = sg->in + lane * kRow;
+                T vc[3];
+                sg->in_id[lane] = make_child(dev_keys(B.seed + (uint64_t)sg->pq_s[j]), step, sg->pq_id[j], sg->pq_k[j], q[3],
+                                             vc);
+                r[0] = q[0]; r[1] = q[1]; r[2] = q[2];
+                r[3] = vc[0]; r[4] = vc[1]; r[5] = vc[2];
+                r[9] = q[7];
+                r[10] = q[8];
+                sg->in_s[lane] = sg->pq_s[j];
+            }
+            n_pq -= cnt;
+            in_head = 0;
+            in_count = cnt;
+            __syncwarp();
+        } else if (in_head >= in_count && !dry) {
             __syncwarp();
             if (w_next >= w_end) {
                 // a new warp-private range: large while much work is left (so a
@@ -550,56 +534,45 @@ __device__ void batch_phase(const BatchArgs<T>& B, const ProcSmem<T>& ps, BatchS
             }
             __syncwarp();
         }
-        if (!__any_sync(kFull, active || (CHILD && stk.n > 0))) {
-            if (dry && in_head >= in_count) break;
+        if (!__any_sync(kFull, active)) {
+            if (dry && in_head >= in_count && n_pq == 0) break;
             continue;
         }
         T sp = (T)0;
         const int r = advance<T, MODE_SWARM, FAST, false>(B.P, R, K, step, &ps, active, L, ls, sp);
         const bool done = r == EV_DONE, ion = r == EV_IONIZED;
         if (r == EV_DONE || r == EV_ATTACHED) active = false;
-        if (CHILD && ion) {
-            if (stk.n < StackSink<T>::kDepth) {
-                T vc[3];
-                const uint64_t cid = make_child(K, step, L.id, L.k - 1, sp, vc);
-                const int t = stk.n++;
-                for (int d = 0; d < 3; ++d) { stk.x[t][d] = L.x[d] + L.d[d]; stk.v[t][d] = vc[d]; }
-                stk.w[t] = L.w;
-                stk.id[t] = cid;
-                stk.t[t] = L.t_left;
-            } else {  // stack full: queue the compact entry for the next generation
-                const unsigned long long q = atomicAdd(dst_cnt, 1ull);
-                if ((long long)q < B.cap_child) {
-                    const ChildQ<T>& Q = B.cq[dstq];
-                    Q.p.r[PX][q] = L.x[0] + L.d[0]; Q.p.r[PY][q] = L.x[1] + L.d[1]; Q.p.r[PZ][q] = L.x[2] + L.d[2];
-                    Q.p.r[VX][q] = sp;
-                    Q.p.r[AX][q] = L.a[0]; Q.p.r[AY][q] = L.a[1]; Q.p.r[AZ][q] = L.a[2];
-                    Q.p.r[PW][q] = L.w;
-                    Q.t_left[q] = L.t_left;
-                    Q.p.id[q] = L.id;
-                    Q.k[q] = L.k - 1;
-                    B.csw[dstq][q] = (uint32_t)s_cur;
-                } else {
-                    atomicOr(&B.bd->err, kErrChildCapacity);
-                }
-            }
-        }
-        const unsigned im = CHILD ? 0u : __ballot_sync(kFull, ion);
+        const unsigned im = __ballot_sync(kFull, ion);
         if (im) {
             if (ion) {
-                const int e = n_ch + __popc(im & lt);
-                T* q = sg->ch + e * kRow;
-                q[0] = L.x[0] + L.d[0]; q[1] = L.x[1] + L.d[1]; q[2] = L.x[2] + L.d[2];
-                q[3] = sp;
-                q[4] = L.a[0]; q[5] = L.a[1]; q[6] = L.a[2];
-                q[7] = L.w;
-                q[8] = L.t_left;
-                sg->ch_id[e] = L.id;
-                sg->ch_k[e] = L.k - 1;
-                sg->ch_s[e] = s_cur;
+                const int slot = n_pq + __popc(im & lt);
+                const T e[kPQRow] = {L.x[0] + L.d[0], L.x[1] + L.d[1], L.x[2] + L.d[2], sp,
+                                     L.a[0], L.a[1], L.a[2], L.w, L.t_left};
+                if (slot < kPQ) {
+                    T* q = sg->pq + slot * kPQRow;
+                    for (int f = 0; f < kPQRow; ++f) q[f] = e[f];
+                    sg->pq_id[slot] = L.id;
+                    sg->pq_k[slot] = L.k - 1;
+                    sg->pq_s[slot] = s_cur;
+                } else {
+                    const unsigned long long q = atomicAdd(dst_cnt, 1ull);
+                    if ((long long)q < B.cap_child) {
+                        const ChildQ<T>& Q = B.cq[dstq];
+                        Q.p.r[PX][q] = e[0]; Q.p.r[PY][q] = e[1]; Q.p.r[PZ][q] = e[2];
+                        Q.p.r[VX][q] = sp;
+                        Q.p.r[AX][q] = e[4]; Q.p.r[AY][q] = e[5]; Q.p.r[AZ][q] = e[6];
+                        Q.p.r[PW][q] = L.w;
+                        Q.t_left[q] = L.t_left;
+                        Q.p.id[q] = L.id;
+                        Q.k[q] = L.k - 1;
+                        B.csw[dstq][q] = (uint32_t)s_cur;
+                    } else {
+                        atomicOr(&B.bd->err, kErrChildCapacity);
+                    }
+                }
             }
-            n_ch += __popc(im);
-            if (n_ch >= 32) batch_flush_children(B, sg, n_ch, 32, dstq, dst_cnt);
+            n_pq += __popc(im);
+            if (n_pq > kPQ) n_pq = kPQ;
         }
         const unsigned dm = __ballot_sync(kFull, done);
         if (dm) {
@@ -618,7 +591,6 @@ __device__ void batch_phase(const BatchArgs<T>& B, const ProcSmem<T>& ps, BatchS
         }
     }
     if (n_out > 0) batch_flush_out<T, FLIP>(B, sg, n_out, n_out, step);
-    if (!CHILD && n_ch > 0) batch_flush_children(B, sg, n_ch, n_ch, dstq, dst_cnt);
     macc_flush(B, sg, step);
     flush_event_weights(B, s_cur, step, ls);
 }
@@ -634,8 +606,10 @@ template <class T> __device__ __forceinline__ void stage_proc_batch(ProcSmem<T>&
 
 // One phase per launch (the step replayed from a CUDA graph): generation
 // B.gen reads queue B.gen & 1 and queues into the other one.
+// Three float blocks an SM: 80 registers and a few spilled words; left to itself the compiler takes 108, two
+// blocks, 124 ms in place of 111 for 256 swarms.
 template <class T, bool FAST, bool CHILD>
-__global__ void __launch_bounds__(256) k_batch_collide(const BatchArgs<T> B) {
+__global__ void __launch_bounds__(256, sizeof(T) == 4 ? 3 : 1) k_batch_collide(const BatchArgs<T> B) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ ProcSmem<T> ps;
     stage_proc_batch(ps, B);

@@ -80,3 +80,19 @@ def test_float64_solve_at_block_and_level_edges(shape):
     rc, st = _solve_noalloc(P, pc, drho, phi2, dmask, 1e-11, 500)
     assert rc == P.PIC_OK and st.cycles == cyc and torch.equal(phi, phi2)
     assert np.linalg.norm(phi.cpu().numpy() - ref) <= 1e-8 * np.linalg.norm(ref)
+
+
+@pytest.mark.parametrize("n0,launch", [(1, 0), (33, 1), (33, 2), (700, 0), (700, 1), (700, 2)])
+def test_batched_products_through_warp_and_global_queues(n0, launch):
+    """Many ionizations a step (2.6 electrons for one after 2 ps at 900 Td): products wait in the
+    warp's queue, what it cannot hold goes to the global one.  Each swarm is the
+    oracle's run: counts equal, moments to 1e-9 as elsewhere for float64."""
+    from paper_2110_14494_gb300 import swarm_run
+    gas, seed, ENs = W.synthetic_air(), 31, [900.0, 600.0]
+    res, mom, cnt = swarm_run(gas, ENs, precision=64, n0=n0, n_steps=6, dt=2e-12, seed=seed, n_lo=1, n_hi=100000,
+                              want_moments=True, batched=True, block=128, blocks_per_sm=1, use_graph=launch)
+    for s, EN in enumerate(ENs):
+        omom, ocnt, _, _ = O.swarm(gas, EN, n0, 6, 2e-12, seed + s, n_lo=1, n_hi=100000)
+        assert np.array_equal(cnt[s], ocnt), s
+        scale = np.abs(omom).max(axis=0) + 1e-300
+        assert np.all(np.abs(mom[s] - omom) <= 1e-9 * scale), s
