@@ -17,6 +17,7 @@
 #include <stdint.h>
 
 #include "common.cuh"
+#include "graph_util.cuh"
 #include "../../include/picmcc.h"
 
 namespace mlp {
@@ -53,201 +54,444 @@ __device__ __forceinline__ void mma_bf16(float (&c)[4], uint32_t a0, uint32_t a1
         : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
 }
 
-// ------------------------------------------------------------------ GEMM
-// C_part[z] = A[M][K-slice z] B[N][K-slice z]^T (both operands K-contiguous
-// BF16), FP32 out.  CTA tile 64 x 64, four warps of 32 x 32, K staged in
-// chunks of 32.  M, N multiples of 64; K a multiple of 32 * splits.
-constexpr int GT = 64, GK = 32, GPAD = 8;
-__global__ void __launch_bounds__(128) k_gemm_nt(const __nv_bfloat16* __restrict__ A,
-                                                 const __nv_bfloat16* __restrict__ B, float* __restrict__ C, int M,
-                                                 int N, int K, int k_per_split) {
-    __shared__ __align__(16) __nv_bfloat16 As[GT][GK + GPAD];
-    __shared__ __align__(16) __nv_bfloat16 Bs[GT][GK + GPAD];
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int g = lane >> 2, t = lane & 3;
-    const int m0 = blockIdx.y * GT, n0 = blockIdx.x * GT, kz0 = blockIdx.z * k_per_split;
-    const int wm = (warp >> 1) * 32, wn = (warp & 1) * 32;
-    float acc[2][4][4] = {};
-    for (int k0 = kz0; k0 < kz0 + k_per_split; k0 += GK) {
-        // 64 rows x 32 bf16 = 256 chunks of 16 B per operand: two per thread
-#pragma unroll
-        for (int u = 0; u < 2; ++u) {
-            const int q = tid + u * 128, r = q >> 2, c8 = (q & 3) * 8;
-            *reinterpret_cast<uint4*>(&As[r][c8]) =
-                *reinterpret_cast<const uint4*>(A + (size_t)(m0 + r) * K + k0 + c8);
-            *reinterpret_cast<uint4*>(&Bs[r][c8]) =
-                *reinterpret_cast<const uint4*>(B + (size_t)(n0 + r) * K + k0 + c8);
-        }
-        __syncthreads();
-#pragma unroll
-        for (int kk = 0; kk < GK; kk += 16) {
-            uint32_t a[2][4], b[4][2];
-#pragma unroll
-            for (int mi = 0; mi < 2; ++mi) {
-                const int r = wm + mi * 16 + g;
-                a[mi][0] = *reinterpret_cast<const uint32_t*>(&As[r][kk + 2 * t]);
-                a[mi][1] = *reinterpret_cast<const uint32_t*>(&As[r + 8][kk + 2 * t]);
-                a[mi][2] = *reinterpret_cast<const uint32_t*>(&As[r][kk + 2 * t + 8]);
-                a[mi][3] = *reinterpret_cast<const uint32_t*>(&As[r + 8][kk + 2 * t + 8]);
-            }
-#pragma unroll
-            for (int ni = 0; ni < 4; ++ni) {
-                const int r = wn + ni * 8 + g;
-                b[ni][0] = *reinterpret_cast<const uint32_t*>(&Bs[r][kk + 2 * t]);
-                b[ni][1] = *reinterpret_cast<const uint32_t*>(&Bs[r][kk + 2 * t + 8]);
-            }
-#pragma unroll
-            for (int mi = 0; mi < 2; ++mi)
-#pragma unroll
-                for (int ni = 0; ni < 4; ++ni)
-                    mma_bf16(acc[mi][ni], a[mi][0], a[mi][1], a[mi][2], a[mi][3], b[ni][0], b[ni][1]);
-        }
-        __syncthreads();
+__device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
+
+constexpr long long kWaitLimit = 1ll << 26;
+// Bounded wait for the barrier phase with the given parity; false on expiry.
+__device__ __forceinline__ bool bar_wait(uint32_t bar, uint32_t parity) {
+    for (long long it = 0; it < kWaitLimit; ++it) {
+        uint32_t done;
+        asm volatile(
+            "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+            "selp.u32 %0, 1, 0, p;\n\t}\n"
+            : "=r"(done)
+            : "r"(bar), "r"(parity)
+            : "memory");
+        if (done) return true;
     }
-    float* Cz = C + (size_t)blockIdx.z * M * N;
-#pragma unroll
-    for (int mi = 0; mi < 2; ++mi)
-#pragma unroll
-        for (int ni = 0; ni < 4; ++ni) {
-            const int r = m0 + wm + mi * 16 + g, c = n0 + wn + ni * 8 + 2 * t;
-            *reinterpret_cast<float2*>(Cz + (size_t)r * N + c) = make_float2(acc[mi][ni][0], acc[mi][ni][1]);
-            *reinterpret_cast<float2*>(Cz + (size_t)(r + 8) * N + c) = make_float2(acc[mi][ni][2], acc[mi][ni][3]);
-        }
+    return false;
 }
+
+__device__ __forceinline__ void fence_async_smem() { asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory"); }
 
 // ------------------------------------------------------------------ training kernels
-// BF16 copies of W2 ([o][i] and its transpose [i][o]).
-__global__ void k_prep(const float* __restrict__ th, __nv_bfloat16* __restrict__ w2b, __nv_bfloat16* __restrict__ w2t) {
+// BF16 copy of W2 ([o][i]).
+__global__ void k_prep(const float* __restrict__ th, __nv_bfloat16* __restrict__ w2b) {
     const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k < NH * NH) {
-        const int o = k / NH, i = k % NH;
-        const __nv_bfloat16 v = __float2bfloat16_rn(th[OFF_W2 + k]);
-        w2b[k] = v;
-        w2t[i * NH + o] = v;
+    if (k < NH * NH) w2b[k] = __float2bfloat16_rn(th[OFF_W2 + k]);
+}
+
+// Forward and backward pass of kPts points in one block: nothing of it but
+// the partial sums of the gradient leaves the chip.  The blocks of a split (up
+// to 256 points, the depth of one accumulator of the weight gradient) form a
+// cluster: every block copies its points' h1, and of dz2 the columns of their
+// rows of gW2, into the others' shared memory as soon as they exist (bulk
+// copies counted by the receiver's barrier: with 16-byte stores the two
+// exchanges took 5000 of 24000 clocks, gathered by loads at the end 7000).
+//
+// What bounds it: the chain of dependent phases (loads, layer 1, two products,
+// the head, its sums, the weight gradient; 600 to 2000 clocks each), one block
+// an SM (220 KB), 16 warps.  64 points a block because that is the length of
+// the partial sums.  4096 points: before, as six kernels with everything
+// between them in global memory (transposed copies with 2-byte stores, sums
+// read and written in shared memory), 51.9 us a step; now
+// 13.3 (this kernel ~10).
+constexpr int kPts = 64, kSplitPts = 256, kTrainThreads = 512, kHeadWarps = 8;
+constexpr int kHeadPart = NO * NH + NO + NH + 1;  // partial sums of a block: gW3[6][128], gb3[6], gb2[128], loss
+constexpr int kL1Part = NH * NI + NH;             // gW1[128][2], gb1[128]
+constexpr int kBRow = NH + 8, kFRow = NH + 4;     // padded rows (16-byte pieces of eight rows on different banks)
+// A cluster of `size` blocks: block r owns the 16-row tiles first(r) .. first(r + 1) - 1 of gW2.  dz2 is kept by
+// owner, [owner][point][columns], rows of 16 BF16 a tile and 8 of padding.
+__host__ __device__ constexpr int own_first(int r, int size) { return r * (NH / 16) / size; }
+__host__ __device__ constexpr int own_row(int r, int size) { return (own_first(r + 1, size) - own_first(r, size)) * 16 + 8; }
+constexpr int gd_size() {
+    int most = 0;
+    for (int size = 1; size <= kSplitPts / kPts; ++size)
+        for (int r = 0; r < size; ++r) {
+            const int n = size * kPts * own_row(r, size);
+            most = n > most ? n : most;
+        }
+    return most;
+}
+
+__device__ __forceinline__ int owner_of(int tile, int size) {
+    int r = 0;
+    while (own_first(r + 1, size) <= tile) ++r;
+    return r;
+}
+__device__ __forceinline__ int dz_base(int r, int size) { return kPts * (16 * own_first(r, size) + 8 * r); }
+
+struct TrainSmem {
+    __nv_bfloat16 gh[kSplitPts][kBRow], gd[gd_size()];  // h1 and dz2 of the split (the others write here)
+    __nv_bfloat16 dzb[kPts * (NH + 8 * (kSplitPts / kPts))];
+    union {
+        __nv_bfloat16 w2[NH][kBRow];
+        float part[kHeadWarps][kHeadPart + 1];  // once W2 is done with
+    };
+    float z[kPts][kFRow];  // z2, then h2, then dz1
+    float h1[kPts][kFRow];
+    float w3[NO * NH], dy[kPts][8], d[kPts][8], x[kPts][NI], tgt[kPts][NO];
+    unsigned long long bar;
+    int own_row[kSplitPts / kPts], own_base[kSplitPts / kPts];  // dzb by owner: columns a row, first element
+    int tile_row[NH / 16], tile_base[NH / 16];                  // and by 16-column tile
+};
+
+// Four 8 x 8 BF16 matrices (TR: transposed); lane l gives the address of row
+// l % 8 of matrix l / 8.
+template <bool TR> __device__ __forceinline__ void ldm4(uint32_t (&r)[4], uint32_t a) {
+    if (TR)
+        asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];"
+                     : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(a) : "memory");
+    else
+        asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
+                     : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(a) : "memory");
+}
+__device__ __forceinline__ uint32_t cluster_rank() {
+    uint32_t r;
+    asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+    return r;
+}
+__device__ __forceinline__ uint32_t cluster_size() {
+    uint32_t r;
+    asm("mov.u32 %0, %%cluster_nctarank;" : "=r"(r));
+    return r;
+}
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
+// Copies bytes (a multiple of 16) from this block's shared address src to
+// address dst of block `rank` of the cluster, whose barrier at bar counts them.
+__device__ __forceinline__ void copy_to_peer(uint32_t dst, uint32_t src, uint32_t bytes, uint32_t bar, uint32_t rank) {
+    uint32_t d, b;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(d) : "r"(dst), "r"(rank));
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(b) : "r"(bar), "r"(rank));
+    asm volatile("cp.async.bulk.shared::cluster.shared::cta.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(d),
+                 "r"(src), "r"(bytes), "r"(b)
+                 : "memory");
+}
+
+// acc += A B over K = 128 for a warp's 16 x 32 tile: A [m][k], the lane's
+// address for 16-column step k given by a_at(k); B from column n0, as [n][k]
+// or (BT) as [k][n]; k ascending, the operands of the next step loaded ahead.
+template <bool BT, class F>
+__device__ __forceinline__ void warp_tile(float (&acc)[4][4], F a_at, const __nv_bfloat16 (*B)[kBRow], int n0) {
+    const int lane = threadIdx.x & 31, r8 = lane & 7, q = lane >> 3;
+    uint32_t ba = BT ? smem_u32(&B[r8 + (q & 1) * 8][n0 + (q >> 1) * 8])
+                     : smem_u32(&B[n0 + r8 + (q >> 1) * 8][(q & 1) * 8]);
+    constexpr uint32_t kB = BT ? 16 * kBRow * 2 : 16 * 2, kH = BT ? 16 * 2 : 16 * kBRow * 2;
+    uint32_t a[2][4], b[2][2][4];
+    auto load = [&](int k) {
+        ldm4<false>(a[k & 1], a_at(k));
+        ldm4<BT>(b[k & 1][0], ba + k * kB);
+        ldm4<BT>(b[k & 1][1], ba + k * kB + kH);
+    };
+    load(0);
+#pragma unroll
+    for (int k = 0; k < NH / 16; ++k) {
+        const int s = k & 1;
+        if (k + 1 < NH / 16) load(k + 1);
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            mma_bf16(acc[2 * h], a[s][0], a[s][1], a[s][2], a[s][3], b[s][h][0], b[s][h][1]);
+            mma_bf16(acc[2 * h + 1], a[s][0], a[s][1], a[s][2], a[s][3], b[s][h][2], b[s][h][3]);
+        }
     }
 }
 
-// h1 = tanh(W1 x + b1): FP32 [n][128], BF16 [n][128] and BF16 transposed [128][n].
-__global__ void k_layer1(const float* __restrict__ th, const float* __restrict__ x, int n, float* __restrict__ h1,
-                         __nv_bfloat16* __restrict__ h1b, __nv_bfloat16* __restrict__ h1t) {
-    const int p = blockIdx.x, u = threadIdx.x;
-    if (p >= n) return;
-    const float z = fmaf(th[OFF_W1 + u * NI + 1], x[p * NI + 1], fmaf(th[OFF_W1 + u * NI], x[p * NI], th[OFF_B1 + u]));
-    const float h = tanh_fast(z);
-    h1[(size_t)p * NH + u] = h;
-    const __nv_bfloat16 hb = __float2bfloat16_rn(h);
-    h1b[(size_t)p * NH + u] = hb;
-    h1t[(size_t)u * n + p] = hb;
+// Sums over the lanes of 24 values, each by the butterfly 16, 8, 4, 2, 1 (lane
+// l adds lane l ^ 16 first), the values halved between the partners on the
+// way: the lane ends with the sum of value sum24_index(lane).
+__device__ __forceinline__ float sum24(float (&v)[24], int lane) {
+#pragma unroll
+    for (int j = 0; j < 12; ++j) {
+        const float keep = lane & 16 ? v[12 + j] : v[j], give = lane & 16 ? v[j] : v[12 + j];
+        v[j] = keep + __shfl_xor_sync(kFull, give, 16);
+    }
+#pragma unroll
+    for (int j = 0; j < 6; ++j) {
+        const float keep = lane & 8 ? v[6 + j] : v[j], give = lane & 8 ? v[j] : v[6 + j];
+        v[j] = keep + __shfl_xor_sync(kFull, give, 8);
+    }
+#pragma unroll
+    for (int j = 0; j < 3; ++j) {
+        const float keep = lane & 4 ? v[3 + j] : v[j], give = lane & 4 ? v[j] : v[3 + j];
+        v[j] = keep + __shfl_xor_sync(kFull, give, 4);
+    }
+    v[3] = 0.0f;
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {
+        const float keep = lane & 2 ? v[2 + j] : v[j], give = lane & 2 ? v[j] : v[2 + j];
+        v[j] = keep + __shfl_xor_sync(kFull, give, 2);
+    }
+    const float keep = lane & 1 ? v[1] : v[0], give = lane & 1 ? v[0] : v[1];
+    return keep + __shfl_xor_sync(kFull, give, 1);
+}
+__device__ __forceinline__ int sum24_index(int lane) {  // 24 and more: none
+    const int low = lane & 3;
+    return low == 3 ? 24 : (lane >> 4) * 12 + ((lane >> 3) & 1) * 6 + ((lane >> 2) & 1) * 3 + low;
 }
 
-// Output layer, loss and the first backward steps.  One warp per point (lane
-// l holds hidden units l, l+32, l+64, l+96), kHeadPts points per block.
-// Per-block partial sums: gW3[6][128], gb3[6], gb2[128], loss.
-constexpr int kHeadWarps = 8, kHeadPts = 64, kHeadPart = NO * NH + NO + NH + 1;
-__global__ void __launch_bounds__(kHeadWarps * 32) k_head(const float* __restrict__ th, const float* __restrict__ z2,
-                                                          const float* __restrict__ tgt, int n, float inv6n,
-                                                          __nv_bfloat16* __restrict__ dz2b,
-                                                          __nv_bfloat16* __restrict__ dz2t, float* __restrict__ part) {
-    __shared__ float sW3[NO * NH], sgW3[kHeadWarps][NO * NH], sgb2[kHeadWarps][NH], sgb3[kHeadWarps][NO],
-        sloss[kHeadWarps];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    for (int k = threadIdx.x; k < NO * NH; k += blockDim.x) sW3[k] = th[OFF_W3 + k];
-    for (int k = lane; k < NO * NH; k += 32) sgW3[warp][k] = 0.0f;
-    for (int k = lane; k < NH; k += 32) sgb2[warp][k] = 0.0f;
-    if (lane < NO) sgb3[warp][lane] = 0.0f;
-    if (lane == 0) sloss[warp] = 0.0f;
+// head: [block][kHeadPart], l1: [block][kL1Part], gw2: [cluster][128][128].
+__global__ void __launch_bounds__(kTrainThreads, 1)
+    k_backprop(const float* __restrict__ th, const __nv_bfloat16* __restrict__ w2b, const float* __restrict__ x,
+               const float* __restrict__ tgt, float inv6n, float* __restrict__ head, float* __restrict__ l1,
+               float* __restrict__ gw2) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    TrainSmem& S = *reinterpret_cast<TrainSmem*>(smem_raw);
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int u = tid & (NH - 1), grp = tid >> 7;
+    const int size = (int)cluster_size(), rank = (int)cluster_rank();
+    const int own0 = own_first(rank, size), nt = own_first(rank + 1, size) - own0, row = own_row(rank, size);
+    const size_t p0 = (size_t)blockIdx.x * kPts;
+    __nv_bfloat16 (*h1b)[kBRow] = S.gh + rank * kPts;
+    const uint32_t bar = smem_u32(&S.bar);
+    if (tid == 0) {
+        // one phase: h1 of the other blocks, dz2 of all
+        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(bar) : "memory");
+        asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
+        const uint32_t bytes = (size - 1) * sizeof(S.gh) / (kSplitPts / kPts) + size * kPts * row * 2;
+        asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"(bar), "r"(bytes) : "memory");
+    }
+    __syncwarp();
+    cluster_arrive();  // (1) this block runs and its barrier stands
+    // nothing of this depends on the kernel before
+    if (tid >= 64 && tid < 64 + size) {
+        S.own_row[tid - 64] = own_row(tid - 64, size);
+        S.own_base[tid - 64] = dz_base(tid - 64, size);
+    }
+    if (tid >= 96 && tid < 96 + NH / 16) {
+        const int k = tid - 96, r = owner_of(k, size);
+        S.tile_row[k] = own_row(r, size);
+        S.tile_base[k] = dz_base(r, size) + 16 * (k - own_first(r, size));
+    }
+    if (tid < kPts * NI) (&S.x[0][0])[tid] = x[p0 * NI + tid];
+    if (tid < kPts * NO) (&S.tgt[0][0])[tid] = tgt[p0 * NO + tid];
     __syncthreads();
+    pic::pdl_wait();
+    cudaTriggerProgrammaticLaunchCompletion();
+    const float w10 = th[OFF_W1 + u * NI], w11 = th[OFF_W1 + u * NI + 1], b1 = th[OFF_B1 + u];
+    uint4 wv[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) wv[j] = reinterpret_cast<const uint4*>(w2b)[tid + j * kTrainThreads];
+    const float w3a = th[OFF_W3 + tid], w3b = tid < NO * NH - kTrainThreads ? th[OFF_W3 + kTrainThreads + tid] : 0.0f;
     float b2[4];
 #pragma unroll
     for (int q = 0; q < 4; ++q) b2[q] = th[OFF_B2 + lane + 32 * q];
-    // training batches are multiples of kHeadPts (train_size_ok): every point
-    // of the block exists; the next point's z2 row is loaded ahead
-    float zn[4];
+    const int si = sum24_index(lane);
+    const float b3 = si < 24 ? th[OFF_B3 + si % NO] : 0.0f;
+    // h1 = tanh(W1 x + b1)
+#pragma unroll 4
+    for (int p = grp; p < kPts; p += kTrainThreads / NH) {
+        const float h = tanh_fast(fmaf(w11, S.x[p][1], fmaf(w10, S.x[p][0], b1)));
+        S.h1[p][u] = h;
+        h1b[p][u] = __float2bfloat16_rn(h);
+    }
 #pragma unroll
-    for (int q = 0; q < 4; ++q) zn[q] = z2[(size_t)(blockIdx.x * kHeadPts + warp) * NH + lane + 32 * q];
-    for (int pp = warp; pp < kHeadPts; pp += kHeadWarps) {
-        const int p = blockIdx.x * kHeadPts + pp;
-        float h2[4];
+    for (int j = 0; j < 4; ++j) {
+        const int q = tid + j * kTrainThreads;  // 16 pieces a row
+        *reinterpret_cast<uint4*>(&S.w2[q >> 4][(q & 15) * 8]) = wv[j];
+    }
+    S.w3[tid] = w3a;
+    if (tid < NO * NH - kTrainThreads) S.w3[kTrainThreads + tid] = w3b;
+    fence_async_smem();
+    __syncthreads();
+    cluster_wait();  // (1)
+    if (tid < size && tid != rank)
+        copy_to_peer(smem_u32(h1b), smem_u32(h1b), sizeof(S.gh) / (kSplitPts / kPts), bar, tid);
+    const int m0 = (warp & 3) * 16, n0 = (warp >> 2) * 32, g = lane >> 2, t = lane & 3;
+    {
+        float acc[4][4] = {};
+        const uint32_t a0 = smem_u32(&h1b[m0 + (lane & 15)][(lane >> 4) * 8]);
+        warp_tile<false>(acc, [&](int k) { return a0 + k * 32; }, S.w2, n0);  // z2 = h1 W2^T
 #pragma unroll
-        for (int q = 0; q < 4; ++q) h2[q] = tanh_fast(zn[q] + b2[q]);
-        if (pp + kHeadWarps < kHeadPts) {
-#pragma unroll
-            for (int q = 0; q < 4; ++q) zn[q] = z2[(size_t)(p + kHeadWarps) * NH + lane + 32 * q];
-        }
-        float dy[NO];
-        float lsum = 0.0f;
-#pragma unroll
-        for (int o = 0; o < NO; ++o) {
-            float s = 0.0f;
-#pragma unroll
-            for (int q = 0; q < 4; ++q) s = fmaf(sW3[o * NH + lane + 32 * q], h2[q], s);
-            for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(kFull, s, off);
-            const float y = s + th[OFF_B3 + o];
-            const float d = y - tgt[(size_t)p * NO + o];
-            lsum = fmaf(d, d, lsum);
-            dy[o] = 2.0f * d * inv6n;
-        }
-        if (lane == 0) sloss[warp] += lsum;
-        if (lane < NO) {
-            float v = 0.0f;
-#pragma unroll
-            for (int o = 0; o < NO; ++o) v = lane == o ? dy[o] : v;
-            sgb3[warp][lane] += v;
-        }
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            const int u = lane + 32 * q;
-            float dh = 0.0f;
-#pragma unroll
-            for (int o = 0; o < NO; ++o) {
-                sgW3[warp][o * NH + u] += dy[o] * h2[q];
-                dh = fmaf(sW3[o * NH + u], dy[o], dh);
-            }
-            const float dz = dh * (1.0f - h2[q] * h2[q]);
-            sgb2[warp][u] += dz;
-            const __nv_bfloat16 db = __float2bfloat16_rn(dz);
-            dz2b[(size_t)p * NH + u] = db;
-            dz2t[(size_t)u * n + p] = db;
+        for (int j = 0; j < 4; ++j) {
+            *reinterpret_cast<float2*>(&S.z[m0 + g][n0 + 8 * j + 2 * t]) = make_float2(acc[j][0], acc[j][1]);
+            *reinterpret_cast<float2*>(&S.z[m0 + g + 8][n0 + 8 * j + 2 * t]) = make_float2(acc[j][2], acc[j][3]);
         }
     }
     __syncthreads();
-    float* out = part + (size_t)blockIdx.x * kHeadPart;
-    for (int k = threadIdx.x; k < kHeadPart; k += blockDim.x) {
-        float s = 0.0f;
-        for (int w = 0; w < kHeadWarps; ++w) {
-            if (k < NO * NH) s += sgW3[w][k];
-            else if (k < NO * NH + NO) s += sgb3[w][k - NO * NH];
-            else if (k < NO * NH + NO + NH) s += sgb2[w][k - NO * NH - NO];
-            else s += sloss[w];
+    // output layer: a warp takes four points, a lane units lane, lane + 32, ...
+    {
+        float y[24], w3[NO][4];
+#pragma unroll
+        for (int o = 0; o < NO; ++o)
+#pragma unroll
+            for (int q = 0; q < 4; ++q) w3[o][q] = S.w3[o * NH + lane + 32 * q];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            float h2[4];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                float* zp = &S.z[warp * 4 + j][lane + 32 * q];
+                h2[q] = tanh_fast(*zp + b2[q]);
+                *zp = h2[q];
+            }
+#pragma unroll
+            for (int o = 0; o < NO; ++o) {
+                float s = 0.0f;
+#pragma unroll
+                for (int q = 0; q < 4; ++q) s = fmaf(w3[o][q], h2[q], s);
+                y[j * NO + o] = s;
+            }
         }
-        out[k] = s;
+        const float yo = sum24(y, lane) + b3;
+        if (si < 24) {
+            const int p = warp * 4 + si / NO, o = si % NO;
+            const float d = yo - S.tgt[p][o];
+            S.d[p][o] = d;
+            S.dy[p][o] = 2.0f * d * inv6n;
+        }
     }
-}
-
-// dz1 = dh1 (1 - h1^2); per-block partials of gW1[128][2] and gb1[128] over
-// kL1Pts points (thread = hidden unit).  Training batches are multiples of
-// kL1Pts (train_size_ok), so every block has all of its points; the loop is
-// unrolled so that the loads of several points are in flight together (the
-// sums still run over the points in order).
-constexpr int kL1Pts = 64, kL1Part = NH * NI + NH;
-__global__ void __launch_bounds__(NH) k_layer1_back(const float* __restrict__ dh1, const float* __restrict__ h1,
-                                                    const float* __restrict__ x, int n, float* __restrict__ part) {
-    (void)n;
-    const int u = threadIdx.x;
-    float g0 = 0.0f, g1 = 0.0f, gb = 0.0f;
-#pragma unroll 16
-    for (int pp = 0; pp < kL1Pts; ++pp) {
-        const int p = blockIdx.x * kL1Pts + pp;
-        const float h = h1[(size_t)p * NH + u];
-        const float dz = dh1[(size_t)p * NH + u] * (1.0f - h * h);
-        g0 = fmaf(dz, x[p * NI], g0);
-        g1 = fmaf(dz, x[p * NI + 1], g1);
-        gb += dz;
+    __syncthreads();
+    // dz2 and the sums over the points: eight chains (points w, w + 8, ...), kept for the sum of the eight in order
+    float acc3[2][NO], gb2[2];
+    {
+        float w3[NO];
+#pragma unroll
+        for (int o = 0; o < NO; ++o) w3[o] = S.w3[o * NH + u];
+        const int dzr = S.tile_row[u / 16];
+        __nv_bfloat16* dzc = S.dzb + S.tile_base[u / 16] + u % 16;
+#pragma unroll
+        for (int v = 0; v < 2; ++v) {
+#pragma unroll
+            for (int o = 0; o < NO; ++o) acc3[v][o] = 0.0f;
+            gb2[v] = 0.0f;
+        }
+#pragma unroll 2
+        for (int c = 0; c < kPts / kHeadWarps; ++c)
+#pragma unroll
+            for (int v = 0; v < 2; ++v) {
+                const int p = 2 * grp + v + c * kHeadWarps;
+                const float h2 = S.z[p][u];
+                const float4 da = *reinterpret_cast<const float4*>(&S.dy[p][0]);
+                const float2 db = *reinterpret_cast<const float2*>(&S.dy[p][4]);
+                const float dy[NO] = {da.x, da.y, da.z, da.w, db.x, db.y};
+                float dh = 0.0f;
+#pragma unroll
+                for (int o = 0; o < NO; ++o) {
+                    acc3[v][o] = fmaf(dy[o], h2, acc3[v][o]);
+                    dh = fmaf(w3[o], dy[o], dh);
+                }
+                const float dz = __fmul_rn(dh, fmaf(-h2, h2, 1.0f));
+                gb2[v] = __fadd_rn(gb2[v], dz);
+                dzc[p * dzr] = __float2bfloat16_rn(dz);
+            }
     }
-    float* out = part + (size_t)blockIdx.x * kL1Part;
-    out[u * NI] = g0;
-    out[u * NI + 1] = g1;
-    out[NH * NI + u] = gb;
+    fence_async_smem();
+    __syncthreads();
+    // dz2 to the owners of its columns
+    if (tid < size) {
+        const int to = S.own_row[tid];
+        copy_to_peer(smem_u32(&S.gd[rank * kPts * to]), smem_u32(&S.dzb[S.own_base[tid]]), kPts * to * 2, bar, tid);
+    }
+    {
+        float acc[4][4] = {};
+        const uint32_t a0 = smem_u32(&S.dzb[(lane >> 4) * 8]);
+        const int pr = m0 + (lane & 15);
+        warp_tile<true>(acc, [&](int k) { return a0 + 2 * (S.tile_base[k] + pr * S.tile_row[k]); },  // dh1 = dz2 W2
+                        S.w2, n0);
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {  // dz1 = dh1 (1 - h1^2)
+                const int p = m0 + g + 8 * h, i = n0 + 8 * j + 2 * t;
+                const float2 h1 = *reinterpret_cast<const float2*>(&S.h1[p][i]);
+                *reinterpret_cast<float2*>(&S.z[p][i]) =
+                    make_float2(__fmul_rn(acc[j][2 * h], fmaf(-h1.x, h1.x, 1.0f)),
+                                __fmul_rn(acc[j][2 * h + 1], fmaf(-h1.y, h1.y, 1.0f)));
+            }
+    }
+    __syncthreads();
+#pragma unroll
+    for (int v = 0; v < 2; ++v) {
+#pragma unroll
+        for (int o = 0; o < NO; ++o) S.part[2 * grp + v][o * NH + u] = acc3[v][o];
+        S.part[2 * grp + v][NO * NH + NO + u] = gb2[v];
+    }
+    if (tid < kHeadWarps * (NO + 1)) {
+        const int w = tid / (NO + 1), o = tid % (NO + 1);
+        float s = 0.0f;
+        for (int p = w; p < kPts; p += kHeadWarps) {
+            if (o < NO) {
+                s += S.dy[p][o];
+            } else {
+                float l = 0.0f;
+                for (int q = 0; q < NO; ++q) l = fmaf(S.d[p][q], S.d[p][q], l);
+                s += l;
+            }
+        }
+        S.part[w][o < NO ? NO * NH + o : kHeadPart - 1] = s;
+    }
+    // sums of dz1 over the points, in order
+    if (grp == 3) {
+        float g0 = 0.0f, g1 = 0.0f, gb = 0.0f;
+#pragma unroll 8
+        for (int p = 0; p < kPts; ++p) {
+            const float dz = S.z[p][u];
+            const float2 xp = *reinterpret_cast<const float2*>(&S.x[p][0]);
+            g0 = fmaf(dz, xp.x, g0);
+            g1 = fmaf(dz, xp.y, g1);
+            gb += dz;
+        }
+        float* out = l1 + (size_t)blockIdx.x * kL1Part;
+        out[u * NI] = g0;
+        out[u * NI + 1] = g1;
+        out[NH * NI + u] = gb;
+    }
+    __syncthreads();
+#pragma unroll 1
+    for (int k = tid; k < kHeadPart; k += kTrainThreads) {
+        float s = 0.0f;
+#pragma unroll
+        for (int w = 0; w < kHeadWarps; ++w) s += S.part[w][k];
+        head[(size_t)blockIdx.x * kHeadPart + k] = s;
+    }
+    const bool got = bar_wait(bar, 0);
+    __syncwarp();
+    cluster_arrive();  // (2) what this block was sent has arrived
+    // gW2 = dz2^T h1 over the split's points, in order: this block's 16-row tiles
+    const int pts = got ? size * kPts : 0;
+    float* out = gw2 + ((size_t)(blockIdx.x / size) * NH + own0 * 16) * NH;
+    // a warp takes 16 columns of two row tiles (half the warps of 32 x 16: 1536 clocks of shared-memory reads
+    // in place of 2048)
+    const int r8 = lane & 7, q4 = lane >> 3;
+#pragma unroll 1
+    for (int it = warp; it < (nt + 1) / 2 * 8; it += kTrainThreads / 32) {
+        const int o0 = (it >> 3) * 32, i0 = (it & 7) * 16;
+        const bool two = o0 + 16 < nt * 16;
+        uint32_t aa = smem_u32(&S.gd[(r8 + (q4 >> 1) * 8) * row + o0 + (q4 & 1) * 8]);
+        uint32_t ba = smem_u32(&S.gh[r8 + (q4 & 1) * 8][i0 + (q4 >> 1) * 8]);
+        const uint32_t a2 = two ? 32 : 0;
+        float acc[4][4] = {};
+        if (!got) acc[0][0] = __int_as_float(0x7fc00000);  // the wait expired: no gradient
+#pragma unroll 1
+        for (int k = 0; k < pts; k += 64) {
+            uint32_t a[4][2][4], b[4][4];
+#pragma unroll
+            for (int s = 0; s < 4; ++s) {
+                ldm4<true>(a[s][0], aa);
+                ldm4<true>(b[s], ba);
+                ldm4<true>(a[s][1], aa + a2);
+                aa += 16 * row * 2;
+                ba += 16 * kBRow * 2;
+            }
+#pragma unroll
+            for (int s = 0; s < 4; ++s)
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    mma_bf16(acc[2 * h], a[s][h][0], a[s][h][1], a[s][h][2], a[s][h][3], b[s][0], b[s][1]);
+                    mma_bf16(acc[2 * h + 1], a[s][h][0], a[s][h][1], a[s][h][2], a[s][h][3], b[s][2], b[s][3]);
+                }
+        }
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const int r = o0 + (j >> 1) * 16 + g, c = i0 + 8 * (j & 1) + 2 * t;
+            if (j >= 2 && !two) break;
+            *reinterpret_cast<float2*>(out + r * NH + c) = make_float2(acc[j][0], acc[j][1]);
+            *reinterpret_cast<float2*>(out + (r + 8) * NH + c) = make_float2(acc[j][2], acc[j][3]);
+        }
+    }
+    __syncwarp();
+    cluster_wait();  // (2) this block's memory has been read
 }
 
 struct Parts {
@@ -257,67 +501,69 @@ struct Parts {
     int splits, n_head, n_l1;
 };
 
-// Gradient of parameter k from the partial sums, added in a fixed order.
-__device__ float grad_of(const Parts& P, int k) {
+// Sum of n values `stride` apart, in order, 64 loads in flight.
+__device__ __forceinline__ float sum_rows(const float* __restrict__ p, size_t stride, int n) {
     float s = 0.0f;
-    if (k < OFF_W2) {
-        const int j = k;  // W1 then b1: same order as the l1 partial layout
-        for (int b = 0; b < P.n_l1; ++b) s += P.l1[(size_t)b * kL1Part + j];
-    } else if (k < OFF_B2) {
-        for (int z = 0; z < P.splits; ++z) s += P.gw2[(size_t)z * NH * NH + (k - OFF_W2)];
-    } else {
-        int j;
-        if (k < OFF_W3) j = NO * NH + NO + (k - OFF_B2);        // b2
-        else if (k < OFF_B3) j = k - OFF_W3;                      // W3
-        else j = NO * NH + (k - OFF_B3);                          // b3
-        for (int b = 0; b < P.n_head; ++b) s += P.head[(size_t)b * kHeadPart + j];
+    for (; n >= 64; n -= 64) {
+        float v[64];
+#pragma unroll
+        for (int q = 0; q < 64; ++q, p += stride) v[q] = *p;
+#pragma unroll
+        for (int q = 0; q < 64; ++q) s += v[q];
     }
+#pragma unroll 16
+    for (; n > 0; --n, p += stride) s += *p;
     return s;
 }
+
+// Gradient of parameter k from the partial sums, added in a fixed order.
+__device__ __forceinline__ float grad_of(const Parts& P, int k) {
+    // W1 then b1, b2, W3, b3: places in the rows of partial sums
+    if (k < OFF_W2) return sum_rows(P.l1 + k, kL1Part, P.n_l1);
+    if (k < OFF_B2) return sum_rows(P.gw2 + (k - OFF_W2), NH * NH, P.splits);
+    const int j = k < OFF_W3 ? NO * NH + NO + (k - OFF_B2) : (k < OFF_B3 ? k - OFF_W3 : NO * NH + (k - OFF_B3));
+    return sum_rows(P.head + j, kHeadPart, P.n_head);
+}
+
+__device__ __forceinline__ void write_loss(const Parts& P, float* loss, float inv6n) {
+    if (loss) *loss = sum_rows(P.head + kHeadPart - 1, kHeadPart, P.n_head) * inv6n;
+}
+// A thread beyond the parameters (of another warp) adds the loss.
+constexpr int kParamThreads = 128, kParamBlocks = NP / kParamThreads + 1, kLossThread = kParamBlocks * kParamThreads - 1;
+static_assert(kLossThread >= NP, "a thread for the loss");
 
 __global__ void k_grad_out(Parts P, float* __restrict__ grad, float* __restrict__ loss, float inv6n) {
     const int k = blockIdx.x * blockDim.x + threadIdx.x;
     if (k < NP) grad[k] = grad_of(P, k);
-    if (k == 0 && loss) {
-        float s = 0.0f;
-        for (int b = 0; b < P.n_head; ++b) s += P.head[(size_t)b * kHeadPart + kHeadPart - 1];
-        *loss = s * inv6n;
-    }
+    if (k == kLossThread) write_loss(P, loss, inv6n);
 }
 
-// Adam (Kingma & Ba 2015, Algorithm 1) on every parameter, then the BF16
-// copies of W2 for the next step.  step_dev holds the step count (t >= 1
-// after the increment here, done by thread 0 of block 0 at the end).
-__global__ void k_adam(Parts P, float* __restrict__ th, float* __restrict__ m, float* __restrict__ v,
-                       int* __restrict__ step_dev, float lr, float beta1, float beta2, float eps,
-                       __nv_bfloat16* __restrict__ w2b, __nv_bfloat16* __restrict__ w2t, float* __restrict__ loss,
-                       float inv6n) {
+// Adam (Kingma & Ba 2015, Algorithm 1), step `step` (from 1), on every
+// parameter, then the BF16 copy of W2 for the next step.  One round trip for
+// up to 64 rows of partial sums, which the rest hides behind; the loss on a warp
+// of its own.  4096 points: ~3 us behind the kernel before (6.3 with dependent
+// loads and a kernel that counted the steps).
+__global__ void __launch_bounds__(kParamThreads) k_adam(Parts P, float* __restrict__ th, float* __restrict__ m,
+                                                        float* __restrict__ v, int step, float lr, float beta1,
+                                                        float beta2, float eps, __nv_bfloat16* __restrict__ w2b,
+                                                        float* __restrict__ loss, float inv6n) {
     const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    const int step = *step_dev + 1;
+    const float c1 = 1.0f - powf(beta1, (float)step), c2 = 1.0f - powf(beta2, (float)step);
+    pic::pdl_wait();
+    cudaTriggerProgrammaticLaunchCompletion();
     if (k < NP) {
+        const float m0 = m[k], v0 = v[k], t0 = th[k];
         const float gk = grad_of(P, k);
-        const float mk = beta1 * m[k] + (1.0f - beta1) * gk;
-        const float vk = beta2 * v[k] + (1.0f - beta2) * gk * gk;
+        const float mk = fmaf(1.0f - beta1, gk, beta1 * m0);
+        const float vk = fmaf((1.0f - beta2) * gk, gk, beta2 * v0);
         m[k] = mk;
         v[k] = vk;
-        const float c1 = 1.0f - powf(beta1, (float)step), c2 = 1.0f - powf(beta2, (float)step);
-        const float nt = th[k] - lr * (mk / c1) / (sqrtf(vk / c2) + eps);
+        const float nt = t0 - lr * (mk / c1) / (sqrtf(vk / c2) + eps);
         th[k] = nt;
-        if (k >= OFF_W2 && k < OFF_B2) {
-            const int o = (k - OFF_W2) / NH, i = (k - OFF_W2) % NH;
-            const __nv_bfloat16 b = __float2bfloat16_rn(nt);
-            w2b[o * NH + i] = b;
-            w2t[i * NH + o] = b;
-        }
+        if (k >= OFF_W2 && k < OFF_B2) w2b[k - OFF_W2] = __float2bfloat16_rn(nt);
     }
-    if (k == 0 && loss) {
-        float s = 0.0f;
-        for (int b = 0; b < P.n_head; ++b) s += P.head[(size_t)b * kHeadPart + kHeadPart - 1];
-        *loss = s * inv6n;
-    }
+    if (k == kLossThread) write_loss(P, loss, inv6n);
 }
-
-__global__ void k_step_inc(int* step_dev) { *step_dev += 1; }
 
 // ------------------------------------------------------------------ inference
 // Fused forward pass.  Four warps per block; each warp takes 16 points at a
@@ -453,7 +699,6 @@ constexpr int kTcThreads = 256, kTcRows = 128;
 constexpr uint32_t kTile = kTcRows * NH * 2;   // one 128 x 128 BF16 operand: 32 KB
 constexpr uint32_t kLbo = 128, kSbo = 2048;    // core-matrix strides (bytes) along K and along M/N
 constexpr uint32_t kB2Bytes = 16 * NH * 2;     // W3 padded to 16 rows: 4 KB
-constexpr long long kWaitLimit = 1ll << 26;
 
 struct TcSmem {
     alignas(1024) unsigned char w2[kTile];   // B of layer 2: row o (output unit), K = input unit
@@ -469,8 +714,6 @@ struct TcSmem {
 __host__ __device__ constexpr uint32_t kmajor_off(uint32_t r, uint32_t k) {
     return (r >> 3) * kSbo + (k >> 3) * kLbo + (r & 7) * 16 + (k & 7) * 2;
 }
-
-__device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
 // Shared-memory matrix descriptor: start address, leading (K) and stride
 // (M/N) byte offsets in 16-byte units, the fixed version bits 46-47 = 1,
@@ -499,24 +742,8 @@ __device__ __forceinline__ void tc_commit(uint32_t bar) {
                  : "memory");
 }
 
-// Bounded wait for the barrier phase with the given parity; false on expiry.
-__device__ __forceinline__ bool bar_wait(uint32_t bar, uint32_t parity) {
-    for (long long it = 0; it < kWaitLimit; ++it) {
-        uint32_t done;
-        asm volatile(
-            "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-            "selp.u32 %0, 1, 0, p;\n\t}\n"
-            : "=r"(done)
-            : "r"(bar), "r"(parity)
-            : "memory");
-        if (done) return true;
-    }
-    return false;
-}
-
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory"); }
-__device__ __forceinline__ void fence_async_smem() { asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory"); }
 
 __device__ __forceinline__ void tmem_ld32(uint32_t taddr, float (&v)[32]) {
     uint32_t r[32];
@@ -747,9 +974,9 @@ namespace {
 size_t al256(size_t b) { return (b + 255) & ~(size_t)255; }
 
 struct TrainWs {
-    __nv_bfloat16 *w2b, *w2t, *h1b, *h1t, *dz2b, *dz2t;
-    float *h1, *z2, *dh1, *gw2, *head, *l1, *loss;
-    int *step, *err;
+    __nv_bfloat16* w2b;
+    float *gw2, *head, *l1;  // partial sums
+    int* err;
     int splits, n_head, n_l1;
 };
 
@@ -762,24 +989,12 @@ size_t carve(void* base, int n, TrainWs* w) {
         p += al256(b);
         return r;
     };
-    const size_t nh = (size_t)n * NH;
-    w->splits = n >= 256 ? n / 256 : 1;
-    w->n_head = (n + kHeadPts - 1) / kHeadPts;
-    w->n_l1 = (n + kL1Pts - 1) / kL1Pts;
+    w->splits = n >= kSplitPts ? n / kSplitPts : 1;
+    w->n_head = w->n_l1 = n / kPts;
     w->w2b = (__nv_bfloat16*)take(NH * NH * 2);
-    w->w2t = (__nv_bfloat16*)take(NH * NH * 2);
-    w->h1 = (float*)take(nh * 4);
-    w->h1b = (__nv_bfloat16*)take(nh * 2);
-    w->h1t = (__nv_bfloat16*)take(nh * 2);
-    w->z2 = (float*)take(nh * 4);
-    w->dz2b = (__nv_bfloat16*)take(nh * 2);
-    w->dz2t = (__nv_bfloat16*)take(nh * 2);
-    w->dh1 = (float*)take(nh * 4);
     w->gw2 = (float*)take((size_t)w->splits * NH * NH * 4);
     w->head = (float*)take((size_t)w->n_head * kHeadPart * 4);
     w->l1 = (float*)take((size_t)w->n_l1 * kL1Part * 4);
-    w->loss = (float*)take(64);
-    w->step = (int*)take(64);
     w->err = (int*)take(64);
     return (size_t)(p - p0);
 }
@@ -796,14 +1011,28 @@ Parts parts_of(const TrainWs& w) {
 }
 
 // Forward and backward over the batch: leaves the partial sums in the workspace.
-void backprop(const float* th, const float* x, const float* t, int n, const TrainWs& w, cudaStream_t s) {
+cudaError_t backprop(const float* th, const float* x, const float* t, int n, const TrainWs& w, cudaStream_t s) {
     const float inv6n = 1.0f / (6.0f * (float)n);
-    k_layer1<<<n, NH, 0, s>>>(th, x, n, w.h1, w.h1b, w.h1t);
-    k_gemm_nt<<<dim3(NH / GT, n / GT, 1), 128, 0, s>>>(w.h1b, w.w2b, w.z2, n, NH, NH, NH);
-    k_head<<<w.n_head, kHeadWarps * 32, 0, s>>>(th, w.z2, t, n, inv6n, w.dz2b, w.dz2t, w.head);
-    k_gemm_nt<<<dim3(NH / GT, n / GT, 1), 128, 0, s>>>(w.dz2b, w.w2t, w.dh1, n, NH, NH, NH);
-    k_layer1_back<<<w.n_l1, NH, 0, s>>>(w.dh1, w.h1, x, n, w.l1);
-    k_gemm_nt<<<dim3(NH / GT, NH / GT, w.splits), 128, 0, s>>>(w.dz2t, w.h1t, w.gw2, NH, NH, n, n / w.splits);
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(n / kPts);
+    cfg.blockDim = dim3(kTrainThreads);
+    cfg.dynamicSmemBytes = sizeof(TrainSmem);
+    cfg.stream = s;
+    cudaLaunchAttribute at[2];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    at[1].id = cudaLaunchAttributeClusterDimension;
+    at[1].val.clusterDim.x = n / kPts / w.splits;
+    at[1].val.clusterDim.y = at[1].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 2;
+    return cudaLaunchKernelEx(&cfg, k_backprop, th, (const __nv_bfloat16*)w.w2b, x, t, inv6n, w.head, w.l1, w.gw2);
+}
+cudaError_t backprop_prepare(const float* params, const TrainWs& w, cudaStream_t s) {
+    const cudaError_t e =
+        cudaFuncSetAttribute(k_backprop, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(TrainSmem));
+    if (e == cudaSuccess) k_prep<<<(NH * NH + 255) / 256, 256, 0, s>>>(params, w.w2b);
+    return e;
 }
 
 bool train_size_ok(int n) { return n >= 64 && n % 64 == 0 && (n < 256 || n % 256 == 0); }
@@ -825,7 +1054,7 @@ extern "C" int mlp_forward_variant(const float* params, const float* x, float* y
     cudaStream_t s = (cudaStream_t)stream;
     TrainWs w;
     carve(ws, 64, &w);
-    k_prep<<<(NH * NH + 255) / 256, 256, 0, s>>>(params, w.w2b, w.w2t);
+    k_prep<<<(NH * NH + 255) / 256, 256, 0, s>>>(params, w.w2b);
     int dev = 0, sms = 0, per_sm = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
@@ -898,9 +1127,9 @@ extern "C" int mlp_loss_grad(const float* params, const float* x, const float* t
     cudaStream_t s = (cudaStream_t)stream;
     TrainWs w;
     carve(ws, n, &w);
-    k_prep<<<(NH * NH + 255) / 256, 256, 0, s>>>(params, w.w2b, w.w2t);
-    backprop(params, x, t, n, w, s);
-    k_grad_out<<<(NP + 255) / 256, 256, 0, s>>>(parts_of(w), grad, loss, 1.0f / (6.0f * (float)n));
+    if (backprop_prepare(params, w, s) != cudaSuccess || backprop(params, x, t, n, w, s) != cudaSuccess)
+        return PIC_ERR_CUDA;
+    k_grad_out<<<kParamBlocks, kParamThreads, 0, s>>>(parts_of(w), grad, loss, 1.0f / (6.0f * (float)n));
     return cudaGetLastError() == cudaSuccess ? PIC_OK : PIC_ERR_CUDA;
 }
 
@@ -916,35 +1145,13 @@ extern "C" int mlp_train(float* params, float* m, float* v, int step0, const flo
     TrainWs w;
     carve(ws, n, &w);
     const float inv6n = 1.0f / (6.0f * (float)n);
-    if (cudaMemcpyAsync(w.step, &step0, sizeof(int), cudaMemcpyHostToDevice, s) != cudaSuccess) return PIC_ERR_CUDA;
-    k_prep<<<(NH * NH + 255) / 256, 256, 0, s>>>(params, w.w2b, w.w2t);
-    auto one_step = [&](cudaStream_t q) {
-        backprop(params, x, t, n, w, q);
-        k_adam<<<(NP + 255) / 256, 256, 0, q>>>(parts_of(w), params, m, v, w.step, lr, beta1, beta2, eps, w.w2b,
-                                               w.w2t, loss, inv6n);
-        k_step_inc<<<1, 1, 0, q>>>(w.step);
-    };
-    if (n_steps < 8) {
-        for (int k = 0; k < n_steps; ++k) one_step(s);
-        return cudaGetLastError() == cudaSuccess ? PIC_OK : PIC_ERR_CUDA;
+    // two launches a step, queued faster than they run (a recorded graph of them would cost more than it saves)
+    cudaError_t e = backprop_prepare(params, w, s);
+    for (int k = 0; k < n_steps && e == cudaSuccess; ++k) {
+        e = backprop(params, x, t, n, w, s);
+        if (e == cudaSuccess)
+            pic::launch_pdl(k_adam, dim3(kParamBlocks), dim3(kParamThreads), 0, s, parts_of(w), params, m, v,
+                            step0 + k + 1, lr, beta1, beta2, eps, w.w2b, loss, inv6n);
     }
-    // longer runs: one step captured as a graph on a private stream, replayed on s
-    cudaStream_t cap = nullptr;
-    cudaGraph_t gr = nullptr;
-    cudaGraphExec_t ge = nullptr;
-    int rc = PIC_OK;
-    if (cudaStreamCreateWithFlags(&cap, cudaStreamNonBlocking) != cudaSuccess) return PIC_ERR_CUDA;
-    if (cudaStreamBeginCapture(cap, cudaStreamCaptureModeThreadLocal) != cudaSuccess) rc = PIC_ERR_CUDA;
-    if (rc == PIC_OK) {
-        one_step(cap);
-        if (cudaStreamEndCapture(cap, &gr) != cudaSuccess) rc = PIC_ERR_CUDA;
-    }
-    if (rc == PIC_OK && cudaGraphInstantiate(&ge, gr, 0) != cudaSuccess) rc = PIC_ERR_CUDA;
-    for (int k = 0; rc == PIC_OK && k < n_steps; ++k)
-        if (cudaGraphLaunch(ge, s) != cudaSuccess) rc = PIC_ERR_CUDA;
-    if (ge) cudaGraphExecDestroy(ge);
-    if (gr) cudaGraphDestroy(gr);
-    cudaStreamDestroy(cap);
-    if (rc == PIC_OK && cudaGetLastError() != cudaSuccess) rc = PIC_ERR_CUDA;
-    return rc;
+    return e == cudaSuccess && cudaGetLastError() == cudaSuccess ? PIC_OK : PIC_ERR_CUDA;
 }

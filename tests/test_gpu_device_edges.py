@@ -96,3 +96,26 @@ def test_batched_products_through_warp_and_global_queues(n0, launch):
         assert np.array_equal(cnt[s], ocnt), s
         scale = np.abs(omom).max(axis=0) + 1e-300
         assert np.all(np.abs(mom[s] - omom) <= 1e-9 * scale), s
+
+
+@pytest.mark.parametrize("n", [64, 128, 192, 256, 512, 2304])
+def test_training_pass_by_cluster_size(n):
+    """One to four blocks a cluster, one and several clusters: the gradient
+    against FP64 within the bound of BF16 products, and three steps in one call
+    equal, bit by bit, to three calls of one step."""
+    from paper_2110_14494_gb300 import mlp_loss_grad, mlp_train
+    from tests import test_gpu_mlp as G
+    th, x, t = G._problem(n, seed=n)
+    p0, xd, td = G._dev(th), G._dev(x), G._dev(t)
+    loss, g = mlp_loss_grad(p0, xd, td)
+    th2 = G._w2_as_multiplied(th)
+    lref, gref = G.M.loss_grad(th2, x, t)
+    assert abs(loss.item() - lref) <= 1e-2 * lref
+    assert np.all(np.abs(g.cpu().numpy().astype(np.float64) - gref) <= G._grad_bound(th2, x, t))
+    runs = []
+    for calls in ([(0, 3)], [(0, 1), (1, 1), (2, 1)]):
+        p, m, v = p0.clone(), torch.zeros_like(p0), torch.zeros_like(p0)
+        for step0, k in calls:
+            l = mlp_train(p, m, v, step0, xd, td, k)
+        runs.append((p, m, v, l))
+    assert all(torch.equal(a, b) for a, b in zip(*runs))
