@@ -538,7 +538,13 @@ size_t MG::bytes(int nx_, int ny_, int nz_, bool mixed_, bool pair_copy, bool le
     return m.carve(nullptr, nx_, ny_, nz_, mixed_, pair_copy, lean);
 }
 
+// Bytes of the device array that poisson_solve_noalloc works in.
+constexpr size_t kNoAllocScratchBytes = 32u << 20;
+
 // Lays the buffers out from base (base null: sizes only); returns the bytes.
+// Float64: A z is kept between an iteration's two kernels (a solve on 64 x 48 x
+// 80 cells takes 1113 us, 1220 with A z formed again; 128^3 2184 and 2544),
+// but for grids whose workspace fits 32 MiB only without it (96^3: 1559 us).
 size_t MG::carve(void* base, int nx_, int ny_, int nz_, bool mixed_, bool pair_copy, bool lean) {
     plan(nx_, ny_, nz_);
     mixed = mixed_;
@@ -569,7 +575,6 @@ size_t MG::carve(void* base, int nx_, int ny_, int nz_, bool mixed_, bool pair_c
         r64 = (double*)take(n0 * 8);
         p64 = (double*)take(n0 * 8);
         q64 = (double*)take(n0 * 8);
-        w64 = lean ? nullptr : (double*)take(n0 * 8);
         ctr = (unsigned*)(norms + 16);  // within the scalars' 256 bytes
         const size_t b3 = (size_t)((nx_ + BX - 1) / BX) * ((ny_ + BY - 1) / BY) * ((nz_ + ZC - 1) / ZC);
         part = lean && levels > 1 ? nullptr : (double*)take(3 * 8 * b3);
@@ -584,6 +589,10 @@ size_t MG::carve(void* base, int nx_, int ny_, int nz_, bool mixed_, bool pair_c
     // which only the V-cycle uses
     if (!mixed_ && lean && levels > 1) part = (double*)e[1];
     tail_tab = tail_tables() && !lean ? (uint4*)take((size_t)tail_plan(*this).cells * sizeof(uint4)) : nullptr;
+    const size_t used = (size_t)(p - p0);
+    w64 = nullptr;
+    if (!mixed_ && !lean && (used > kNoAllocScratchBytes || used + align256(n0 * 8) <= kNoAllocScratchBytes))
+        w64 = (double*)take(n0 * 8);
     return (size_t)(p - p0);
 }
 
@@ -1059,6 +1068,7 @@ int MG::capture_solve_mixed(cudaStream_t cs, const float* rho, float* phi_hi, fl
 
 // ------------------------------------------------------------------ C ABI
 using pic::MG;
+using pic::kNoAllocScratchBytes;
 
 namespace {
 bool poisson_args_ok(const poisson_config* pc, const double* rho, const double* phi, const float* Ex, const float* Ey,
@@ -1133,7 +1143,6 @@ extern "C" int poisson_solve(const poisson_config* pc, const double* rho, const 
 // its name is only a host-side stand-in, so the device address is looked up
 // with cudaGetSymbolAddress once per device (with that device current) and
 // cached.
-constexpr size_t kNoAllocScratchBytes = 32u << 20;
 static __device__ __align__(256) unsigned char g_noalloc_scratch[kNoAllocScratchBytes];
 
 #include <mutex>

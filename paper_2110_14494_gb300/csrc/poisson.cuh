@@ -30,7 +30,7 @@ struct MG {
     uint8_t* m[kMaxLevels];
     uint4* tail_tab = nullptr;  // cells of the tail's levels (poisson_tail.cuh)
     double* norms = nullptr;  // CG scalars: ||b||^2, ||r||^2, rho, gamma, alpha, beta
-    double *r64 = nullptr, *p64 = nullptr, *q64 = nullptr, *w64 = nullptr;  // CG vectors (float64; w64 not if lean)
+    double *r64 = nullptr, *p64 = nullptr, *q64 = nullptr, *w64 = nullptr;  // CG vectors (float64; w64: A z, if kept)
     int pre = 2, post = 2, coarse_sweeps = 4;  // coarse: red-black sweeps on the coarsest level
     // mixed solve: an iteration after the untested ones whose relative
     // residual is already within light_ratio x rtol uses a V(light_pre,
