@@ -676,18 +676,29 @@ __global__ void __launch_bounds__(kInfWarps * 32) k_infer(const float* __restric
 }
 
 // ------------------------------------------------------------------ inference on tcgen05
-// Fused forward pass on the fifth-generation tensor cores.  A block of 256
-// threads takes 128 points at a time (thread t: point t % 128, hidden units
-// 64 (t / 128) .. 64 (t / 128) + 63):
-//   1. layer 1 in FP32, tanh in packed BF16, written as the A operand (128
-//      points x 128 units) in shared memory;
+// Fused forward pass on the fifth-generation tensor cores.  A block holds W2
+// once and has four groups of 256 threads; a group takes 128 points at a time:
+//   1. layer 1 in FP32 (thread: eight units of every 16th point, the units'
+//      weights in registers), tanh in packed BF16, written as the A operand
+//      (128 points x 128 units) in shared memory;
 //   2. one thread issues eight 128 x 128 x 16 MMAs (A: h1, B: W2 resident in
 //      shared memory) into a 128-column FP32 accumulator in tensor memory;
-//   3. the accumulator rows are read back (row = point = TMEM lane), bias and
-//      tanh applied, and h2 written over the A operand;
+//   3. the accumulator rows are read back (row = point = TMEM lane; thread t:
+//      point t % 128, units 64 (t / 128) on), bias and tanh applied, and h2
+//      written over the A operand;
 //   4. eight 128 x 16 x 16 MMAs against W3 (padded to 16 outputs) into the
 //      first 16 accumulator columns; the first half of the threads read the
 //      six outputs back, add b3 and store.
+//
+// What bounds it: the tanh unit (16 clocks of a scheduler for a packed pair a
+// lane, measured: 2048 of a tile's 2530 clocks on a multiprocessor).  A group
+// alone would leave it idle for two thirds of a tile (both products and their
+// waits), so the four run independently of one another, each with its own
+// named barrier, A operand and 128 of the 512 tensor-memory columns.  16.8
+// million points: three blocks of one group an SM, a thread's weights loaded
+// as broadcasts (63 % of the shared-memory pipe) 1323 us; weights by unit 1286;
+// four groups in a block 1156.  Layer 1 of the next tile during the waits
+// (held in registers, which then spill): 1188.
 // Operands use the canonical K-major layout without swizzle: core matrices
 // of 8 rows x 16 bytes stored contiguously, the next core matrix along K at
 // +128 bytes, the next 8-row group at +2048 bytes (the same strides for the
@@ -695,19 +706,21 @@ __global__ void __launch_bounds__(kInfWarps * 32) k_infer(const float* __restric
 // bytes, inside its 32 KB (4 KB) tile.  Waits on the MMA completion barrier are
 // bounded; on expiry the block writes NaN outputs, records the error and
 // leaves, releasing its tensor memory.
-constexpr int kTcThreads = 256, kTcRows = 128;
+constexpr int kTcGroups = 4, kTcGroup = 256, kTcThreads = kTcGroups * kTcGroup, kTcRows = 128;
 constexpr uint32_t kTile = kTcRows * NH * 2;   // one 128 x 128 BF16 operand: 32 KB
 constexpr uint32_t kLbo = 128, kSbo = 2048;    // core-matrix strides (bytes) along K and along M/N
 constexpr uint32_t kB2Bytes = 16 * NH * 2;     // W3 padded to 16 rows: 4 KB
 
 struct TcSmem {
     alignas(1024) unsigned char w2[kTile];   // B of layer 2: row o (output unit), K = input unit
-    alignas(1024) unsigned char a[kTile];    // A: row = point, K = unit (h1, then h2)
+    alignas(1024) unsigned char a[kTcGroups][kTile];  // A of a group: row = point, K = unit (h1, then h2)
     alignas(1024) unsigned char w3[kB2Bytes];
-    float w1[NH * NI], b1[NH], b2[NH], b3[NO];
-    alignas(8) unsigned long long bar;
+    alignas(16) float w1a[NH], w1b[NH], b1[NH], b2[NH];  // w1a, w1b: weights of the two inputs
+    float2 xs[kTcGroups][2][kTcRows];                    // inputs of this tile and the next
+    float b3[NO];
+    alignas(8) unsigned long long bar[kTcGroups];
     uint32_t tmem;
-    int abort;
+    int abort[kTcGroups];
 };
 
 // byte offset of element (row r, k) in a K-major no-swizzle operand
@@ -770,14 +783,39 @@ __device__ __forceinline__ void tmem_ld8(uint32_t taddr, float (&v)[8]) {
     for (int q = 0; q < 8; ++q) v[q] = __uint_as_float(r[q]);
 }
 
-// tanh of two floats as packed BF16 (hardware approximation)
-__device__ __forceinline__ uint32_t tanh_bf16x2(float lo, float hi) {
+// Pairs of floats in a 64-bit register, and the packed operations on them
+// (each half rounded as the scalar operation).
+__device__ __forceinline__ uint64_t pair_of(float lo, float hi) {
+    uint64_t v;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(v) : "f"(lo), "f"(hi));
+    return v;
+}
+__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
+    uint64_t v;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(v) : "l"(a), "l"(b), "l"(c));
+    return v;
+}
+__device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
+    uint64_t v;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(v) : "l"(a), "l"(b));
+    return v;
+}
+__device__ __forceinline__ void ld_pairs(const float* p, uint64_t& a, uint64_t& b) {
+    const ulonglong2 v = *reinterpret_cast<const ulonglong2*>(p);
+    a = v.x;
+    b = v.y;
+}
+
+// tanh of a pair as packed BF16 (hardware approximation)
+__device__ __forceinline__ uint32_t tanh_bf16x2(uint64_t v) {
+    float lo, hi;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
     uint32_t in = pack_bf16(lo, hi), out;
     asm("tanh.approx.bf16x2 %0, %1;" : "=r"(out) : "r"(in));
     return out;
 }
 
-__global__ void __launch_bounds__(kTcThreads) k_infer_tc(const float* __restrict__ th,
+__global__ void __launch_bounds__(kTcThreads, 1) k_infer_tc(const float* __restrict__ th,
                                                          const __nv_bfloat16* __restrict__ w2b,
                                                          const float* __restrict__ x, float* __restrict__ y,
                                                          long long n, int* __restrict__ err) {
@@ -785,7 +823,7 @@ __global__ void __launch_bounds__(kTcThreads) k_infer_tc(const float* __restrict
     // align the operand tiles to 1024 bytes
     TcSmem& S = *reinterpret_cast<TcSmem*>(tc_raw + ((1024 - (smem_u32(tc_raw) & 1023)) & 1023));
     const int tid = threadIdx.x, warp = tid >> 5;
-    const int row = tid & (kTcRows - 1), half = tid >> 7;
+    const int group = tid / kTcGroup, gt = tid % kTcGroup, row = gt & (kTcRows - 1), half = gt >> 7;
     // operands and parameters
     for (int k = tid; k < NH * NH; k += kTcThreads) {
         const int o = k / NH, i = k % NH;
@@ -796,21 +834,25 @@ __global__ void __launch_bounds__(kTcThreads) k_infer_tc(const float* __restrict
         *reinterpret_cast<__nv_bfloat16*>(S.w3 + kmajor_off(o, i)) =
             __float2bfloat16_rn(o < NO ? th[OFF_W3 + o * NH + i] : 0.0f);
     }
-    for (int k = tid; k < NH * NI; k += kTcThreads) S.w1[k] = th[OFF_W1 + k];
     for (int k = tid; k < NH; k += kTcThreads) {
+        S.w1a[k] = th[OFF_W1 + k * NI];
+        S.w1b[k] = th[OFF_W1 + k * NI + 1];
         S.b1[k] = th[OFF_B1 + k];
         S.b2[k] = th[OFF_B2 + k];
     }
     if (tid < NO) S.b3[tid] = th[OFF_B3 + tid];
-    const uint32_t bar = smem_u32(&S.bar);
-    if (tid == 0) {
-        S.abort = 0;
+    const auto x_of = [&](long long p) { return p < n ? make_float2(x[p * NI], x[p * NI + 1]) : make_float2(0.0f, 0.0f); };
+    const long long first = blockIdx.x + (long long)gridDim.x * group, stride = (long long)gridDim.x * kTcGroups;
+    if (half == 0) S.xs[group][0][row] = x_of(first * kTcRows + row);
+    const uint32_t bar = smem_u32(&S.bar[group]);
+    if (gt == 0) {
+        S.abort[group] = 0;
         asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(bar) : "memory");
         asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
     }
     if (warp == 0) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(smem_u32(&S.tmem)),
-                     "r"(128)
+                     "r"(128 * kTcGroups)
                      : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n" ::: "memory");
     }
@@ -818,45 +860,46 @@ __global__ void __launch_bounds__(kTcThreads) k_infer_tc(const float* __restrict
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    const uint32_t tmem = S.tmem;
+    const uint32_t tmem = S.tmem + 128u * group;
     const uint32_t lane_base = (uint32_t)((warp & 3) * 32) << 16;
-    const uint32_t a_addr = smem_u32(S.a), w2_addr = smem_u32(S.w2), w3_addr = smem_u32(S.w3);
+    const uint32_t a_addr = smem_u32(S.a[group]), w2_addr = smem_u32(S.w2), w3_addr = smem_u32(S.w3);
     uint32_t parity = 0;
     const long long n_tiles = (n + kTcRows - 1) / kTcRows;
-    // this thread's point of the next tile is loaded one tile ahead
-    float xn0 = 0.0f, xn1 = 0.0f;
-    {
-        const long long p0 = (long long)blockIdx.x * kTcRows + row;
-        if (p0 < n) { xn0 = x[p0 * NI]; xn1 = x[p0 * NI + 1]; }
-    }
-    for (long long tile = blockIdx.x; tile < n_tiles; tile += gridDim.x) {
+    // layer 1: units u1 .. u1 + 7 of rows r1, r1 + 16, ...
+    const int lane = tid & 31, u1 = ((lane >> 3) + 4 * (warp & 3)) * 8, r1 = (lane & 7) + 8 * ((warp >> 2) & 1);
+    unsigned char* const A = S.a[group];
+    const auto sync = [&]() { pic::bar_named(1 + group, kTcGroup); };
+    int buf = 0;
+    for (long long tile = first; tile < n_tiles; tile += stride, buf ^= 1) {
         const long long p = tile * kTcRows + row;
         const bool valid = p < n;
-        const float x0 = xn0, x1 = xn1;
+        // the next tile's inputs, loaded one tile ahead
+        float2 xn = make_float2(0.0f, 0.0f);
+        if (half == 0) xn = x_of((tile + stride) * kTcRows + row);
+        // 1. layer 1 into the A operand
         {
-            const long long pn = (tile + gridDim.x) * kTcRows + row;
-            if (pn < n) { xn0 = x[pn * NI]; xn1 = x[pn * NI + 1]; }
-        }
-        // 1. layer 1 into the A operand (this thread: 64 units of its point)
-        {
+            uint64_t wa[4], wb[4], bb[4];
 #pragma unroll
-            for (int c = 0; c < 8; ++c) {
-                const int u0 = half * 64 + c * 8;
+            for (int e = 0; e < 4; e += 2) {
+                ld_pairs(&S.w1a[u1 + 2 * e], wa[e], wa[e + 1]);
+                ld_pairs(&S.w1b[u1 + 2 * e], wb[e], wb[e + 1]);
+                ld_pairs(&S.b1[u1 + 2 * e], bb[e], bb[e + 1]);
+            }
+#pragma unroll
+            for (int j = 0; j < kTcRows / 16; ++j) {
+                const float2 xr = S.xs[group][buf][r1 + 16 * j];
+                const uint64_t x0 = pair_of(xr.x, xr.x), x1 = pair_of(xr.y, xr.y);
                 uint32_t w[4];
 #pragma unroll
-                for (int e = 0; e < 4; ++e) {
-                    const int u = u0 + 2 * e;
-                    const float z0 = fmaf(S.w1[u * NI + 1], x1, fmaf(S.w1[u * NI], x0, S.b1[u]));
-                    const float z1 = fmaf(S.w1[(u + 1) * NI + 1], x1, fmaf(S.w1[(u + 1) * NI], x0, S.b1[u + 1]));
-                    w[e] = tanh_bf16x2(z0, z1);
-                }
-                *reinterpret_cast<uint4*>(S.a + kmajor_off(row, u0)) = make_uint4(w[0], w[1], w[2], w[3]);
+                for (int e = 0; e < 4; ++e) w[e] = tanh_bf16x2(fma2(wb[e], x1, fma2(wa[e], x0, bb[e])));
+                *reinterpret_cast<uint4*>(A + kmajor_off(r1 + 16 * j, u1)) = make_uint4(w[0], w[1], w[2], w[3]);
             }
         }
+        if (half == 0) S.xs[group][buf ^ 1][row] = xn;
         fence_async_smem();
-        __syncthreads();
+        sync();
         // 2. h1 W2^T into the accumulator
-        if (tid == 0) {
+        if (gt == 0) {
             tc_fence_after();
 #pragma unroll
             for (int kk = 0; kk < NH / 16; ++kk)
@@ -864,11 +907,11 @@ __global__ void __launch_bounds__(kTcThreads) k_infer_tc(const float* __restrict
                        idesc_bf16(128, 128), kk > 0 ? 1u : 0u);
             tc_commit(bar);
         }
-        if (!bar_wait(bar, parity)) S.abort = 1;
+        if (!bar_wait(bar, parity)) S.abort[group] = 1;
         parity ^= 1;
         tc_fence_after();
-        __syncthreads();
-        if (S.abort) break;
+        sync();
+        if (S.abort[group]) break;
         // 3. bias, tanh, h2 over the A operand
 #pragma unroll
         for (int ch = 0; ch < 2; ++ch) {
@@ -879,18 +922,21 @@ __global__ void __launch_bounds__(kTcThreads) k_infer_tc(const float* __restrict
             for (int c = 0; c < 4; ++c) {
                 uint32_t w[4];
 #pragma unroll
-                for (int e = 0; e < 4; ++e) {
+                for (int e = 0; e < 4; e += 2) {
                     const int q = c * 8 + 2 * e;
-                    w[e] = tanh_bf16x2(acc[q] + S.b2[c0 + q], acc[q + 1] + S.b2[c0 + q + 1]);
+                    uint64_t b0, b1;
+                    ld_pairs(&S.b2[c0 + q], b0, b1);
+                    w[e] = tanh_bf16x2(add2(pair_of(acc[q], acc[q + 1]), b0));
+                    w[e + 1] = tanh_bf16x2(add2(pair_of(acc[q + 2], acc[q + 3]), b1));
                 }
-                *reinterpret_cast<uint4*>(S.a + kmajor_off(row, c0 + c * 8)) = make_uint4(w[0], w[1], w[2], w[3]);
+                *reinterpret_cast<uint4*>(A + kmajor_off(row, c0 + c * 8)) = make_uint4(w[0], w[1], w[2], w[3]);
             }
         }
         tc_fence_before();
         fence_async_smem();
-        __syncthreads();
+        sync();
         // 4. h2 W3^T (16 padded outputs) into accumulator columns 0..15
-        if (tid == 0) {
+        if (gt == 0) {
             tc_fence_after();
 #pragma unroll
             for (int kk = 0; kk < NH / 16; ++kk)
@@ -898,11 +944,11 @@ __global__ void __launch_bounds__(kTcThreads) k_infer_tc(const float* __restrict
                        idesc_bf16(128, 16), kk > 0 ? 1u : 0u);
             tc_commit(bar);
         }
-        if (!bar_wait(bar, parity)) S.abort = 1;
+        if (!bar_wait(bar, parity)) S.abort[group] = 1;
         parity ^= 1;
         tc_fence_after();
-        __syncthreads();
-        if (S.abort) break;
+        sync();
+        if (S.abort[group]) break;
         if (half == 0) {
             float o8[8];
             tmem_ld8(tmem + lane_base, o8);
@@ -911,12 +957,12 @@ __global__ void __launch_bounds__(kTcThreads) k_infer_tc(const float* __restrict
                 for (int o = 0; o < NO; ++o) y[p * NO + o] = o8[o] + S.b3[o];
         }
         tc_fence_before();
-        __syncthreads();
+        sync();
     }
-    if (S.abort) {
+    if (S.abort[group]) {
         // a wait expired: mark this block's remaining outputs and report
-        if (tid == 0) atomicOr(err, 1);
-        for (long long tile = blockIdx.x; tile < n_tiles; tile += gridDim.x) {
+        if (gt == 0) atomicOr(err, 1);
+        for (long long tile = first; tile < n_tiles; tile += stride) {
             const long long p = tile * kTcRows + row;
             if (half == 0 && p < n)
                 for (int o = 0; o < NO; ++o) y[p * NO + o] = __int_as_float(0x7fc00000);
@@ -926,7 +972,7 @@ __global__ void __launch_bounds__(kTcThreads) k_infer_tc(const float* __restrict
     __syncthreads();
     if (warp == 0) {
         tc_fence_after();
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem), "r"(128) : "memory");
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(S.tmem), "r"(128 * kTcGroups) : "memory");
     }
 }
 
@@ -1062,16 +1108,8 @@ extern "C" int mlp_forward_variant(const float* params, const float* x, float* y
         const int smem = (int)sizeof(TcSmem) + 1024;
         if (cudaFuncSetAttribute(k_infer_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess)
             return PIC_ERR_CUDA;
-        // blocks per SM from the shared memory each needs (plus the 1 KB the
-        // runtime reserves per block); each block also holds 128 of the 512
-        // tensor-memory columns, so at most 4
-        int smem_sm = 0;
-        cudaDeviceGetAttribute(&smem_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev);
-        per_sm = smem_sm / (smem + 1024);
-        per_sm = per_sm < 1 ? 1 : (per_sm > 4 ? 4 : per_sm);
-        const long long tiles = (n + kTcRows - 1) / kTcRows;
-        long long blocks = (long long)sms * per_sm;
-        if (blocks > tiles) blocks = tiles;
+        // one block an SM (shared memory, 512 tensor-memory columns); few tiles are spread over the SMs
+        const long long tiles = (n + kTcRows - 1) / kTcRows, blocks = tiles < sms ? tiles : sms;
         k_infer_tc<<<(unsigned)blocks, kTcThreads, smem, s>>>(params, w.w2b, x, y, n, w.err);
     } else {
         const int smem = (int)sizeof(InfSmem);

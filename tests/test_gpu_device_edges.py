@@ -119,3 +119,15 @@ def test_training_pass_by_cluster_size(n):
             l = mlp_train(p, m, v, step0, xd, td, k)
         runs.append((p, m, v, l))
     assert all(torch.equal(a, b) for a, b in zip(*runs))
+
+
+@pytest.mark.parametrize("n", [1, 129, 128 * 152 + 1, 4 * 128 * 152 - 1, 4 * 128 * 152 + 129])
+def test_queries_do_not_depend_on_their_tile(n):
+    """Ragged tiles, idle groups of a block, one and two tiles a group: each
+    point's outputs are, bit by bit, those of the same point in calls of 1000."""
+    from paper_2110_14494_gb300 import mlp_forward
+    from tests import test_gpu_mlp as G
+    th, x, _ = G._problem(n, seed=5)
+    p, xd = G._dev(th), G._dev(x)
+    y = mlp_forward(p, xd)
+    assert torch.equal(y, torch.cat([mlp_forward(p, xd[k:k + 1000].contiguous()) for k in range(0, n, 1000)]))
