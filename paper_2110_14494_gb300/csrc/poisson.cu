@@ -56,104 +56,199 @@ __device__ __forceinline__ float nb_sum_e(const float* __restrict__ e, int i, in
 
 __device__ __forceinline__ float inv_diag(float diag) { return diag == 6.0f ? (1.0f / 6.0f) : 1.0f / diag; }
 
-// One colour of red-black Gauss-Seidel for A e = g (masked cells stay 0).
-// Thread (ii, j) handles ZS planes k0 .. k0 + ZS - 1, at each the cell
-// i = 2 ii + ((j + k + colour) & 1).  All loads of the ZS cells (the other
-// colour, not written by this launch) are issued before the first store.
-// Large levels take ZS = 4 (fewer, longer threads); small ones ZS = 1 (more
-// parallelism).  With omega != 1 the update is over-relaxed:
-// e + omega ((g + s) / diag - e).
-template <int ZS>
+// One colour of red-black Gauss-Seidel for A e = g (masked cells stay 0), on a
+// small level: thread (ii, j, k) updates the cell i = 2 ii + ((j + k + colour)
+// & 1).
 __global__ void __launch_bounds__(BX * BY) k_smooth(float* __restrict__ e, const float* __restrict__ g,
-                                                    const uint8_t* __restrict__ mask, int nx, int ny, int nz,
-                                                    int color, float omega) {
+                                                    const uint8_t* __restrict__ mask, int nx, int ny, int nz, int color) {
     pdl_wait();
-    const int j = blockIdx.y * BY + threadIdx.y, k0 = blockIdx.z * ZS, ii = blockIdx.x * BX + threadIdx.x;
-    if (j >= ny) return;
-    const bool relax = omega != 1.0f;
-    float s[ZS], gv[ZS], dg[ZS], eo[ZS];
+    const int j = blockIdx.y * BY + threadIdx.y, k = blockIdx.z, ii = blockIdx.x * BX + threadIdx.x;
+    const int i = 2 * ii + ((j + k + color) & 1);
+    if (j >= ny || i >= nx) return;
+    const int c = lin(i, j, k, nx, ny);
+    float dg;
+    const float s = nb_sum_e(e, i, j, k, nx, ny, nz, c, dg), gv = g[c];
+    if (!mask[c]) e[c] = (gv + s) * inv_diag(dg);
+}
+
+// The sweeps of large levels (nx even: every level with a coarser one) work on
+// x pairs: a cell's six neighbours of the other colour are the other cell of
+// its own pair, the other cell of one adjacent pair and those of the pairs of
+// the same index in the rows and planes around.  Thread (ii, row) takes ZS
+// planes of its pair with all loads issued first; rows trade values through
+// shared memory (two rows around the block load and trade only), x neighbours
+// come from the adjacent lane, and the warp's end lanes load theirs.
+//
+// What bounds them: memory on grids beyond the L2, and within it the issue
+// rate: with a thread for each cell that loads its six neighbours, its limits
+// and its diagonal 115 instructions a cell.  So which cell of a pair is which
+// is known at compile time (P: the row's parity), limits are only looked at in
+// the first and last slab of planes, and the reciprocal diagonals are formed
+// once a thread.  A V-cycle's half-sweeps (large levels) and first sweeps (all
+// levels), before and now: 128^3 cells 36.5 and 28.7 us, 25.5 and 13.0; 3.4e7
+// cells 458 and 375, 258 and 113.
+constexpr int SY = 8;  // rows of a block
+struct PairTile {
+    int ii, j, k0, c0, pl;  // pair, row, first plane; index of the pair in plane 0; cells of a plane
+    bool in, own;           // the pair exists; it belongs to the block
+    float inv[2], inv_x;    // reciprocal diagonals of the two cells and of a neighbour in x, interior planes
+    float inv1[2], inv1_x;  // in the planes at the plates
+};
+__device__ __forceinline__ PairTile pair_tile(int nx, int ny, int zs) {
+    PairTile t;
+    t.ii = blockIdx.x * BX + threadIdx.x;
+    t.j = (int)(blockIdx.y * SY + threadIdx.y) - 1;
+    t.k0 = blockIdx.z * zs;
+    t.pl = nx * ny;
+    t.in = t.j >= 0 && t.j < ny && 2 * t.ii < nx;
+    t.own = t.in && threadIdx.y >= 1 && threadIdx.y <= SY;
+    t.c0 = t.in ? lin(2 * t.ii, t.j, 0, nx, ny) : 0;
+    const float d = 6.0f - (float)((t.j == 0) + (t.j == ny - 1));
+    const float d0 = t.ii == 0 ? d - 1.0f : d, d1 = 2 * t.ii + 2 >= nx ? d - 1.0f : d;
+    t.inv[0] = __frcp_rn(d0);
+    t.inv[1] = __frcp_rn(d1);
+    t.inv_x = __frcp_rn(d);
+    t.inv1[0] = __frcp_rn(d0 + 1.0f);
+    t.inv1[1] = __frcp_rn(d1 + 1.0f);
+    t.inv1_x = __frcp_rn(d + 1.0f);
+    return t;
+}
+// Neighbour sum of a cell (par: which of its pair) whose other-colour values
+// are o, at planes around om and op, in the rows around ym and yp; xe: beyond
+// the warp's end.
+template <int PAR> __device__ __forceinline__ float pair_sum(float o, float xe, float ym, float yp, float om, float op) {
+    const int lane = threadIdx.x;
+    const float nb = PAR ? __shfl_down_sync(kFull, o, 1) : __shfl_up_sync(kFull, o, 1);
+    const float x = lane == (PAR ? BX - 1 : 0) ? xe : nb;
+    return ((((PAR ? o + x : x + o) + ym) + yp) + om) + op;
+}
+
+// One colour of red-black Gauss-Seidel.  P: which cell of the pair is updated
+// in plane k0; IN: all planes and those around lie inside the grid.
+template <int ZS, int P, bool IN>
+__device__ __forceinline__ void smooth_pair(float* __restrict__ e, const float* __restrict__ g,
+                                            const uint8_t* __restrict__ mask, int nx, int nz, const PairTile& t,
+                                            float (*so)[SY + 2][BX]) {
+    const int lane = threadIdx.x, ty = threadIdx.y;
+    float o[ZS + 2], xe[ZS], gv[ZS];  // the pair's other cell, the outer x neighbour
     uint8_t mv[ZS];
-    int cc[ZS];
+    const int q0 = t.c0 + (t.k0 - 1) * t.pl;
+    const bool edge_x = t.own && (lane == 0 ? t.ii > 0 : (lane == BX - 1 && 2 * t.ii + 2 < nx));
+#pragma unroll
+    for (int d = 0; d < ZS + 2; ++d) {
+        const int par = (P + d + 1) & 1, k = t.k0 - 1 + d;
+        // rows around the block need no planes around
+        const bool ok = ((d == 0 || d == ZS + 1) ? t.own : t.in) && (IN || (k >= 0 && k < nz));
+        o[d] = ok ? e[q0 + d * t.pl + (1 - par)] : 0.0f;
+    }
 #pragma unroll
     for (int d = 0; d < ZS; ++d) {
-        const int k = k0 + d;
-        const int i = 2 * ii + ((j + k + color) & 1);
-        const bool ok = i < nx && k < nz;
-        cc[d] = ok ? lin(i, j, k, nx, ny) : -1;
-        s[d] = ok ? nb_sum_e(e, i, j, k, nx, ny, nz, cc[d], dg[d]) : 0.0f;
-        gv[d] = ok ? g[cc[d]] : 0.0f;
-        mv[d] = ok ? mask[cc[d]] : 1;
-        eo[d] = ok && relax ? e[cc[d]] : 0.0f;
+        const int par = (P + d) & 1, c = q0 + (d + 1) * t.pl;
+        const bool ok = t.own && (IN || t.k0 + d < nz);
+        gv[d] = ok ? g[c + par] : 0.0f;
+        mv[d] = ok ? mask[c + par] : 1;
+        xe[d] = edge_x && ok && lane == (par ? BX - 1 : 0) ? e[par ? c + 2 : c - 1] : 0.0f;
+        so[d][ty][lane] = o[d + 1];
+    }
+    bar_named(1, BX * (SY + 2));  // rows of either parity meet here
+    if (ty < 1 || ty > SY) return;
+#pragma unroll
+    for (int d = 0; d < ZS; ++d) {
+        const int par = (P + d) & 1, k = t.k0 + d;
+        const float ym = so[d][ty - 1][lane], yp = so[d][ty + 1][lane];
+        const float s = par ? pair_sum<1>(o[d + 1], xe[d], ym, yp, o[d], o[d + 2])
+                            : pair_sum<0>(o[d + 1], xe[d], ym, yp, o[d], o[d + 2]);
+        const float inv = IN || (k > 0 && k < nz - 1) ? t.inv[par] : t.inv1[par];
+        if (!mv[d]) e[q0 + (d + 1) * t.pl + par] = (gv[d] + s) * inv;
+    }
+}
+template <int ZS>
+__global__ void __launch_bounds__(BX * (SY + 2)) k_smooth_pair(float* __restrict__ e, const float* __restrict__ g,
+                                                               const uint8_t* __restrict__ mask, int nx, int ny, int nz,
+                                                               int color) {
+    __shared__ float so[ZS][SY + 2][BX];
+    const PairTile t = pair_tile(nx, ny, ZS);
+    pdl_wait();
+    const bool in = t.k0 > 0 && t.k0 + ZS < nz;
+    if ((t.j + t.k0 + color) & 1) {
+        if (in) smooth_pair<ZS, 1, true>(e, g, mask, nx, nz, t, so);
+        else smooth_pair<ZS, 1, false>(e, g, mask, nx, nz, t, so);
+    } else {
+        if (in) smooth_pair<ZS, 0, true>(e, g, mask, nx, nz, t, so);
+        else smooth_pair<ZS, 0, false>(e, g, mask, nx, nz, t, so);
+    }
+}
+
+// The first full red-black sweep of a V-cycle level, from e = 0, in one pass
+// that needs no e: colour 0 cells get g * inv_diag (their neighbours are still
+// 0), colour 1 cells get (g + sum of those colour-0 values at their neighbours)
+// * inv_diag.  The same operations in the same order as a zero fill followed by
+// two half-sweeps, so the values are identical.  Electrode cells get 0.
+// P: which cell of the pair is colour 0 in plane k0; IN: as above, and the
+// planes around are not at a plate.
+template <int ZS, int P, bool IN>
+__device__ __forceinline__ void sweep_first_pair(float* __restrict__ e, const float* __restrict__ g,
+                                                 const uint8_t* __restrict__ mask, int nx, int nz, const PairTile& t,
+                                                 float (*sr)[SY + 2][BX]) {
+    const int lane = threadIdx.x, ty = threadIdx.y;
+    float2 gp[ZS + 2];
+    uchar2 mp[ZS + 2];
+    float r[ZS + 2], gx[ZS];  // the pair's colour-0 value; g of the outer x neighbour
+    uint8_t mx[ZS];
+    const int q0 = t.c0 + (t.k0 - 1) * t.pl;
+    const bool edge_x = t.own && (lane == 0 ? t.ii > 0 : (lane == BX - 1 && 2 * t.ii + 2 < nx));
+#pragma unroll
+    for (int d = 0; d < ZS + 2; ++d) {
+        const int k = t.k0 - 1 + d;
+        const bool ok = ((d == 0 || d == ZS + 1) ? t.own : t.in) && (IN || (k >= 0 && k < nz));
+        gp[d] = ok ? *reinterpret_cast<const float2*>(g + q0 + d * t.pl) : make_float2(0.0f, 0.0f);
+        mp[d] = ok ? *reinterpret_cast<const uchar2*>(mask + q0 + d * t.pl) : make_uchar2(1, 1);
     }
 #pragma unroll
-    for (int d = 0; d < ZS; ++d)
-        if (cc[d] >= 0 && !mv[d]) {
-            const float v = (gv[d] + s[d]) * inv_diag(dg[d]);
-            e[cc[d]] = relax ? fmaf(omega, v - eo[d], eo[d]) : v;
-        }
+    for (int d = 0; d < ZS; ++d) {
+        // colour 1 lies at 2 ii + 1 - par, its outer x neighbour at 2 ii - 1 or 2 ii + 2
+        const int par = (P + d) & 1, c = q0 + (d + 1) * t.pl + (par ? -1 : 2);
+        const bool ok = edge_x && lane == (par ? 0 : BX - 1) && (IN || t.k0 + d < nz);
+        gx[d] = ok ? g[c] : 0.0f;
+        mx[d] = ok ? mask[c] : 1;
+    }
+#pragma unroll
+    for (int d = 0; d < ZS + 2; ++d) {
+        const int par = (P + d + 1) & 1, k = t.k0 - 1 + d;
+        const float inv = IN || (k > 0 && k < nz - 1) ? t.inv[par] : t.inv1[par];
+        r[d] = (par ? mp[d].y : mp[d].x) ? 0.0f : ((par ? gp[d].y : gp[d].x) + 0.0f) * inv;
+        if (d >= 1 && d <= ZS) sr[d - 1][ty][lane] = r[d];
+    }
+    bar_named(1, BX * (SY + 2));  // rows of either parity meet here
+    if (ty < 1 || ty > SY) return;
+#pragma unroll
+    for (int d = 0; d < ZS; ++d) {
+        const int par = (P + d) & 1, k = t.k0 + d;
+        const bool inner = IN || (k > 0 && k < nz - 1);
+        const float xe = mx[d] ? 0.0f : (gx[d] + 0.0f) * (inner ? t.inv_x : t.inv1_x);
+        const float ym = sr[d][ty - 1][lane], yp = sr[d][ty + 1][lane];
+        const float s = par ? pair_sum<0>(r[d + 1], xe, ym, yp, r[d], r[d + 2])
+                            : pair_sum<1>(r[d + 1], xe, ym, yp, r[d], r[d + 2]);
+        const float v = ((par ? gp[d + 1].x : gp[d + 1].y) + s) * (inner ? t.inv[1 - par] : t.inv1[1 - par]);
+        const float b = (par ? mp[d + 1].x : mp[d + 1].y) ? 0.0f : v;
+        if (t.own && (IN || k < nz))
+            *reinterpret_cast<float2*>(e + q0 + (d + 1) * t.pl) = par ? make_float2(b, r[d + 1]) : make_float2(r[d + 1], b);
+    }
 }
-
-__device__ __forceinline__ float diag_at(int i, int j, int k, int nx, int ny, int nz) {
-    return 6.0f - (float)((i == 0) + (i == nx - 1) + (j == 0) + (j == ny - 1)) + (float)((k == 0) + (k == nz - 1));
-}
-
-// The first full red-black sweep of a V-cycle level, from e = 0, in one
-// pass that needs no e: colour 0 cells get g * inv_diag (their neighbours
-// are still 0), colour 1 cells get (g + sum of those colour-0 values at
-// their neighbours) * inv_diag.  The same operations in the same order as a
-// zero fill followed by two smooth_half launches, so the values are
-// identical.  Thread (ii, j, k) takes the x pair (2 ii, 2 ii + 1) of row
-// (j, k); the colour-0 value of the adjacent pair comes from the next or
-// previous lane.  Electrode cells get 0.  With omega != 1 both values are
-// scaled by omega (over-relaxation from e = 0).
-__device__ __forceinline__ float first_red(const float* __restrict__ g, const uint8_t* __restrict__ mask, int i, int j,
-                                           int k, int nx, int ny, int nz, float omega) {
-    const int c = lin(i, j, k, nx, ny);
-    const float zero = 0.0f;
-    const float s = ((((zero + zero) + zero) + zero) + zero) + zero;
-    const float v = (g[c] + s) * inv_diag(diag_at(i, j, k, nx, ny, nz));
-    return mask[c] ? 0.0f : (omega != 1.0f ? omega * v : v);
-}
-__global__ void __launch_bounds__(BX * BY) k_sweep_first(float* __restrict__ e, const float* __restrict__ g,
-                                                         const uint8_t* __restrict__ mask, int nx, int ny, int nz,
-                                                         float omega) {
+template <int ZS>
+__global__ void __launch_bounds__(BX * (SY + 2)) k_sweep_first(float* __restrict__ e, const float* __restrict__ g,
+                                                               const uint8_t* __restrict__ mask, int nx, int ny, int nz) {
+    __shared__ float sr[ZS][SY + 2][BX];
+    const PairTile t = pair_tile(nx, ny, ZS);
     pdl_wait();
-    const int ii = blockIdx.x * BX + threadIdx.x, j = blockIdx.y * BY + threadIdx.y, k = blockIdx.z;
-    const int lane = threadIdx.x;
-    const int par = (j + k) & 1;       // x offset of the colour-0 cell in the pair
-    const int i0 = 2 * ii + par;       // colour 0
-    const int i1 = 2 * ii + (1 - par); // colour 1
-    const bool in = j < ny && 2 * ii < nx;
-    const bool ok0 = in && i0 < nx, ok1 = in && i1 < nx;
-    // colour-0 value of this pair, shared with the neighbouring lanes
-    const float r0 = ok0 ? first_red(g, mask, i0, j, k, nx, ny, nz, omega) : 0.0f;
-    // the colour-1 cell's x neighbours: one is this pair's colour-0 cell, the
-    // other the adjacent pair's (previous pair when i1 < i0, else next)
-    const float prev = __shfl_up_sync(kFull, r0, 1), next = __shfl_down_sync(kFull, r0, 1);
-    if (!in) return;
-    if (ok0) e[lin(i0, j, k, nx, ny)] = r0;
-    if (!ok1) return;
-    const int c1 = lin(i1, j, k, nx, ny);
-    if (mask[c1]) {
-        e[c1] = 0.0f;
-        return;
+    const bool in = t.k0 > 1 && t.k0 + ZS < nz - 1;
+    if ((t.j + t.k0) & 1) {
+        if (in) sweep_first_pair<ZS, 1, true>(e, g, mask, nx, nz, t, sr);
+        else sweep_first_pair<ZS, 1, false>(e, g, mask, nx, nz, t, sr);
+    } else {
+        if (in) sweep_first_pair<ZS, 0, true>(e, g, mask, nx, nz, t, sr);
+        else sweep_first_pair<ZS, 0, false>(e, g, mask, nx, nz, t, sr);
     }
-    // x neighbours of i1: i1 - 1 and i1 + 1
-    float xm, xp;
-    if (par == 1) {  // i1 = 2 ii: left neighbour in the previous pair, right one is i0
-        xm = i1 > 0 ? (lane > 0 ? prev : first_red(g, mask, i1 - 1, j, k, nx, ny, nz, omega)) : 0.0f;
-        xp = i0 < nx ? r0 : 0.0f;
-    } else {         // i1 = 2 ii + 1: left neighbour is i0, right one in the next pair
-        xm = r0;
-        xp = i1 < nx - 1 ? (lane < BX - 1 ? next : first_red(g, mask, i1 + 1, j, k, nx, ny, nz, omega)) : 0.0f;
-    }
-    const float ym = j > 0 ? first_red(g, mask, i1, j - 1, k, nx, ny, nz, omega) : 0.0f;
-    const float yp = j < ny - 1 ? first_red(g, mask, i1, j + 1, k, nx, ny, nz, omega) : 0.0f;
-    const float zm = k > 0 ? first_red(g, mask, i1, j, k - 1, nx, ny, nz, omega) : 0.0f;
-    const float zp = k < nz - 1 ? first_red(g, mask, i1, j, k + 1, nx, ny, nz, omega) : 0.0f;
-    const float s = ((((xm + xp) + ym) + yp) + zm) + zp;
-    const float v = (g[c1] + s) * inv_diag(diag_at(i1, j, k, nx, ny, nz));
-    e[c1] = omega != 1.0f ? omega * v : v;
 }
 
 // Coarse right-hand side: g_c = 4 * mean of the 8 fine residuals g - A e
@@ -276,7 +371,6 @@ struct TailLevels {
     const uint8_t* m[12];    // global masks
     int nx[12], ny[12], nz[12], off[12];  // shared-memory offsets (cells)
     int first, last, warp_from, pre, post, coarse, total;
-    float omega;             // over-relaxation of the pre- and post-smoothing sweeps
 };
 
 struct TailSmem {
@@ -305,7 +399,7 @@ template <bool WARP> __device__ __forceinline__ void tail_sync() {
 }
 
 template <bool WARP>
-__device__ void tail_half(const TailLevels& T, const TailSmem& S, int l, int color, const Dec& D, float omega) {
+__device__ void tail_half(const TailLevels& T, const TailSmem& S, int l, int color, const Dec& D) {
     const int nx = T.nx[l], ny = T.ny[l], nz = T.nz[l], hx = (nx + 1) / 2, o = T.off[l];
     float* e = S.e + o;
     const float* g = S.g + o;
@@ -322,7 +416,7 @@ __device__ void tail_half(const TailLevels& T, const TailSmem& S, int l, int col
                     if (!m[c]) {
                         // the diagonal is an integer (2..8): its reciprocal from the table (the same values)
                         const float v = (g[c] + s) * S.rdiag[(int)diag];
-                        e[c] = omega != 1.0f ? fmaf(omega, v - e[c], e[c]) : v;
+                        e[c] = v;
                     }
                 }
     tail_sync<WARP>();
@@ -387,17 +481,17 @@ template <bool WARP> __device__ void tail_prolong(const TailLevels& T, const Tai
 }
 
 template <bool WARP> __device__ void tail_down(const TailLevels& T, const TailSmem& S, int l, const Dec& D) {
-    for (int s = 0; s < T.pre; ++s) { tail_half<WARP>(T, S, l, 0, D, T.omega); tail_half<WARP>(T, S, l, 1, D, T.omega); }
+    for (int s = 0; s < T.pre; ++s) { tail_half<WARP>(T, S, l, 0, D); tail_half<WARP>(T, S, l, 1, D); }
     tail_restrict<WARP>(T, S, l, D);
 }
 template <bool WARP> __device__ void tail_up(const TailLevels& T, const TailSmem& S, int l, const Dec& D) {
     tail_prolong<WARP>(T, S, l, D);
-    for (int s = 0; s < T.post; ++s) { tail_half<WARP>(T, S, l, 1, D, T.omega); tail_half<WARP>(T, S, l, 0, D, T.omega); }
+    for (int s = 0; s < T.post; ++s) { tail_half<WARP>(T, S, l, 1, D); tail_half<WARP>(T, S, l, 0, D); }
 }
 template <bool WARP> __device__ void tail_coarse(const TailLevels& T, const TailSmem& S, const Dec& D) {
     for (int s = 0; s < T.coarse; ++s) {
-        tail_half<WARP>(T, S, T.last, 0, D, 1.0f);
-        tail_half<WARP>(T, S, T.last, 1, D, 1.0f);
+        tail_half<WARP>(T, S, T.last, 0, D);
+        tail_half<WARP>(T, S, T.last, 1, D);
     }
 }
 
@@ -495,12 +589,21 @@ __global__ void k_grad(const double* __restrict__ phi, int nx, int ny, int nz, d
 dim3 grid3(int nx, int ny, int nz) { return dim3((nx + BX - 1) / BX, (ny + BY - 1) / BY, nz); }
 const dim3 kBlk(BX, BY, 1);
 constexpr long long kSmoothDeep = 1ll << 20;  // levels with at least this many cells use 4 planes per thread
-void smooth_half(float* e, const float* g, const uint8_t* m, int nx, int ny, int nz, int color, float omega,
-                 cudaStream_t s) {
-    const int zs = (long long)nx * ny * nz >= kSmoothDeep ? 4 : 1;
-    const dim3 gr(((nx + 1) / 2 + BX - 1) / BX, (ny + BY - 1) / BY, (nz + zs - 1) / zs);
-    if (zs == 4) launch_pdl(k_smooth<4>, gr, kBlk, 0, s, e, g, m, nx, ny, nz, color, omega);
-    else launch_pdl(k_smooth<1>, gr, kBlk, 0, s, e, g, m, nx, ny, nz, color, omega);
+dim3 grid_pair(int nx, int ny, int nz, int zs) {
+    return dim3((nx / 2 + BX - 1) / BX, (ny + SY - 1) / SY, (nz + zs - 1) / zs);
+}
+const dim3 kPairBlk(BX, SY + 2, 1);
+void smooth_half(float* e, const float* g, const uint8_t* m, int nx, int ny, int nz, int color, cudaStream_t s) {
+    if ((long long)nx * ny * nz >= kSmoothDeep)
+        launch_pdl(k_smooth_pair<4>, grid_pair(nx, ny, nz, 4), kPairBlk, 0, s, e, g, m, nx, ny, nz, color);
+    else
+        launch_pdl(k_smooth, grid3((nx + 1) / 2, ny, nz), kBlk, 0, s, e, g, m, nx, ny, nz, color);
+}
+void sweep_first(float* e, const float* g, const uint8_t* m, int nx, int ny, int nz, cudaStream_t s) {
+    if ((long long)nx * ny * nz >= kSmoothDeep)
+        launch_pdl(k_sweep_first<4>, grid_pair(nx, ny, nz, 4), kPairBlk, 0, s, e, g, m, nx, ny, nz);
+    else
+        launch_pdl(k_sweep_first<1>, grid_pair(nx, ny, nz, 1), kPairBlk, 0, s, e, g, m, nx, ny, nz);
 }
 dim3 grid_mx3(int nx, int ny, int nz) { return dim3((nx + BX - 1) / BX, (ny + BY - 1) / BY, (nz + ZC - 1) / ZC); }
 
@@ -627,7 +730,7 @@ static TailPlan tail_plan(const MG& mg) {
 // extreme aspect); a single level of more cells keeps the plain kernel.
 bool MG::tail_tables() const {
     const int t = tail_level();
-    if (omega != 1.0f || levels - t > kTailMaxLevels) return false;
+    if (levels - t > kTailMaxLevels) return false;
     const TailPlan T = tail_plan(*this);
     if ((size_t)T.words * 4 > kTailSmem || T.L[0].ca > 0xffff || T.L[0].h > kTailPerThread * kTailThreads) return false;
     for (int l = 1; l < T.levels; ++l)
@@ -692,7 +795,6 @@ void MG::tail(cudaStream_t s, int pre, int post) {
     T.pre = pre;
     T.post = post;
     T.coarse = coarse_sweeps;
-    T.omega = omega;
     T.total = off;
     const size_t smem = tail_smem_bytes(off);
     if (smem > 48 * 1024) cudaFuncSetAttribute(k_tail_vcycle, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
@@ -710,14 +812,13 @@ void MG::vcycle(cudaStream_t s, bool light) {
     for (int l = 0; l < t; ++l) {
         const long long n = (long long)lx[l] * ly[l] * lz[l];
         if (pre > 0) {
-            launch_pdl(k_sweep_first, dim3(((lx[l] + 1) / 2 + BX - 1) / BX, (ly[l] + BY - 1) / BY, lz[l]), kBlk, 0,
-                       s, e[l], (const float*)g[l], (const uint8_t*)m[l], lx[l], ly[l], lz[l], omega);
+            sweep_first(e[l], g[l], m[l], lx[l], ly[l], lz[l], s);
         } else {
             cudaMemsetAsync(e[l], 0, n * sizeof(float), s);
         }
         for (int it = 1; it < pre; ++it) {
-            smooth_half(e[l], g[l], m[l], lx[l], ly[l], lz[l], 0, omega, s);
-            smooth_half(e[l], g[l], m[l], lx[l], ly[l], lz[l], 1, omega, s);
+            smooth_half(e[l], g[l], m[l], lx[l], ly[l], lz[l], 0, s);
+            smooth_half(e[l], g[l], m[l], lx[l], ly[l], lz[l], 1, s);
         }
         launch_pdl(k_resid_restrict, grid3(lx[l + 1], ly[l + 1], lz[l + 1]), kBlk, 0, s, (const float*)e[l],
                    (const float*)g[l], (const uint8_t*)m[l], lx[l], ly[l], lz[l], g[l + 1], (const uint8_t*)m[l + 1],
@@ -728,8 +829,8 @@ void MG::vcycle(cudaStream_t s, bool light) {
         launch_pdl(k_prolong_add, grid3(lx[l + 1], ly[l + 1], lz[l + 1]), kBlk, 0, s, (const float*)e[l + 1], e[l],
                    (const uint8_t*)m[l], lx[l], ly[l], lz[l]);
         for (int it = 0; it < post; ++it) {
-            smooth_half(e[l], g[l], m[l], lx[l], ly[l], lz[l], 1, omega, s);
-            smooth_half(e[l], g[l], m[l], lx[l], ly[l], lz[l], 0, omega, s);
+            smooth_half(e[l], g[l], m[l], lx[l], ly[l], lz[l], 1, s);
+            smooth_half(e[l], g[l], m[l], lx[l], ly[l], lz[l], 0, s);
         }
     }
 }

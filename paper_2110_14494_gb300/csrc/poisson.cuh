@@ -37,7 +37,6 @@ struct MG {
     // light_post)-cycle (0: never)
     double light_ratio = 0.0;
     int light_pre = 1, light_post = 1;
-    float omega = 1.0f;          // over-relaxation of the pre- and post-smoothing sweeps (1: Gauss-Seidel)
     // mixed solve: CG iterations run before the first convergence or
     // refinement test (0 to 2; at most max_cycles).  A coupled PIC context
     // takes 2 (its warm-started solves nearly always need two), so that the

@@ -131,3 +131,46 @@ def test_queries_do_not_depend_on_their_tile(n):
     p, xd = G._dev(th), G._dev(x)
     y = mlp_forward(p, xd)
     assert torch.equal(y, torch.cat([mlp_forward(p, xd[k:k + 1000].contiguous()) for k in range(0, n, 1000)]))
+
+
+@pytest.mark.parametrize("shape,cycles,pair", [((132, 92, 92), 24, (16, 8.340650992245674e-07)),
+                                               ((68, 132, 124), 25, (17, 6.384658163628055e-07)),
+                                               ((64, 128, 132), 25, (17, 6.774815300983311e-07)),
+                                               ((516, 44, 52), 22, (15, 5.360662387261354e-07))])
+def test_large_level_sweeps_on_ragged_tiles(shape, cycles, pair):
+    """Levels of 2^20 cells and more (pairs of cells, four planes a thread):
+    widths that end inside a warp, rows that end inside a block, scattered
+    electrode cells.  The float64 solve's residual, formed here, is what the
+    solve reports; the iterations of both solves and the residual of the
+    float-pair solve (deterministic sums) are those of sweeps with one thread a
+    cell and its six neighbours loaded, recorded once, bit by bit."""
+    from paper_2110_14494_gb300 import picmcc as P
+    nx, ny, nz = shape
+    grid = W.grid_spec(nx, ny, nz, 4e-5)
+    rng = np.random.default_rng(nx)
+    mask = (rng.random((nz, ny, nx)) < 0.002).astype(np.uint8)
+    rho = rng.uniform(-5e-2, 5e-2, (nz, ny, nx))
+    vm, lo, hi = 700.0, -100.0, 1500.0
+    dphi = torch.zeros((nz, ny, nx), dtype=torch.float64, device="cuda")
+    cyc, rel = P.poisson_solve(grid, torch.as_tensor(rho).cuda(), dphi, mask=torch.as_tensor(mask).cuda(), v_lo=lo,
+                               v_hi=hi, v_mask=vm, rtol=1e-9, max_cycles=40, precision=64)
+    f = dphi.cpu().numpy()
+    f[mask != 0] = vm
+    p = np.pad(f, 1, mode="edge")
+    p[0, 1:-1, 1:-1], p[-1, 1:-1, 1:-1] = 2 * lo - f[0], 2 * hi - f[-1]
+    nb = (p[1:-1, 1:-1, :-2] + p[1:-1, 1:-1, 2:] + p[1:-1, :-2, 1:-1] + p[1:-1, 2:, 1:-1] + p[:-2, 1:-1, 1:-1]
+          + p[2:, 1:-1, 1:-1])
+    h2e = 4e-5 ** 2 / 8.8541878128e-12
+    q = np.pad(np.where(mask, vm, 0.0), 1)
+    b = h2e * rho + (q[1:-1, 1:-1, :-2] + q[1:-1, 1:-1, 2:] + q[1:-1, :-2, 1:-1] + q[1:-1, 2:, 1:-1]
+                     + q[:-2, 1:-1, 1:-1] + q[2:, 1:-1, 1:-1])
+    b[0] += 2 * lo
+    b[-1] += 2 * hi
+    free = mask == 0
+    r = (h2e * rho + nb - 6.0 * f)[free]
+    res = np.linalg.norm(r) / np.linalg.norm(b[free])
+    assert rel <= 1e-9 and abs(res - rel) <= 1e-3 * rel + 1e-13
+    assert cyc == cycles
+    dphi.zero_()
+    assert P.poisson_solve(grid, torch.as_tensor(rho).cuda(), dphi, mask=torch.as_tensor(mask).cuda(), v_lo=lo, v_hi=hi,
+                           v_mask=vm, rtol=1e-6, max_cycles=40, precision=32) == pair
