@@ -394,8 +394,10 @@ __global__ void __launch_bounds__(BX * BY) k_mx_apply(const float* __restrict__ 
 __device__ __forceinline__ float4 ld4g(const float* p, int c) { return __ldg(reinterpret_cast<const float4*>(p + c)); }
 __device__ __forceinline__ float f4c(const float4& v, int e) { return e == 0 ? v.x : (e == 1 ? v.y : (e == 2 ? v.z : v.w)); }
 
-// Registers capped for six blocks per SM (latency-bound: more warps in flight).
-__global__ void __launch_bounds__(BX * BY, 6) k_mx_apply4(const float* __restrict__ z, const float* __restrict__ r,
+// Registers capped for seven blocks per SM (latency-bound: more warps in
+// flight, and 128^3 cells are one wave: 13.8 us, 16.5 with six; 3.4e7 cells
+// 169 and 174).
+__global__ void __launch_bounds__(BX * BY, 7) k_mx_apply4(const float* __restrict__ z, const float* __restrict__ r,
                                                        const float* __restrict__ q_prev, float* __restrict__ w,
                                                        const uint8_t* __restrict__ mask, int nx, int ny, int nz,
                                                        int first, double* part, unsigned* ctr, double* sc) {
