@@ -1327,11 +1327,9 @@ extern "C" int pic_init(const pic_config* cfg, void* d_ws, size_t ws_bytes, cons
     int dev = 0, sms = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    // Double precision: two blocks of four warps an SM fill the double pipe, and a warp that takes many
-    // electrons in turn keeps its lanes busy (2e5 electrons: two blocks 7.9 ms a step, four 8.15, one 8.3).
+    // Double precision: two blocks of four warps an SM fill the double pipe, and shared memory holds no more.
     int bps = c->prec == 32 ? PushLaunch<float>::blocks_per_sm(MODE_PIC, c->n_bins)
                             : PushLaunch<double>::blocks_per_sm(MODE_PIC, c->n_bins);
-    if (c->prec == 64 && bps > 2) bps = 2;
     c->grid_push = sms * bps;
     if (cfg->coupled) {
         if (c->g.axi) {

@@ -653,8 +653,9 @@ __device__ __forceinline__ int collide(const PushArgs<T>& A, const Rates<T>& R, 
 // electron).  Single precision: two draws, the second by the lanes whose first
 // was a null collision, then the collisions of all hits together: six of ten
 // draws are null, and a warp pays for a collision whatever its lanes.  Double
-// precision: two rounds of a draw and its collision (both cost the same on the
-// narrow double pipe, so a draw with fewer lanes gains nothing).  Measured per
+// precision (batched swarms; a single population: collide_pool): two rounds of
+// a draw and its collision (both cost the same on the narrow double pipe, so a
+// draw with fewer lanes gains nothing).  Measured per
 // pass, 1e6 electrons, float: two draws 330 us, three 355, two rounds 390;
 // 1.4e4 electrons, double: two rounds 579 us a step, two draws 610.
 template <class T, int MODE, bool FAST, bool STATS>
@@ -913,15 +914,32 @@ template <class T> struct Stage {
     T att[kAtt * 4];        // x y z w of negative-ion events
 };
 
+// Double precision: the electrons a warp has in flight (collide_pool).
+constexpr int kPool = 64;
+template <class T> struct Pool {
+    T f[14][kPool];         // x, displacement, v, a (three each), w, remaining time
+    T ht[kPool], hr[kPool]; // a hit's table coordinate and rate
+    uint64_t id[kPool];
+    uint32_t k[kPool], hz[kPool], hw[kPool];
+    T out[kOut * kRow];
+    uint64_t out_id[kOut];
+    T pq[kPQ * kPQRow];
+    uint64_t pq_id[kPQ];
+    uint32_t pq_k[kPQ];
+    T att[kAtt * 4];
+    uint8_t draw[kPool], hit[kPool], idle[kPool];  // places whose next step is a draw, a collision; free ones
+};
+template <class T> struct WarpStage { typedef Stage<T> type; };
+template <> struct WarpStage<double> { typedef Pool<double> type; };
+
 template <class T> constexpr size_t collide_smem() {
-    return ((sizeof(ProcSmem<T>) + 15) & ~(size_t)15) + 4 * sizeof(Stage<T>);
+    return ((sizeof(ProcSmem<T>) + 15) & ~(size_t)15) + 4 * sizeof(typename WarpStage<T>::type);
 }
 
 // Writes staged finished electrons [0, cnt) (lane l takes entry l): faces,
 // electrode, output append, deposit or moments; then moves entries cnt..n-1 down.
-template <class T, int MODE>
-__device__ __forceinline__ void flush_out(const PushArgs<T>& A, Stage<T>* sg, int& n, int cnt, LStats& ls,
-                                          MomAcc<T>& M) {
+template <class T, int MODE, class S>
+__device__ __forceinline__ void flush_out(const PushArgs<T>& A, S* sg, int& n, int cnt, LStats& ls, MomAcc<T>& M) {
     const int lane = threadIdx.x & 31;
     __syncwarp();
     bool live = lane < cnt;
@@ -995,8 +1013,7 @@ __device__ __forceinline__ void build_product(const PushArgs<T>& A, const T* e, 
 }
 
 // Deposits the buffered negative-ion events [0, n) of the warp, one per lane.
-template <class T>
-__device__ __forceinline__ void flush_att(const PushArgs<T>& A, Stage<T>* sg, int& n) {
+template <class T, class S> __device__ __forceinline__ void flush_att(const PushArgs<T>& A, S* sg, int& n) {
     const int lane = threadIdx.x & 31;
     __syncwarp();
     if (lane < n) {
@@ -1077,14 +1094,13 @@ __device__ __forceinline__ void collide_loop(const PushArgs<T>& A, const ProcSme
             } else {
                 // A warp's first items follow from its place, in an order that
                 // fills the SMs and their four schedulers evenly; later ones
-                // come from the cursor.  With few items a warp of single
-                // precision takes fewer at a time, so that more schedulers work
-                // (a lane's chain of draws, not the issue rate, takes the time
-                // then); double precision fills its warps, whose cost is the
-                // same for any number of lanes.  (Capacities are below 2^31.)
+                // come from the cursor.  With few items a warp takes fewer at a
+                // time, so that more schedulers work (a lane's chain of draws,
+                // not the issue rate, takes the time then).  (Capacities are
+                // below 2^31.)
                 const unsigned warps = gridDim.x * (blockDim.x >> 5), n_items = (unsigned)items();
                 unsigned chunk = 32;
-                if (FAST && n_items <= 24u * warps) chunk = (n_items / warps + 8u) & ~7u;
+                if (n_items <= 24u * warps) chunk = (n_items / warps + 8u) & ~7u;
                 unsigned b = 0;
                 if (first) {
                     b = ((((threadIdx.x >> 5) - blockIdx.x / (unsigned)A.sms) & 3u) * gridDim.x + blockIdx.x) * chunk;
@@ -1206,6 +1222,277 @@ __device__ __forceinline__ void collide_loop(const PushArgs<T>& A, const ProcSme
     }
 }
 
+// The collision loop of double precision.  A warp operation costs the double
+// pipe 18 clocks of the whole multiprocessor whatever its lanes, a draw about
+// 1900 of them and a collision 2300, and six of ten draws are null collisions:
+// a lane that owns an electron makes every warp pay for both at every draw.
+// So a warp keeps up to 64 electrons in shared memory (moving one costs ~30
+// shared accesses) and does, as long as there are enough, 32 draws or 32
+// collisions at a time; places wait in lists.  A draw whose rate lies clearly
+// above the interpolated total (by more than the two sums can differ) is a null
+// collision at once; any other goes to the collision, which decides exactly.
+// Same draws, same operations on each electron as collide_loop.  1e5 streamer
+// electrons: 2.76 ms a step, a lane an electron 3.95; 1.4e4 swarm electrons,
+// which hardly fill the warps: 197 and 190 us.
+template <class T, int MODE, bool STATS, bool CHILD>
+__device__ __forceinline__ void collide_pool(const PushArgs<T>& A, const ProcSmem<T>* ps, Pool<T>* sg) {
+    const int lane = threadIdx.x & 31;
+    const unsigned lt = (1u << lane) - 1u;
+    unsigned long long* cursor = CHILD ? &A.st->n_fetch_c : &A.st->n_fetch;
+    const ChildQ<T>& src = (A.gen & 1) ? A.cq2 : A.cq;
+    const ChildQ<T>& dst = CHILD ? ((A.gen & 1) ? A.cq : A.cq2) : A.cq;  // products the warp queue cannot take
+    unsigned long long* dst_cnt = CHILD ? ((A.gen & 1) ? &A.st->n_child : &A.st->n_spill) : &A.st->n_child;
+    long long items = (long long)(CHILD ? ((A.gen & 1) ? A.st->n_spill : A.st->n_child) : A.st->n_in);
+    if (CHILD) {
+        if (items > A.cap_child) items = A.cap_child;
+        if (items == 0) return;
+        if (blockIdx.x == 0 && threadIdx.x == 0) atomicAdd(&A.st->n_updates, (unsigned long long)items);
+    }
+    LStats ls;
+    ls.zero();
+    MomAcc<T> M;
+    if (MODE == MODE_SWARM) M.zero();
+    const Rates<T> rates{A.table, A.nu_max, A.tau_scale};
+    // First items by place, one range a warp: as many warps on each SM as its
+    // share fills with 32 electrons each (1.4e4 electrons, three warps an SM:
+    // 197 us; two of 46 208, four of 23 210), then from the cursor.
+    const unsigned n_items = (unsigned)items, sms = (unsigned)A.sms, warps = gridDim.x * (blockDim.x >> 5);
+    const unsigned per_sm = (n_items + 32u * sms - 1) / (32u * sms);
+    const unsigned chunk = per_sm > 0 ? (n_items + sms * per_sm - 1) / (sms * per_sm) : 1u;  // 32 at most
+    unsigned next = ((((threadIdx.x >> 5) - blockIdx.x / sms) & 3u) * gridDim.x + blockIdx.x) * chunk;
+    unsigned end = next < n_items ? (n_items - next < chunk ? n_items : next + chunk) : 0u;
+    if (end == 0u) next = 0u;
+    // warp-uniform: sizes of the lists, of the output stage, queued products, buffered negative-ion events
+    int nd = 0, nh = 0, nf = kPool, n_out = 0, n_pq = 0, n_att = 0, trips = 0;
+    bool dry = false;
+    for (int q = lane; q < kPool; q += 32) sg->idle[q] = (uint8_t)q;
+    for (;;) {
+        if (++trips > kTripLimit) { atomicOr(&A.st->err, kErrStack); break; }
+        __syncwarp();
+        const bool products = n_pq >= 32 || (dry && n_pq > 0);
+        // 1. places are filled while fewer than 32 electrons wait for a draw
+        if (nh < 32 && nd < 32 && (products || !dry) && (nf >= 8 || nd + nh == 0)) {
+            int cnt = n_pq < 32 ? n_pq : 32;
+            if (!products) {
+                if (next >= end) {
+                    unsigned long long c = 0;
+                    if (lane == 0) c = atomicAdd(cursor, (unsigned long long)(nf < 32 ? nf : 32));
+                    c = __shfl_sync(kFull, c, 0) + (unsigned long long)warps * chunk;
+                    next = c < n_items ? (unsigned)c : n_items;
+                    const unsigned most = (unsigned)(nf < 32 ? nf : 32);
+                    end = n_items - next < most ? n_items : next + most;
+                }
+                cnt = (int)(end - next) < 32 ? (int)(end - next) : 32;
+                if (cnt <= 0) {
+                    dry = true;
+                    continue;
+                }
+            }
+            if (cnt > nf) cnt = nf;
+            const bool on = lane < cnt;
+            int p = 0;
+            T r[kRow] = {};
+            uint64_t id = 0;
+            if (on) {
+                p = sg->idle[nf - cnt + lane];
+                if (products) {
+                    const int j = n_pq - cnt + lane;
+                    build_product<T, MODE>(A, sg->pq + j * kPQRow, sg->pq_id[j], sg->pq_k[j], r, &id);
+                } else {
+                    const long long it = (long long)next + lane;
+                    if (CHILD) {
+                        const Soa<T>& q = src.p;
+                        const T e[kPQRow] = {q.r[PX][it], q.r[PY][it], q.r[PZ][it], q.r[VX][it], q.r[AX][it],
+                                             q.r[AY][it], q.r[AZ][it], q.r[PW][it], src.t_left[it]};
+                        build_product<T, MODE>(A, e, q.id[it], src.k[it], r, &id);
+                    } else {
+                        for (int q = 0; q < 10; ++q) r[q] = A.in.r[q][it];
+                        if (MODE == MODE_PIC && A.kick_on_load) half_kick(A, r);
+                        r[10] = A.dt;
+                        id = A.in.id[it];
+                    }
+                }
+            }
+            if (products) {
+                if (lane == 0) atomicAdd(&A.st->n_updates, (unsigned long long)cnt);
+                n_pq -= cnt;
+            } else {
+                next += (unsigned)cnt;
+            }
+            nf -= cnt;
+            const bool alive = on && r[9] > (T)0;
+            const unsigned am = __ballot_sync(kFull, alive), em = __ballot_sync(kFull, on && !alive);
+            if (alive) {
+                ++ls.processed;
+                for (int q = 0; q < 3; ++q) {
+                    sg->f[q][p] = r[q];
+                    sg->f[3 + q][p] = (T)0;
+                    sg->f[6 + q][p] = r[3 + q];
+                    sg->f[9 + q][p] = r[6 + q];
+                }
+                sg->f[12][p] = r[9];
+                sg->f[13][p] = r[10];
+                sg->id[p] = id;
+                sg->k[p] = 1;
+                sg->draw[nd + __popc(am & lt)] = (uint8_t)p;
+            }
+            __syncwarp();
+            if (on && !alive) sg->idle[nf + __popc(em & lt)] = (uint8_t)p;
+            nd += __popc(am);
+            nf += __popc(em);
+            continue;
+        }
+        if (nd + nh == 0) break;  // nothing in flight, nothing to come
+        Lane<T> L;
+        Hit<T> h;
+        int p = 0, r = EV_CONTINUE;
+        T sp = (T)0;
+        bool on;
+        const bool draws = nh < 32 && nd >= nh;
+        if (draws) {
+            // 2. draws
+            const int cnt = nd < 32 ? nd : 32;
+            on = lane < cnt;
+            nd -= cnt;
+            if (on) {
+                p = sg->draw[nd + lane];
+                for (int q = 0; q < 3; ++q) { L.d[q] = sg->f[3 + q][p]; L.v[q] = sg->f[6 + q][p]; L.a[q] = sg->f[9 + q][p]; }
+                L.t_left = sg->f[13][p];
+                L.id = sg->id[p];
+                L.k = sg->k[p];
+                r = candidate<T, false>(A, rates, A.K, A.step, L, ls, h);
+                if (r == EV_HIT) {
+                    int j;
+                    T f, t0, dt;
+                    table_split(A, h.t, j, f);
+                    LdTab<T>::pair(A.table + A.n_bins * kTableRow + 2 * j, t0, dt);
+                    if (h.target >= (t0 + f * dt) * (T)(1.0 + 1e-12)) { ++ls.nulls; r = EV_CONTINUE; }
+                }
+                for (int q = 0; q < 3; ++q) { sg->f[3 + q][p] = L.d[q]; sg->f[6 + q][p] = L.v[q]; }
+                sg->f[13][p] = L.t_left;
+                sg->k[p] = L.k;
+                if (r == EV_HIT) {
+                    sg->ht[p] = h.t;
+                    sg->hr[p] = h.target;
+                    sg->hz[p] = h.z;
+                    sg->hw[p] = h.w;
+                }
+            }
+        } else {
+            // 3. collisions
+            const int cnt = nh < 32 ? nh : 32;
+            on = lane < cnt;
+            nh -= cnt;
+            if (on) {
+                p = sg->hit[nh + lane];
+                for (int q = 0; q < 3; ++q) L.v[q] = sg->f[6 + q][p];
+                L.w = sg->f[12][p];
+                h.t = sg->ht[p];
+                h.target = sg->hr[p];
+                h.z = sg->hz[p];
+                h.w = sg->hw[p];
+                r = collide<T, MODE, STATS>(A, rates, ps, h, L, ls, sp);
+                for (int q = 0; q < 3; ++q) sg->f[6 + q][p] = L.v[q];
+            }
+        }
+        __syncwarp();
+        const bool done = on && r == EV_DONE, ion = on && r == EV_IONIZED, att = on && r == EV_ATTACHED;
+        // 4. back into the lists
+        const unsigned cm = __ballot_sync(kFull, on && (r == EV_CONTINUE || ion)), hm = __ballot_sync(kFull, on && r == EV_HIT),
+                       xm = __ballot_sync(kFull, done || att);
+        if (cm >> lane & 1u) sg->draw[nd + __popc(cm & lt)] = (uint8_t)p;
+        if (hm >> lane & 1u) sg->hit[nh + __popc(hm & lt)] = (uint8_t)p;
+        if (xm >> lane & 1u) sg->idle[nf + __popc(xm & lt)] = (uint8_t)p;
+        nd += __popc(cm);
+        nh += __popc(hm);
+        nf += __popc(xm);
+        if (draws) {
+            // 5. finished electrons
+            const unsigned dm = __ballot_sync(kFull, done);
+            if (dm) {
+                if (done) {
+                    const int e = n_out + __popc(dm & lt);
+                    T* q = sg->out + e * kRow;
+                    for (int d = 0; d < 3; ++d) {
+                        q[d] = sg->f[d][p] + L.d[d];
+                        q[3 + d] = L.v[d];
+                        q[6 + d] = L.a[d];
+                    }
+                    q[9] = sg->f[12][p];
+                    sg->out_id[e] = L.id;
+                }
+                n_out += __popc(dm);
+                if (n_out >= 32) flush_out<T, MODE>(A, sg, n_out, 32, ls, M);
+            }
+            continue;
+        }
+        // 6. ionization products wait in the warp queue (the queue of the next launch when it is full)
+        const unsigned im = __ballot_sync(kFull, ion);
+        if (im) {
+            if (ion) {
+                const int slot = n_pq + __popc(im & lt);
+                const T e[kPQRow] = {sg->f[0][p] + sg->f[3][p], sg->f[1][p] + sg->f[4][p], sg->f[2][p] + sg->f[5][p], sp,
+                                     sg->f[9][p], sg->f[10][p], sg->f[11][p], L.w, sg->f[13][p]};
+                const uint64_t id = sg->id[p];
+                const uint32_t k = sg->k[p] - 1;
+                if (slot < kPQ) {
+                    T* q = sg->pq + slot * kPQRow;
+                    for (int f = 0; f < kPQRow; ++f) q[f] = e[f];
+                    sg->pq_id[slot] = id;
+                    sg->pq_k[slot] = k;
+                    ++ls.children;
+                } else {
+                    const unsigned long long q = atomicAdd(dst_cnt, 1ull);
+                    if ((long long)q < A.cap_child) {
+                        const Soa<T>& d = dst.p;
+                        d.r[PX][q] = e[0]; d.r[PY][q] = e[1]; d.r[PZ][q] = e[2];
+                        d.r[VX][q] = sp;
+                        d.r[AX][q] = e[4]; d.r[AY][q] = e[5]; d.r[AZ][q] = e[6];
+                        d.r[PW][q] = L.w;
+                        d.id[q] = id;
+                        dst.t_left[q] = e[8];
+                        dst.k[q] = k;
+                        ++ls.children;
+                    } else {
+                        atomicOr(&A.st->err, kErrChildCapacity);
+                    }
+                }
+            }
+            n_pq += __popc(im);
+            if (n_pq > kPQ) n_pq = kPQ;
+        }
+        // 7. negative-ion events wait for a deposit by 32 lanes at once
+        if (MODE == MODE_PIC) {
+            const unsigned am = __ballot_sync(kFull, att);
+            if (am && A.q_neg) {
+                if (n_att + __popc(am) > kAtt) flush_att(A, sg, n_att);
+                if (att) {
+                    T* q = sg->att + (n_att + __popc(am & lt)) * 4;
+                    for (int d = 0; d < 3; ++d) q[d] = sg->f[d][p] + sg->f[3 + d][p];
+                    q[3] = L.w;
+                }
+                n_att += __popc(am);
+            }
+        }
+    }
+    if (n_out > 0) flush_out<T, MODE>(A, sg, n_out, n_out, ls, M);
+    if (MODE == MODE_PIC && n_att > 0) flush_att(A, sg, n_att);
+    if (STATS) flush_stats(A, ls, A.n_proc);
+    if (MODE == MODE_SWARM) {
+        M.m[14] += ls.w_ion;
+        M.m[15] += ls.w_att;
+        __syncthreads();
+        flush_moments(A, M, reinterpret_cast<double*>(sg - (threadIdx.x >> 5)));  // block-wide scratch
+    }
+}
+
+// Single precision keeps an electron on a lane; double precision pools them.
+template <class T, int MODE, bool FAST, bool STATS, bool CHILD>
+__device__ __forceinline__ void collide_items(const PushArgs<T>& A, const ProcSmem<T>* ps, typename WarpStage<T>::type* sg) {
+    if constexpr (FAST) collide_loop<T, MODE, FAST, STATS, CHILD>(A, ps, sg);
+    else collide_pool<T, MODE, STATS, CHILD>(A, ps, sg);
+}
+
 template <class T> __device__ __forceinline__ ProcSmem<T>* stage_proc(unsigned char* raw, const PushArgs<T>& A) {
     ProcSmem<T>* ps = reinterpret_cast<ProcSmem<T>*>(raw);
     if (threadIdx.x < 8) {
@@ -1217,29 +1504,31 @@ template <class T> __device__ __forceinline__ ProcSmem<T>* stage_proc(unsigned c
     return ps;
 }
 
-template <class T> __device__ __forceinline__ Stage<T>* warp_stage(unsigned char* raw) {
-    return reinterpret_cast<Stage<T>*>(raw + ((sizeof(ProcSmem<T>) + 15) & ~(size_t)15)) + (threadIdx.x >> 5);
+template <class T> __device__ __forceinline__ typename WarpStage<T>::type* warp_stage(unsigned char* raw) {
+    typedef typename WarpStage<T>::type S;
+    return reinterpret_cast<S*>(raw + ((sizeof(ProcSmem<T>) + 15) & ~(size_t)15)) + (threadIdx.x >> 5);
 }
 
 constexpr int kCollideThreads = 128;
 // Resident blocks per SM the collision kernels are compiled for: six (24
 // warps, 80 registers, 76 KB of L1 left beside their stages for the 40 KB of
-// tables) in single precision, four in double precision.  1e6 electrons in
+// tables) in single precision, two in double precision (their double pipe is
+// full then).  1e6 electrons in
 // float: six 330 us, seven 356 (72 registers, 47 KB of L1), five 346.
-template <class T> constexpr int collide_min_blocks() { return sizeof(T) == 4 ? 6 : 4; }
+template <class T> constexpr int collide_min_blocks() { return sizeof(T) == 4 ? 6 : 2; }
 
 template <class T, int MODE, bool FAST, bool STATS>
 __global__ void __launch_bounds__(kCollideThreads, collide_min_blocks<T>()) k_push(const PushArgs<T> A) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const ProcSmem<T>* ps = stage_proc(smem_raw, A);
-    collide_loop<T, MODE, FAST, STATS, false>(A, ps, warp_stage<T>(smem_raw));
+    collide_items<T, MODE, FAST, STATS, false>(A, ps, warp_stage<T>(smem_raw));
 }
 
 template <class T, int MODE, bool FAST, bool STATS>
 __global__ void __launch_bounds__(kCollideThreads, collide_min_blocks<T>()) k_children(const PushArgs<T> A) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const ProcSmem<T>* ps = stage_proc(smem_raw, A);
-    collide_loop<T, MODE, FAST, STATS, true>(A, ps, warp_stage<T>(smem_raw));
+    collide_items<T, MODE, FAST, STATS, true>(A, ps, warp_stage<T>(smem_raw));
 }
 
 // Deposit of the current particle set (no push).

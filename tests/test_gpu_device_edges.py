@@ -174,3 +174,42 @@ def test_large_level_sweeps_on_ragged_tiles(shape, cycles, pair):
     dphi.zero_()
     assert P.poisson_solve(grid, torch.as_tensor(rho).cuda(), dphi, mask=torch.as_tensor(mask).cuda(), v_lo=lo, v_hi=hi,
                            v_mask=vm, rtol=1e-6, max_cycles=40, precision=32) == pair
+
+
+def _push_case(n, prec, steps):
+    """n electrons by the device and by the oracle: (common, only device, only oracle, outside, worst)."""
+    from paper_2110_14494_gb300 import PicContext
+    from tests import test_gpu_pic as G
+    from tests.gpu_common import compare_sets
+    gas, F, mk, p0 = G._setup(n, prec, 11)
+    dt, cap = 2e-12, 8 * n + 4096
+    ctx = PicContext(gas, G.GRID, precision=prec, capacity=cap, seed=SEED, dt=dt, mask=mk)
+    ctx.set_field(*G._field_dev(F))
+    ctx.set_particles(p0)
+    ctx.step(steps)
+    m = O.Model(gas, dt, SEED, prec, G.GRID, F, mask=mk)
+    P = O.Particles(cap, p0)
+    nc = G.GRID["nx"] * G.GRID["ny"] * G.GRID["nz"]
+    rq = [np.zeros(nc, np.int64) for _ in range(2)]
+    for s in range(1, steps + 1):
+        rc, _ = O.step(m, P, s, s == 1, np.zeros(nc, np.int64), *rq)
+        assert rc == 0
+    return compare_sets(ctx.get_particles(), P.view(), G.GRID["dx"], 1e-12 if prec == 64 else 1e-3, v_floor=1.0)
+
+
+@pytest.mark.parametrize("n", [2, 31, 32, 64, 65, 32 * 152, 32 * 152 + 1, 8 * 32 * 152 + 77])
+def test_pool_of_electrons_at_its_edges(n):
+    """Double precision: warps with one electron to a full pool, ranges that end
+    inside a warp, items beyond the first ranges; particle by particle to 1e-12,
+    as elsewhere for float64."""
+    nc, og, orf, bad, worst = _push_case(n, 64, 2)
+    assert og == 0 and orf == 0 and bad == 0, (og, orf, worst)
+
+
+@pytest.mark.parametrize("n", [1, 7, 8, 9, 33, 4096, 24 * 3648 - 1, 24 * 3648 + 1])
+def test_electrons_by_place_at_range_edges(n):
+    """Single precision: ranges of 8, 16, 24 and 32 electrons and their last
+    ones.  Decision flips (gross differences) at most 1e-5 of the particles plus
+    two, as elsewhere for float32."""
+    nc, og, orf, bad, worst = _push_case(n, 32, 1)
+    assert nc >= n * 0.9 and og + orf + worst["gross"] <= 1e-5 * nc + 2, (og, orf, worst)
