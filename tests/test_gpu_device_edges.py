@@ -213,3 +213,33 @@ def test_electrons_by_place_at_range_edges(n):
     two, as elsewhere for float32."""
     nc, og, orf, bad, worst = _push_case(n, 32, 1)
     assert nc >= n * 0.9 and og + orf + worst["gross"] <= 1e-5 * nc + 2, (og, orf, worst)
+
+
+@pytest.mark.parametrize("shape", [(2, 2, 2), (33, 6, 10), (35, 9, 13), (20, 20, 20), (64, 48, 40), (100, 20, 36)])
+def test_pair_solve_and_field_at_block_edges(shape):
+    """Float-pair residual and field: grids whose rows end inside a warp, whose
+    rows and planes end inside a block, planes at the plates and those between,
+    with and without electrode cells.  The potential is the oracle's; the field
+    is the centred difference of that potential, whose pair difference and scaling
+    round three times (2e-7), the pair itself to 2^-47."""
+    from paper_2110_14494_gb300 import picmcc as P
+    nx, ny, nz = shape
+    h, lo, hi, vm = 4e-5, -100.0, 1500.0, 700.0
+    grid = W.grid_spec(nx, ny, nz, h)
+    rng = np.random.default_rng(nx + ny)
+    rho = rng.uniform(-5e-2, 5e-2, (nz, ny, nx))
+    for density in (0.0, 0.03):
+        mask = (rng.random((nz, ny, nx)) < density).astype(np.uint8)
+        ref, _, _ = O.poisson(grid, rho, mask, vm, lo, hi, rtol=1e-12)
+        phi = torch.zeros((nz, ny, nx), dtype=torch.float64, device="cuda")
+        E = tuple(torch.zeros((nz, ny, nx), dtype=torch.float32, device="cuda") for _ in range(3))
+        P.poisson_solve(grid, torch.as_tensor(rho).cuda(), phi, mask=torch.as_tensor(mask).cuda(), E=E, v_lo=lo, v_hi=hi,
+                        v_mask=vm, rtol=1e-8, max_cycles=500, precision=32)
+        f = phi.cpu().numpy()
+        assert np.linalg.norm(f - ref) <= 1e-5 * np.linalg.norm(ref)
+        p = np.pad(f, 1, mode="edge")
+        p[0, 1:-1, 1:-1], p[-1, 1:-1, 1:-1] = 2 * lo - f[0], 2 * hi - f[-1]
+        want = (-(p[1:-1, 1:-1, 2:] - p[1:-1, 1:-1, :-2]) / (2 * h), -(p[1:-1, 2:, 1:-1] - p[1:-1, :-2, 1:-1]) / (2 * h),
+                -(p[2:, 1:-1, 1:-1] - p[:-2, 1:-1, 1:-1]) / (2 * h))
+        for e, w in zip(E, want):
+            assert np.all(np.abs(e.cpu().numpy() - w) <= 5e-7 * np.abs(w) + 2.0 ** -44 * np.abs(f).max() / h)
