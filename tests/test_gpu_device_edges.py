@@ -243,3 +243,30 @@ def test_pair_solve_and_field_at_block_edges(shape):
                 -(p[2:, 1:-1, 1:-1] - p[:-2, 1:-1, 1:-1]) / (2 * h))
         for e, w in zip(E, want):
             assert np.all(np.abs(e.cpu().numpy() - w) <= 5e-7 * np.abs(w) + 2.0 ** -44 * np.abs(f).max() / h)
+
+
+@pytest.mark.parametrize("shape", [(2, 2, 2), (13, 17, 31), (16, 16, 32), (264, 256, 256)])
+def test_weight_update_on_grids_around_the_scan_tiles(shape):
+    """The cell scan's tiles of 2048 and its second level's 8192 tiles: fewer
+    cells than a thread's eight, a ragged last tile, whole tiles, more than 8192
+    tiles; cells with thousands of electrons beside empty ones.  The merged and
+    split set is the oracle's, bit for bit."""
+    from paper_2110_14494_gb300 import PicContext
+    from tests.gpu_common import by_id
+    grid = W.grid_spec(*shape, 1e-4)
+    p0 = W.random_particles(6000, grid, 51, w_range=(1.0, 3.0))
+    for k in ("x", "y", "z"):  # half of them in the first and the last cells
+        p0[k][:2000] = np.float32(0.5e-4)
+        p0[k][2000:3000] = np.float32((dict(x=shape[0], y=shape[1], z=shape[2])[k] - 0.5) * 1e-4)
+    gas = W.synthetic_air()
+    ctx = PicContext(gas, grid, precision=32, capacity=40000, seed=SEED, dt=1e-12, n_ppc=10, w_min=1.0, particle_cap=0)
+    ctx.set_particles(p0)
+    ctx.weight_update()
+    gpu = by_id(ctx.get_particles())
+    P = O.Particles(40000, p0)
+    rc, _ = O.merge_split(O.Model(gas, 1e-12, SEED, 32, grid), P, 0, n_ppc=10, w_min=1.0, cap=0)
+    ref = by_id(P.view())
+    assert rc == 0 and len(ref["id"]) != len(p0["id"])
+    assert np.array_equal(gpu["id"], ref["id"])
+    for k in ("x", "y", "z", "vx", "vy", "vz", "w"):
+        assert np.array_equal(gpu[k], ref[k]), k
