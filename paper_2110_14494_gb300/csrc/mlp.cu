@@ -825,10 +825,9 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_infer_tc(const float* __restr
     const int tid = threadIdx.x, warp = tid >> 5;
     const int group = tid / kTcGroup, gt = tid % kTcGroup, row = gt & (kTcRows - 1), half = gt >> 7;
     // operands and parameters
-    for (int k = tid; k < NH * NH; k += kTcThreads) {
-        const int o = k / NH, i = k % NH;
-        *reinterpret_cast<__nv_bfloat16*>(S.w2 + kmajor_off(o, i)) = w2b[k];
-    }
+    for (int q = tid; q < NH * NH / 8; q += kTcThreads)  // eight inputs of a unit are 16 bytes in both layouts
+        *reinterpret_cast<uint4*>(S.w2 + kmajor_off(q / (NH / 8), q % (NH / 8) * 8)) =
+            reinterpret_cast<const uint4*>(w2b)[q];
     for (int k = tid; k < 16 * NH; k += kTcThreads) {
         const int o = k / NH, i = k % NH;
         *reinterpret_cast<__nv_bfloat16*>(S.w3 + kmajor_off(o, i)) =
