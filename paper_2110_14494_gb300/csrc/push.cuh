@@ -878,25 +878,24 @@ static __global__ void k_resample_commit(DevState* st) {
 
 // ------------------------------------------------------------------ collisions
 // Lanes refill from per-warp shared-memory stages.  Every lane owns one
-// electron at a time and advances it by up to two draws per loop iteration
-// (advance); a lane whose electron has finished the step takes the next
-// electron from the warp's input stage at once, so the warp stays converged
-// while electrons need different numbers of events.  All per-electron memory
-// work is done by the whole warp, 32 electrons at a time: the input stage is
-// filled with one coalesced load of 32 consecutive work items, finished
-// electrons wait in the output stage until 32 are there and are then
+// electron at a time and advances it by up to two draws and a collision per
+// loop iteration (advance); a lane whose electron has finished the step takes
+// the next electron from the warp's input stage at once, so the warp stays
+// converged while electrons need different numbers of events.  All
+// per-electron memory work is done by the whole warp, 32 electrons at a time:
+// the input stage is filled with one coalesced load of consecutive work items,
+// finished electrons wait in the output stage until 32 are there and are then
 // reflected at the faces, tested against the electrode, appended with one
-// cursor increment, stored and deposited by 32 lanes together.  An
-// ionization product is built at once (derived id, direction from its own
-// draw, positive-ion event of its birth) and pushed on the lane's stack;
-// the lane finishes its stack before it takes the next work item, flying
-// each product for the remaining time with the acceleration of the electron
-// the stack started from.  A product that finds the stack full waits, as a
-// compact entry, in the queue of the next (children) launch.
+// cursor increment, stored and deposited by 32 lanes together.  An ionization
+// product waits as a compact entry in the warp's queue and is built (derived
+// id, direction from its own draw, positive-ion event of its birth) with 31
+// others as the stage's next work items; it flies the remaining time with the
+// acceleration of the electron that ionized.  A product that finds the queue
+// full waits in the queue of the next (children) launch.
 //
-// CHILD = false: work item = one electron of the input buffer (already kicked
-// by k_field_kick), flying dt.  CHILD = true: work item = one queued
-// ionization product, built when it is staged.
+// CHILD = false: work item = one electron of the input buffer (kicked by
+// k_field_kick, or as it is staged), flying dt.  CHILD = true: work item = one
+// queued ionization product, built when it is staged.
 constexpr int kTripLimit = 1 << 24;  // of a warp in one launch (a minute): an error instead of an endless kernel
 constexpr int kRow = 11;    // padded row of a stage entry: x y z vx vy vz ax ay az w t
 constexpr int kOut = 64;    // output stage capacity (flushed at 32)
