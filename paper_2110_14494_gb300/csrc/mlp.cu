@@ -1004,9 +1004,24 @@ __global__ void k_fold(const float* __restrict__ th, Affine a, float* __restrict
 // O2 fraction, in float32 (the network's input precision; a float64
 // logarithm would run on this GPU's slow float64 units).
 __global__ void k_features(const double* __restrict__ en, const double* __restrict__ f, float* __restrict__ x,
-                           long long n) {
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
+                           long long n, bool wide) {
+    const long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x, step = (long long)gridDim.x * blockDim.x;
+    auto one = [&](long long i) {
         reinterpret_cast<float2*>(x)[i] = make_float2(log10f((float)en[i]), (float)f[i]);
+    };
+    if (!wide) {
+        for (long long i = t; i < n; i += step) one(i);
+        return;
+    }
+    for (long long i = t; i < n / 4; i += step) {
+        const double2* q = reinterpret_cast<const double2*>(en) + 2 * i;
+        const double2* g = reinterpret_cast<const double2*>(f) + 2 * i;
+        const double2 a = q[0], b = q[1], c = g[0], d = g[1];
+        float4* o = reinterpret_cast<float4*>(x) + 2 * i;
+        o[0] = make_float4(log10f((float)a.x), (float)c.x, log10f((float)a.y), (float)c.y);
+        o[1] = make_float4(log10f((float)b.x), (float)d.x, log10f((float)b.y), (float)d.y);
+    }
+    if (t < (n & 3)) one((n & ~3ll) + t);
 }
 
 }  // namespace mlp
@@ -1142,12 +1157,16 @@ extern "C" int mlp_fold_standardization(const float* params, const double x_mean
     return cudaGetLastError() == cudaSuccess ? PIC_OK : PIC_ERR_CUDA;
 }
 
+// Four points a thread from 16-byte aligned arrays: more bytes in flight (1.7e7 points 83 us with one, 59 now);
+// below 2^18 points one a thread fills more SMs.
+constexpr long long kWideFeatures = 1ll << 18;
 extern "C" int mlp_features(const double* EN_Td, const double* f_o2, float* x, long long n, pic_stream_t stream) {
     if (n < 0 || (n > 0 && (!EN_Td || !f_o2 || !x))) return PIC_ERR_ARG;
     if (n == 0) return PIC_OK;
-    long long g = (n + 255) / 256;
+    const bool wide = (((uintptr_t)EN_Td | (uintptr_t)f_o2 | (uintptr_t)x) & 15) == 0 && n >= kWideFeatures;
+    long long g = (wide ? n / 4 + 255 : n + 255) / 256;
     if (g > 65535) g = 65535;
-    mlp::k_features<<<(unsigned)g, 256, 0, (cudaStream_t)stream>>>(EN_Td, f_o2, x, n);
+    mlp::k_features<<<(unsigned)g, 256, 0, (cudaStream_t)stream>>>(EN_Td, f_o2, x, n, wide);
     return cudaGetLastError() == cudaSuccess ? PIC_OK : PIC_ERR_CUDA;
 }
 

@@ -270,3 +270,21 @@ def test_weight_update_on_grids_around_the_scan_tiles(shape):
     assert np.array_equal(gpu["id"], ref["id"])
     for k in ("x", "y", "z", "vx", "vy", "vz", "w"):
         assert np.array_equal(gpu[k], ref[k]), k
+
+
+@pytest.mark.parametrize("n", [1, 3, (1 << 18) - 1, 1 << 18, (1 << 18) + 3])
+def test_features_of_aligned_and_shifted_arrays(n):
+    """Four points a thread, with a remainder, and one a thread (few points, or
+    arrays that begin eight bytes off a 16-byte boundary): the same bits; and
+    log10 of the float32 value to 2 units in the last place, its stated error."""
+    from paper_2110_14494_gb300 import mlp_features
+    rng = np.random.default_rng(n)
+    en = torch.as_tensor(10 ** rng.uniform(0, 3.5, n + 1)).cuda()
+    f = torch.as_tensor(rng.uniform(0, 1, n + 1)).cuda()
+    shifted = mlp_features(en[1:], f[1:])
+    aligned = mlp_features(en[1:].clone(), f[1:].clone())
+    assert torch.equal(shifted, aligned)
+    ref = np.log10(en[1:].cpu().numpy().astype(np.float32).astype(np.float64))
+    x = aligned.cpu().numpy()
+    assert np.all(np.abs(x[:, 0] - ref) <= 2 * np.spacing(np.abs(ref).astype(np.float32)))
+    assert np.array_equal(x[:, 1], f[1:].cpu().numpy().astype(np.float32))
