@@ -285,6 +285,10 @@ __global__ void k_extrapolate(double* __restrict__ phi, double* __restrict__ pre
 }
 
 __global__ void k_end_step(DevState* st, long long* count_slot, long long cap) {
+    if (count_slot && st->n_extra) {  // a swarm step that began by doubling its electrons
+        st->n_in = st->n_extra;
+        st->n_extra = 0;
+    }
     st->n_updates += st->n_in;
     st->n_parents += st->n_in;
     st->n_spill = 0;
@@ -2572,7 +2576,6 @@ template <class T> static int swarm_one(pic_ctx* c, const swarm_config* sc, doub
         A.mask = nullptr;
         A.q_e = A.q_pos = A.q_neg = nullptr;
         cudaError_t e = PushLaunch<T>::resample(A, grid_n(2 * sc->n_hi), c->s);
-        if (e == cudaSuccess) e = PushLaunch<T>::field_kick(A, grid_n(2 * sc->n_hi), c->s);
         if (e == cudaSuccess) e = PushLaunch<T>::parents(A, MODE_SWARM, false, c->grid_push, c->s);
         if (e == cudaSuccess) e = PushLaunch<T>::children(A, MODE_SWARM, false, c->grid_push, c->s);
         if (e != cudaSuccess) return c->cuda_fail(e, "swarm push");

@@ -731,31 +731,26 @@ __device__ __forceinline__ void store(const Soa<T>& o, unsigned long long s, con
     o.r[PW][s] = w; o.id[s] = id;
 }
 
-// ------------------------------------------------------------------ field kick
-// Sec. 2.1.1, Eq. 2: a_new = -(e/m_e) E(x) from the trilinear gather; the
-// half-kick v += dt/2 (a_new - a_old) completes the previous step's velocity
-// update (skipped when a_old is unknown); a_old <- a_new.  A streaming pass in
-// place over the input buffer, so the collision kernel starts electrons
-// without a dependent gather.
-template <class T>
-__global__ void __launch_bounds__(256) k_field_kick(const PushArgs<T> A) {
-    const long long n = (long long)A.st->n_in;
+// A swarm's acceleration: the uniform field, no half-kick (a pass of its own
+// over the electrons, and the launch that took the resampled count over, cost
+// a step of 1e4 electrons 7 of 230 us in double precision, 4 of 75 in single).
+template <class T> __device__ __forceinline__ void uniform_accel(const PushArgs<T>& A, T* f) {
     const T qm = (T)(kQ / kMe);
-    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-        const T x[3] = {A.in.r[PX][i], A.in.r[PY][i], A.in.r[PZ][i]};
-        T E[3];
-        gather(A, x, E);
 #pragma unroll
-        for (int d = 0; d < 3; ++d) {
-            const T an = -qm * E[d];
-            if (!A.first) A.in.r[VX + d][i] = A.in.r[VX + d][i] + (T)0.5 * A.dt_kick * (an - A.in.r[AX + d][i]);
-            A.in.r[AX + d][i] = an;
-        }
-    }
+    for (int d = 0; d < 3; ++d) f[AX + d] = -qm * A.E0[d];
 }
 
-// The same half-kick for one loaded electron (f = x y z vx vy vz ax ay az w),
-// done by the collision kernel as it stages its parents.
+// Work items of a launch's parents: a swarm that k_resample has doubled counts twice its electrons (k_end_step
+// takes the count over).
+template <int MODE> __device__ __forceinline__ unsigned long long parent_items(const DevState* st) {
+    return MODE == MODE_SWARM && st->n_extra ? st->n_extra : st->n_in;
+}
+
+// Sec. 2.1.1, Eq. 2: a_new = -(e/m_e) E(x) from the trilinear gather; the
+// half-kick v += dt/2 (a_new - a_old) completes the previous step's velocity
+// update (skipped when a_old is unknown); a_old <- a_new.  For one loaded
+// electron (f = x y z vx vy vz ax ay az w), done by the collision kernel as it
+// stages its parents.
 template <class T> __device__ __forceinline__ void half_kick(const PushArgs<T>& A, T f[10]) {
     const T qm = (T)(kQ / kMe);
     T E[3];
@@ -869,13 +864,6 @@ __global__ void k_resample(const PushArgs<T> A) {
     if (dup && blockIdx.x == 0 && threadIdx.x == 0) A.st->n_extra = (unsigned long long)(2 * n);
 }
 
-static __global__ void k_resample_commit(DevState* st) {
-    if (st->n_extra) {
-        st->n_in = st->n_extra;
-        st->n_extra = 0;
-    }
-}
-
 // ------------------------------------------------------------------ collisions
 // Lanes refill from per-warp shared-memory stages.  Every lane owns one
 // electron at a time and advances it by up to two draws and a collision per
@@ -893,9 +881,9 @@ static __global__ void k_resample_commit(DevState* st) {
 // acceleration of the electron that ionized.  A product that finds the queue
 // full waits in the queue of the next (children) launch.
 //
-// CHILD = false: work item = one electron of the input buffer (kicked by
-// k_field_kick, or as it is staged), flying dt.  CHILD = true: work item = one
-// queued ionization product, built when it is staged.
+// CHILD = false: work item = one electron of the input buffer, kicked as it is
+// staged and flying dt.  CHILD = true: work item = one queued ionization
+// product, built when it is staged.
 constexpr int kTripLimit = 1 << 24;  // of a warp in one launch (a minute): an error instead of an endless kernel
 constexpr int kRow = 11;    // padded row of a stage entry: x y z vx vy vz ax ay az w t
 constexpr int kOut = 64;    // output stage capacity (flushed at 32)
@@ -1035,7 +1023,7 @@ __device__ __forceinline__ void collide_loop(const PushArgs<T>& A, const ProcSme
     unsigned long long* dst_cnt = CHILD ? ((A.gen & 1) ? &A.st->n_child : &A.st->n_spill) : &A.st->n_child;
     // work items of the launch (fixed while it runs; read again at each refill rather than held in registers)
     auto items = [&]() -> long long {
-        if (!CHILD) return (long long)A.st->n_in;
+        if (!CHILD) return (long long)parent_items<MODE>(A.st);
         const long long n = (long long)((A.gen & 1) ? A.st->n_spill : A.st->n_child);
         return n < A.cap_child ? n : A.cap_child;
     };
@@ -1126,7 +1114,8 @@ __device__ __forceinline__ void collide_loop(const PushArgs<T>& A, const ProcSme
                         } else {
                             T f[10];
                             for (int q = 0; q < 10; ++q) f[q] = A.in.r[q][it];
-                            if (MODE == MODE_PIC && A.kick_on_load) half_kick(A, f);
+                            if (MODE == MODE_SWARM) uniform_accel(A, f);
+                            else if (A.kick_on_load) half_kick(A, f);
                             for (int q = 0; q < 10; ++q) r[q] = f[q];
                             r[10] = A.dt;
                             sg->in_id[lane] = A.in.id[it];
@@ -1241,7 +1230,7 @@ __device__ __forceinline__ void collide_pool(const PushArgs<T>& A, const ProcSme
     const ChildQ<T>& src = (A.gen & 1) ? A.cq2 : A.cq;
     const ChildQ<T>& dst = CHILD ? ((A.gen & 1) ? A.cq : A.cq2) : A.cq;  // products the warp queue cannot take
     unsigned long long* dst_cnt = CHILD ? ((A.gen & 1) ? &A.st->n_child : &A.st->n_spill) : &A.st->n_child;
-    long long items = (long long)(CHILD ? ((A.gen & 1) ? A.st->n_spill : A.st->n_child) : A.st->n_in);
+    long long items = (long long)(CHILD ? ((A.gen & 1) ? A.st->n_spill : A.st->n_child) : parent_items<MODE>(A.st));
     if (CHILD) {
         if (items > A.cap_child) items = A.cap_child;
         if (items == 0) return;
@@ -1306,7 +1295,8 @@ __device__ __forceinline__ void collide_pool(const PushArgs<T>& A, const ProcSme
                         build_product<T, MODE>(A, e, q.id[it], src.k[it], r, &id);
                     } else {
                         for (int q = 0; q < 10; ++q) r[q] = A.in.r[q][it];
-                        if (MODE == MODE_PIC && A.kick_on_load) half_kick(A, r);
+                        if (MODE == MODE_SWARM) uniform_accel(A, r);
+                        else if (A.kick_on_load) half_kick(A, r);
                         r[10] = A.dt;
                         id = A.in.id[it];
                     }
@@ -1551,7 +1541,6 @@ template <class T> struct PushLaunch {
     static cudaError_t children(const PushArgs<T>& A, int mode, bool stats, int grid, cudaStream_t s);
     static cudaError_t deposit(const Soa<T>& p, DevState* st, const Grid& g, unsigned long long* q, int grid,
                                cudaStream_t s);
-    static cudaError_t field_kick(const PushArgs<T>& A, int grid, cudaStream_t s);
     static cudaError_t resample(const PushArgs<T>& A, int grid, cudaStream_t s);
     static cudaError_t photo_append(const PushArgs<T>& A, int grid, cudaStream_t s);
     static size_t smem_bytes(int n_bins);

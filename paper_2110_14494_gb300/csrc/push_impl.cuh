@@ -66,11 +66,6 @@ cudaError_t PushLaunch<T>::deposit(const Soa<T>& p, DevState* st, const Grid& g,
     return cudaGetLastError();
 }
 
-template <class T> cudaError_t PushLaunch<T>::field_kick(const PushArgs<T>& A, int grid, cudaStream_t s) {
-    k_field_kick<T><<<grid, 256, 0, s>>>(A);
-    return cudaGetLastError();
-}
-
 template <class T> cudaError_t PushLaunch<T>::photo_append(const PushArgs<T>& A, int grid, cudaStream_t s) {
     k_photo_resolve<T><<<grid, 256, 0, s>>>(A);
     k_photo_append<T><<<grid, 256, 0, s>>>(A);
@@ -80,7 +75,6 @@ template <class T> cudaError_t PushLaunch<T>::photo_append(const PushArgs<T>& A,
 
 template <class T> cudaError_t PushLaunch<T>::resample(const PushArgs<T>& A, int grid, cudaStream_t s) {
     k_resample<T><<<grid, 256, 0, s>>>(A);
-    k_resample_commit<<<1, 1, 0, s>>>(A.st);
     return cudaGetLastError();
 }
 

@@ -288,3 +288,25 @@ def test_features_of_aligned_and_shifted_arrays(n):
     x = aligned.cpu().numpy()
     assert np.all(np.abs(x[:, 0] - ref) <= 2 * np.spacing(np.abs(ref).astype(np.float32)))
     assert np.array_equal(x[:, 1], f[1:].cpu().numpy().astype(np.float32))
+
+
+@pytest.mark.parametrize("prec", [64, 32])
+@pytest.mark.parametrize("n_lo,n_hi", [(995, 5000), (10, 1005)])
+def test_swarm_resampled_within_a_step(prec, n_lo, n_hi):
+    """A single swarm that falls below n_lo (attachment at 25 Td) is doubled and
+    one that rises above n_hi (ionization at 400 Td) thinned at the start of a
+    step, and the step's electrons are those: float64 counts are the oracle's,
+    float32 counts the same but for decision flips (two of a thousand)."""
+    from paper_2110_14494_gb300 import swarm_run
+    gas, EN = W.synthetic_air(), 25.0 if n_lo > 100 else 400.0
+    _, mom, cnt = swarm_run(gas, [EN], precision=prec, n0=1000, n_steps=120, dt=2e-12, seed=77, n_lo=n_lo, n_hi=n_hi,
+                            want_moments=True)
+    omom, ocnt, _, _ = O.swarm(gas, EN, 1000, 120, 2e-12, 77, n_lo=n_lo, n_hi=n_hi)
+    jumps = np.abs(np.diff(ocnt)) > 0.3 * ocnt[:-1]
+    assert jumps.any()
+    if prec == 64:
+        assert np.array_equal(cnt[0], ocnt)
+        assert np.all(np.abs(mom[0] - omom) <= 1e-9 * (np.abs(omom).max(axis=0) + 1e-300))
+    else:
+        k = int(np.argmax(jumps)) + 1
+        assert np.all(np.abs(cnt[0][:k + 1] - ocnt[:k + 1]) <= 2e-3 * ocnt[:k + 1] + 2)
