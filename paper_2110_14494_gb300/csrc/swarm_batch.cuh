@@ -269,6 +269,53 @@ template <class T> struct BatchStage {
     int macc_s;
 };
 
+// a + b and its exact error (Knuth).
+__device__ __forceinline__ void sum_err(float a, float b, float& s, float& e) {
+    s = __fadd_rn(a, b);
+    const float bb = __fsub_rn(s, a);
+    e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb));
+}
+// Sums over the lanes of 14 values (all lanes call; v is overwritten), halved
+// between partners on the way (15 exchanges in place of 70); single precision
+// carries each addition's error along, so the sums of a flush are exact to
+// 2^-45 whichever electrons share it.  Lane l gets the sum of value
+// sum14_index(l).
+template <class T> __device__ __forceinline__ double sum14(T (&v)[14]) {
+    const int lane = threadIdx.x & 31;
+    T h[8], l[8];
+#pragma unroll
+    for (int j = 0; j < 7; ++j) {
+        const T keep = lane & 16 ? v[7 + j] : v[j], got = __shfl_xor_sync(kFull, lane & 16 ? v[j] : v[7 + j], 16);
+        if constexpr (sizeof(T) == 4) sum_err(keep, got, h[j], l[j]);
+        else h[j] = keep + got;
+    }
+    h[7] = l[7] = (T)0;
+#pragma unroll
+    for (int w = 4; w > 0; w >>= 1) {
+        const bool up = (lane & (2 * w)) != 0;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            if (j >= w) break;
+            const T kh = up ? h[w + j] : h[j], gh = __shfl_xor_sync(kFull, up ? h[j] : h[w + j], 2 * w);
+            if constexpr (sizeof(T) == 4) {
+                const T kl = up ? l[w + j] : l[j], gl = __shfl_xor_sync(kFull, up ? l[j] : l[w + j], 2 * w);
+                T e;
+                sum_err(kh, gh, h[j], e);
+                l[j] = (kl + gl) + e;
+            } else {
+                h[j] = kh + gh;
+            }
+        }
+    }
+    const T gh = __shfl_xor_sync(kFull, h[0], 1);
+    if constexpr (sizeof(T) == 4) return ((double)h[0] + (double)gh) + (double)(l[0] + __shfl_xor_sync(kFull, l[0], 1));
+    else return h[0] + gh;
+}
+__device__ __forceinline__ int sum14_index(int lane) {  // 14 and more: none
+    const int q = (lane >> 1) & 7, at = (lane & 8 ? 4 : 0) + (lane & 4 ? 2 : 0) + (lane & 2 ? 1 : 0);
+    return (lane & 1) || q == 7 ? 14 : (lane >> 4) * 7 + at;
+}
+
 // Moment contributions of the lanes' electrons (all lanes call).  When all
 // 32 lanes carry electrons of one swarm (the common case: items are
 // contiguous per swarm) the warp reduces them and keeps the running sums in
@@ -312,26 +359,19 @@ __device__ __forceinline__ void swarm_moments(const BatchArgs<T>& B, BatchStage<
         todo &= ~__ballot_sync(kFull, mine);
         T red[14];
 #pragma unroll
-        for (int q = 0; q < 14; ++q) {
-            T v2 = mine ? m[q] : (T)0;
-            for (int o = 16; o > 0; o >>= 1) v2 += __shfl_xor_sync(kFull, v2, o);
-            red[q] = v2;
-        }
+        for (int q = 0; q < 14; ++q) red[q] = mine ? m[q] : (T)0;
+        const double add = sum14(red);
         if (sg->macc_s != sg_s && (sg->macc_s < 0 || todo == 0)) {
             // the warp has moved on to another swarm: write the old sums out
             macc_flush(B, sg, step);
             if ((threadIdx.x & 31) == 0) sg->macc_s = sg_s;
             __syncwarp();
         }
-        const int lane = threadIdx.x & 31;
-        T mine_sum = (T)0;
-#pragma unroll
-        for (int k = 0; k < 14; ++k) mine_sum = k == lane ? red[k] : mine_sum;
-        const double add = (double)mine_sum;
+        const int at = sum14_index(threadIdx.x & 31);
         if (sg->macc_s == sg_s) {
-            if (lane < 14) sg->macc[lane] += add;
-        } else if (lane < 14 && add != 0.0) {
-            atomicAdd(B.mom + ((size_t)sg_s * B.n_steps + (step - 1)) * kNMom + lane, add);
+            if (at < 14) sg->macc[at] += add;
+        } else if (at < 14 && add != 0.0) {
+            atomicAdd(B.mom + ((size_t)sg_s * B.n_steps + (step - 1)) * kNMom + at, add);
         }
         __syncwarp();
     }
