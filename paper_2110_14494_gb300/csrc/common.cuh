@@ -20,6 +20,10 @@ constexpr int kMaxProc = PIC_MAX_PROC;
 // (8 KB of single precision for 1000 nodes, all of it in L1), only a draw that
 // may collide the two rows around its energy, 64 consecutive bytes.
 constexpr int kTableRow = 8, kTableStride = kTableRow + 2;  // kTableStride: reals per node in all
+// Reals from one table to the next in a batch.  Rows are read 16 bytes at a
+// time, so every table begins on a multiple of 16 bytes: with single
+// precision's 40 bytes a node that takes a rounding for odd n_bins.
+__host__ __device__ constexpr size_t table_reals(int n_bins) { return ((size_t)n_bins * kTableStride + 3) & ~(size_t)3; }
 constexpr int kNMom = PIC_SWARM_NMOM;
 constexpr unsigned kFull = 0xffffffffu;
 constexpr double kPi = 3.14159265358979323846;

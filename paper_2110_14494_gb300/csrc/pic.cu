@@ -141,7 +141,7 @@ __global__ void k_rate_table(const double* __restrict__ eps, const double* __res
     const int j = blockIdx.x * blockDim.x + threadIdx.x;
     if (j >= n_bins) return;
     dens += (size_t)blockIdx.y * n_proc;
-    tab += (size_t)blockIdx.y * n_bins * kTableStride;
+    tab += blockIdx.y * table_reals(n_bins);
     const int j1 = j + 1 < n_bins ? j + 1 : j;
     const double v = sqrt(2.0 * kQ * eps[j] / kMe), v1 = sqrt(2.0 * kQ * eps[j1] / kMe);
     double tot = 0.0, tot1 = 0.0;
@@ -1005,7 +1005,7 @@ static Layout make_layout(const pic_config* c) {
         take(cap * 4);                               // draw index of the ionization
     }
     const int nb = c->gas.n_bins > 0 ? c->gas.n_bins : 2;
-    L.table = take((size_t)nb * kTableStride * R);
+    L.table = take(table_reals(nb) * R);
     L.E4 = take(ncell * 4 * R);
     // float32 Cartesian coupled contexts alternate between two packed fields
     // (the solve writes the one the current push does not read)
@@ -2449,7 +2449,7 @@ static BatchLayout batch_layout(const swarm_config* sc, int n) {
     L.zref = take((size_t)n * 8);
     L.zhist = take((size_t)n * sc->n_steps * 8);
     const int nb = sc->gas.n_bins, np = sc->gas.n_proc > 0 ? sc->gas.n_proc : 1;
-    L.tabs = take((size_t)n * nb * kTableStride * R);
+    L.tabs = take((size_t)n * table_reals(nb) * R);
     L.numax = take((size_t)n * R);
     L.tau = take((size_t)n * R);
     L.dens = take((size_t)n * np * 8);
@@ -2646,7 +2646,7 @@ template <class T> struct BatchRunner {
         if (e == cudaSuccess) e = cudaStreamSynchronize(s);
         if (e != cudaSuccess) return PIC_ERR_CUDA;
         B.tab_s = tabs;
-        B.tab_stride = (long long)nb * kTableStride;
+        B.tab_stride = (long long)table_reals(nb);
         B.numax_s = (const T*)(ws + L.numax);
         B.tau_s = (const T*)(ws + L.tau);
         return PIC_OK;

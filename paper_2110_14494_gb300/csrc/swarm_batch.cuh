@@ -53,7 +53,7 @@ template <class T> struct BatchArgs {
     long long n_lo, n_hi;
     int gen;
     // collision rates of each swarm's gas: table of swarm s at tab_s + s *
-    // tab_stride (stride 0: one gas for all), nu_max and its flight_scale
+    // tab_stride (table_reals), nu_max and its flight_scale
     const T* tab_s;
     long long tab_stride;
     const T* numax_s;

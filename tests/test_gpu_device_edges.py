@@ -310,3 +310,25 @@ def test_swarm_resampled_within_a_step(prec, n_lo, n_hi):
     else:
         k = int(np.argmax(jumps)) + 1
         assert np.all(np.abs(cnt[0][:k + 1] - ocnt[:k + 1]) <= 2e-3 * ocnt[:k + 1] + 2)
+
+
+@pytest.mark.parametrize("launch", [1, 2])
+@pytest.mark.parametrize("prec", [64, 32])
+@pytest.mark.parametrize("n_bins", [3, 11, 1001])
+def test_batched_tables_of_odd_length(n_bins, prec, launch):
+    """Gas tables with an odd number of nodes, three swarms (the second table
+    begins 40 n_bins bytes after the first in float32, 8 modulo 16 unless the
+    stride is rounded up).  Float64 counts are the oracle's; in float32 a
+    rounding turns about 1e-6 of the decisions, some 10 draws a picosecond for
+    20 ps: 2e-4 of the electrons; at most two in a thousand and two here."""
+    from paper_2110_14494_gb300 import swarm_run
+    gas, seed, ENs = W.synthetic_air(n_bins=n_bins), 91, [150.0, 250.0, 120.0]
+    _, mom, cnt = swarm_run(gas, ENs, precision=prec, n0=1000, n_steps=20, dt=1e-12, seed=seed, n_lo=10, n_hi=100000,
+                            want_moments=True, batched=True, block=128, blocks_per_sm=1, use_graph=launch)
+    for s, EN in enumerate(ENs):
+        omom, ocnt, _, _ = O.swarm(gas, EN, 1000, 20, 1e-12, seed + s, n_lo=10, n_hi=100000)
+        if prec == 64:
+            assert np.array_equal(cnt[s], ocnt), s
+            assert np.all(np.abs(mom[s] - omom) <= 1e-9 * (np.abs(omom).max(axis=0) + 1e-300)), s
+        else:
+            assert np.all(np.abs(cnt[s] - ocnt) <= 2e-3 * ocnt + 2), s
