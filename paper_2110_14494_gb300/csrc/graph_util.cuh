@@ -12,8 +12,10 @@ namespace pic {
 // its first access.  Without the launch attribute the wait returns at once.
 __device__ __forceinline__ void pdl_wait() { cudaGridDependencySynchronize(); }
 
+// A launch's error is its return value: a later call that succeeds can reset
+// the last error, so callers keep what this returns.
 template <class... P, class... A>
-void launch_pdl(void (*k)(P...), dim3 g, dim3 b, size_t smem, cudaStream_t s, A... args) {
+cudaError_t launch_pdl(void (*k)(P...), dim3 g, dim3 b, size_t smem, cudaStream_t s, A... args) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = g;
     cfg.blockDim = b;
@@ -24,8 +26,22 @@ void launch_pdl(void (*k)(P...), dim3 g, dim3 b, size_t smem, cudaStream_t s, A.
     at[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = at;
     cfg.numAttrs = 1;
-    cudaLaunchKernelEx(&cfg, k, args...);
+    return cudaLaunchKernelEx(&cfg, k, args...);
 }
+
+// First error of a sequence of launches; launched() reports and clears it.
+struct LaunchStatus {
+    cudaError_t launch_err = cudaSuccess;
+    void note(cudaError_t e) {
+        if (launch_err == cudaSuccess) launch_err = e;
+    }
+    bool launched() {
+        const bool ok = launch_err == cudaSuccess;
+        if (!ok) cudaGetLastError();
+        launch_err = cudaSuccess;
+        return ok;
+    }
+};
 
 __device__ __forceinline__ void bar_named(int id, int threads) {
     asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(threads) : "memory");

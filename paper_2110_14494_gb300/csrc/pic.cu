@@ -2744,7 +2744,7 @@ template <class T> struct BatchRunner {
     }
 
     int run_steps(int steps, int block, int grid, bool graph) {
-        if (BatchLaunch<T>::prepare(block) != cudaSuccess) return PIC_ERR_CUDA;
+        if (BatchLaunch<T>::prepare() != cudaSuccess) return PIC_ERR_CUDA;
         BatchArgs<T> Bo = B;
         std::swap(Bo.in, Bo.out);
         if (!graph) {
@@ -2807,7 +2807,7 @@ template <class T> struct BatchRunner {
         long long bc = kWarpChunk;
         int rc = PIC_OK;
         for (int block : {64, 128, 256}) {
-            if (BatchLaunch<T>::prepare(block) != cudaSuccess) continue;
+            if (BatchLaunch<T>::prepare() != cudaSuccess) continue;
             const int maxb = BatchLaunch<T>::max_blocks_per_sm(block);
             for (int bps : {1, 2, 3, 4, maxb}) {
                 if (bps > maxb) continue;

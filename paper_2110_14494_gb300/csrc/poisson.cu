@@ -380,6 +380,7 @@ struct TailSmem {
     float* rdiag;  // [16]: inv_diag(d) for the integer diagonals d = 0..15
 };
 __host__ __device__ constexpr size_t tail_smem_bytes(int cells) { return (((size_t)cells * (2 * sizeof(float) + 1) + 15) & ~(size_t)15) + 16 * sizeof(float); }
+constexpr int kTailMaxCells = 200 * 1024 / 9;  // of its levels together: e, g and mask in shared memory
 
 // Thread decomposition of a phase: thread owns (tx + a sx, ty + b sy, tz + c sz).
 struct Dec {
@@ -593,17 +594,15 @@ dim3 grid_pair(int nx, int ny, int nz, int zs) {
     return dim3((nx / 2 + BX - 1) / BX, (ny + SY - 1) / SY, (nz + zs - 1) / zs);
 }
 const dim3 kPairBlk(BX, SY + 2, 1);
-void smooth_half(float* e, const float* g, const uint8_t* m, int nx, int ny, int nz, int color, cudaStream_t s) {
+cudaError_t smooth_half(float* e, const float* g, const uint8_t* m, int nx, int ny, int nz, int color, cudaStream_t s) {
     if ((long long)nx * ny * nz >= kSmoothDeep)
-        launch_pdl(k_smooth_pair<4>, grid_pair(nx, ny, nz, 4), kPairBlk, 0, s, e, g, m, nx, ny, nz, color);
-    else
-        launch_pdl(k_smooth, grid3((nx + 1) / 2, ny, nz), kBlk, 0, s, e, g, m, nx, ny, nz, color);
+        return launch_pdl(k_smooth_pair<4>, grid_pair(nx, ny, nz, 4), kPairBlk, 0, s, e, g, m, nx, ny, nz, color);
+    return launch_pdl(k_smooth, grid3((nx + 1) / 2, ny, nz), kBlk, 0, s, e, g, m, nx, ny, nz, color);
 }
-void sweep_first(float* e, const float* g, const uint8_t* m, int nx, int ny, int nz, cudaStream_t s) {
+cudaError_t sweep_first(float* e, const float* g, const uint8_t* m, int nx, int ny, int nz, cudaStream_t s) {
     if ((long long)nx * ny * nz >= kSmoothDeep)
-        launch_pdl(k_sweep_first<4>, grid_pair(nx, ny, nz, 4), kPairBlk, 0, s, e, g, m, nx, ny, nz);
-    else
-        launch_pdl(k_sweep_first<1>, grid_pair(nx, ny, nz, 1), kPairBlk, 0, s, e, g, m, nx, ny, nz);
+        return launch_pdl(k_sweep_first<4>, grid_pair(nx, ny, nz, 4), kPairBlk, 0, s, e, g, m, nx, ny, nz);
+    return launch_pdl(k_sweep_first<1>, grid_pair(nx, ny, nz, 1), kPairBlk, 0, s, e, g, m, nx, ny, nz);
 }
 dim3 grid_mx3(int nx, int ny, int nz) { return dim3((nx + BX - 1) / BX, (ny + BY - 1) / BY, (nz + ZC - 1) / ZC); }
 
@@ -633,7 +632,7 @@ bool MG::supported(int nx_, int ny_, int nz_) {
     MG m;
     m.plan(nx_, ny_, nz_);
     const int L = m.levels - 1;
-    return (long long)m.lx[L] * m.ly[L] * m.lz[L] * 9 <= 200 * 1024;
+    return (long long)m.lx[L] * m.ly[L] * m.lz[L] <= kTailMaxCells;
 }
 
 size_t MG::bytes(int nx_, int ny_, int nz_, bool mixed_, bool pair_copy, bool lean) {
@@ -707,7 +706,7 @@ int MG::tail_level() const {
     while (t < levels - 1) {
         long long cells = 0;
         for (int l = t; l < levels; ++l) cells += (long long)lx[l] * ly[l] * lz[l];
-        if (cells * 9 <= 200 * 1024) break;
+        if (cells <= kTailMaxCells) break;
         ++t;
     }
     return t;
@@ -768,9 +767,11 @@ void MG::tail(cudaStream_t s, int pre, int post) {
         T.post = post;
         T.coarse = coarse_sweeps;
         const size_t smem = (size_t)T.words * 4;
+        // The limit belongs to the kernel, not to this launch: it is the same for every hierarchy, since a smaller
+        // one would fail the launches of other threads.
         auto go = [&](void (*k)(TailPlan)) {
-            if (smem > 48 * 1024) cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-            launch_pdl(k, dim3(1), dim3(T.L[0].act), smem, s, T);
+            if (smem > 48 * 1024) note(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTailSmem));
+            note(launch_pdl(k, dim3(1), dim3(T.L[0].act), smem, s, T));
         };
         const int per = (T.L[0].h + T.L[0].act - 1) / T.L[0].act;
         if (per == 1) go(k_tail_cycle<1>);
@@ -797,8 +798,10 @@ void MG::tail(cudaStream_t s, int pre, int post) {
     T.coarse = coarse_sweeps;
     T.total = off;
     const size_t smem = tail_smem_bytes(off);
-    if (smem > 48 * 1024) cudaFuncSetAttribute(k_tail_vcycle, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    launch_pdl(k_tail_vcycle, dim3(1), dim3(1024), smem, s, T);
+    if (smem > 48 * 1024)
+        note(cudaFuncSetAttribute(k_tail_vcycle, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                  (int)tail_smem_bytes(kTailMaxCells)));
+    note(launch_pdl(k_tail_vcycle, dim3(1), dim3(1024), smem, s, T));
 }
 
 // One V(pre, post)-cycle on A e0 = g0 (light: V(light_pre, light_post)); e0 is overwritten.  Levels above the
@@ -812,25 +815,25 @@ void MG::vcycle(cudaStream_t s, bool light) {
     for (int l = 0; l < t; ++l) {
         const long long n = (long long)lx[l] * ly[l] * lz[l];
         if (pre > 0) {
-            sweep_first(e[l], g[l], m[l], lx[l], ly[l], lz[l], s);
+            note(sweep_first(e[l], g[l], m[l], lx[l], ly[l], lz[l], s));
         } else {
             cudaMemsetAsync(e[l], 0, n * sizeof(float), s);
         }
         for (int it = 1; it < pre; ++it) {
-            smooth_half(e[l], g[l], m[l], lx[l], ly[l], lz[l], 0, s);
-            smooth_half(e[l], g[l], m[l], lx[l], ly[l], lz[l], 1, s);
+            note(smooth_half(e[l], g[l], m[l], lx[l], ly[l], lz[l], 0, s));
+            note(smooth_half(e[l], g[l], m[l], lx[l], ly[l], lz[l], 1, s));
         }
-        launch_pdl(k_resid_restrict, grid3(lx[l + 1], ly[l + 1], lz[l + 1]), kBlk, 0, s, (const float*)e[l],
-                   (const float*)g[l], (const uint8_t*)m[l], lx[l], ly[l], lz[l], g[l + 1], (const uint8_t*)m[l + 1],
-                   pre > 0 ? 1 : 0);
+        note(launch_pdl(k_resid_restrict, grid3(lx[l + 1], ly[l + 1], lz[l + 1]), kBlk, 0, s, (const float*)e[l],
+                        (const float*)g[l], (const uint8_t*)m[l], lx[l], ly[l], lz[l], g[l + 1],
+                        (const uint8_t*)m[l + 1], pre > 0 ? 1 : 0));
     }
     tail(s, pre, post);
     for (int l = t - 1; l >= 0; --l) {
-        launch_pdl(k_prolong_add, grid3(lx[l + 1], ly[l + 1], lz[l + 1]), kBlk, 0, s, (const float*)e[l + 1], e[l],
-                   (const uint8_t*)m[l], lx[l], ly[l], lz[l]);
+        note(launch_pdl(k_prolong_add, grid3(lx[l + 1], ly[l + 1], lz[l + 1]), kBlk, 0, s, (const float*)e[l + 1], e[l],
+                        (const uint8_t*)m[l], lx[l], ly[l], lz[l]));
         for (int it = 0; it < post; ++it) {
-            smooth_half(e[l], g[l], m[l], lx[l], ly[l], lz[l], 1, s);
-            smooth_half(e[l], g[l], m[l], lx[l], ly[l], lz[l], 0, s);
+            note(smooth_half(e[l], g[l], m[l], lx[l], ly[l], lz[l], 1, s));
+            note(smooth_half(e[l], g[l], m[l], lx[l], ly[l], lz[l], 0, s));
         }
     }
 }
@@ -841,10 +844,10 @@ void MG::iteration(cudaStream_t s, double* phi, const uint8_t* mk, bool first) {
     const int nx = lx[0], ny = ly[0], nz = lz[0];
     const int f = first ? 1 : 0;
     vcycle(s, false);
-    launch_pdl(k_apply64, grid_mx3(nx, ny, nz), kBlk, 0, s, (const float*)e[0], (const double*)r64, (const double*)q64,
-               w64, mk, nx, ny, nz, f, part, ctr + 1, norms);
-    launch_pdl(k_step64, grid_mx3(nx, ny, nz), kBlk, 0, s, (const float*)e[0], (const double*)w64, mk, p64, q64, phi,
-               r64, g[0], nx, ny, nz, f, part, ctr + 2, norms);
+    note(launch_pdl(k_apply64, grid_mx3(nx, ny, nz), kBlk, 0, s, (const float*)e[0], (const double*)r64,
+                    (const double*)q64, w64, mk, nx, ny, nz, f, part, ctr + 1, norms));
+    note(launch_pdl(k_step64, grid_mx3(nx, ny, nz), kBlk, 0, s, (const float*)e[0], (const double*)w64, mk, p64, q64, phi,
+                    r64, g[0], nx, ny, nz, f, part, ctr + 2, norms));
     launches += 2;
 }
 
@@ -899,7 +902,10 @@ int MG::solve(const double* rho, const uint8_t* mask, double* phi, double h, dou
                     return PIC_ERR_CUDA;
                 iteration(cap_stream, phi, mk, cyc == 0);
                 if (cudaStreamEndCapture(cap_stream, &gr) != cudaSuccess) return PIC_ERR_CUDA;
-                if (cudaGraphInstantiate(&g_iter[gi], gr, 0) != cudaSuccess) { cudaGraphDestroy(gr); return PIC_ERR_CUDA; }
+                if (!launched() || cudaGraphInstantiate(&g_iter[gi], gr, 0) != cudaSuccess) {
+                    cudaGraphDestroy(gr);
+                    return PIC_ERR_CUDA;
+                }
                 cudaGraphDestroy(gr);
                 graph_kernels[gi] = launches - l0;
                 launches = l0;
@@ -908,6 +914,7 @@ int MG::solve(const double* rho, const uint8_t* mask, double* phi, double h, dou
             launches += graph_kernels[gi];
         } else {
             iteration(s, phi, mk, cyc == 0);
+            if (!launched()) return PIC_ERR_CUDA;
         }
         ++cyc;
     }
@@ -957,13 +964,13 @@ void MG::iteration_mixed(cudaStream_t s, int it, bool light) {
     // w = A z goes to p32[cur] (the direction of two iterations ago, free
     // here), where the second kernel replaces it by the new direction
     if (nx % 4 == 0)
-        launch_pdl(k_mx_apply4, grid_mx3v(nx, ny, nz), kBlk, 0, s, (const float*)e[0], (const float*)g[0],
-                   (const float*)q32, p32[cur], (const uint8_t*)m[0], nx, ny, nz, first, part, ctr + 1, norms);
+        note(launch_pdl(k_mx_apply4, grid_mx3v(nx, ny, nz), kBlk, 0, s, (const float*)e[0], (const float*)g[0],
+                        (const float*)q32, p32[cur], (const uint8_t*)m[0], nx, ny, nz, first, part, ctr + 1, norms));
     else
-        launch_pdl(k_mx_apply, grid_mx3(nx, ny, nz), kBlk, 0, s, (const float*)e[0], (const float*)g[0],
-                   (const float*)q32, p32[cur], (const uint8_t*)m[0], nx, ny, nz, first, part, ctr + 1, norms);
-    launch_pdl(k_mx_step, grid_mxf(n), dim3(kFlatBlock), 0, s, (const float*)e[0], (const float*)p32[cur ^ 1],
-               p32[cur], q32, d32, g[0], n, first, part, ctr + 3, norms);
+        note(launch_pdl(k_mx_apply, grid_mx3(nx, ny, nz), kBlk, 0, s, (const float*)e[0], (const float*)g[0],
+                        (const float*)q32, p32[cur], (const uint8_t*)m[0], nx, ny, nz, first, part, ctr + 1, norms));
+    note(launch_pdl(k_mx_step, grid_mxf(n), dim3(kFlatBlock), 0, s, (const float*)e[0], (const float*)p32[cur ^ 1],
+                    p32[cur], q32, d32, g[0], n, first, part, ctr + 3, norms));
     launches += 2;
 }
 
@@ -1038,7 +1045,10 @@ int MG::solve_mixed(const void* rho, bool rho64, const uint8_t* mask, float* phi
                     return PIC_ERR_CUDA;
                 iteration_mixed(cap_stream, it, light);
                 if (cudaStreamEndCapture(cap_stream, &gr) != cudaSuccess) return PIC_ERR_CUDA;
-                if (cudaGraphInstantiate(&g_mx[gi], gr, 0) != cudaSuccess) { cudaGraphDestroy(gr); return PIC_ERR_CUDA; }
+                if (!launched() || cudaGraphInstantiate(&g_mx[gi], gr, 0) != cudaSuccess) {
+                    cudaGraphDestroy(gr);
+                    return PIC_ERR_CUDA;
+                }
                 cudaGraphDestroy(gr);
                 graph_kernels_mx[gi] = launches - l0;
                 launches = l0;
@@ -1047,6 +1057,7 @@ int MG::solve_mixed(const void* rho, bool rho64, const uint8_t* mask, float* phi
             launches += graph_kernels_mx[gi];
         } else {
             iteration_mixed(s, it, light);
+            if (!launched()) return PIC_ERR_CUDA;
         }
         ++it;
         ++cyc;
@@ -1162,7 +1173,7 @@ int MG::capture_solve_mixed(cudaStream_t cs, const float* rho, float* phi_hi, fl
                                    nullptr, E4, loop);
     k_mx_report<<<1, 1, 0, cs>>>(loop, cycles_dst, rel_dst, err_dst, err_bit, kernels_dst, kb);
     if (fixed_kernels) *fixed_kernels = 3 + (min_c > 0 ? 2 : 0);  // residual, gradient, report, prime, check
-    return cudaGetLastError() == cudaSuccess ? PIC_OK : PIC_ERR_CUDA;
+    return launched() && cudaGetLastError() == cudaSuccess ? PIC_OK : PIC_ERR_CUDA;
 }
 
 }  // namespace pic

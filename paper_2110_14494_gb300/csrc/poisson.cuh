@@ -3,6 +3,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "graph_util.cuh"
+
 namespace pic {
 
 // State of the flexible-CG loop of a device-driven mixed solve (device
@@ -21,7 +23,7 @@ struct MxBranchKernels {
     int k[kMxBranches];  // kernels each branch runs
 };
 
-struct MG {
+struct MG : LaunchStatus {
     static constexpr int kMaxLevels = 12;
     int levels = 0;
     int lx[kMaxLevels], ly[kMaxLevels], lz[kMaxLevels];

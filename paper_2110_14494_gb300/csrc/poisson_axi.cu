@@ -700,14 +700,15 @@ int AxiMG::tail_level() const {
 void AxiMG::vcycle(cudaStream_t s) {
     const int tl = tail_level(), top = tl < levels ? tl : levels - 1;
     for (int l = 0; l < top; ++l) {
-        launch_pdl(deep(lr[l], lz[l]) ? k_axi_sweep_first<kRows> : k_axi_sweep_first<1>, agrid_half(lr[l], lz[l]), kABlk, 0, s, e[l], (const double*)g[l],
-                   (const uint8_t*)m[l], (const double*)rd[l], lr[l], lz[l]);
+        note(launch_pdl(deep(lr[l], lz[l]) ? k_axi_sweep_first<kRows> : k_axi_sweep_first<1>, agrid_half(lr[l], lz[l]),
+                        kABlk, 0, s, e[l], (const double*)g[l], (const uint8_t*)m[l], (const double*)rd[l], lr[l], lz[l]));
         for (int it = 1; it < pre; ++it)
             for (int col = 0; col < 2; ++col)
-                launch_pdl(deep(lr[l], lz[l]) ? k_axi_smooth<kRows> : k_axi_smooth<1>, agrid_half(lr[l], lz[l]), kABlk, 0, s, e[l], (const double*)g[l],
-                           (const uint8_t*)m[l], (const double*)rd[l], lr[l], lz[l], col);
-        launch_pdl(k_axi_resid_restrict, agrid(lr[l + 1], lz[l + 1]), kABlk, 0, s, (const double*)e[l],
-                   (const double*)g[l], (const uint8_t*)m[l], lr[l], lz[l], g[l + 1], (const uint8_t*)m[l + 1]);
+                note(launch_pdl(deep(lr[l], lz[l]) ? k_axi_smooth<kRows> : k_axi_smooth<1>, agrid_half(lr[l], lz[l]), kABlk,
+                                0, s, e[l], (const double*)g[l], (const uint8_t*)m[l], (const double*)rd[l], lr[l], lz[l],
+                                col));
+        note(launch_pdl(k_axi_resid_restrict, agrid(lr[l + 1], lz[l + 1]), kABlk, 0, s, (const double*)e[l],
+                        (const double*)g[l], (const uint8_t*)m[l], lr[l], lz[l], g[l + 1], (const uint8_t*)m[l + 1]));
     }
     if (tl < levels) {
         AxiTail T = {};
@@ -726,20 +727,20 @@ void AxiMG::vcycle(cudaStream_t s) {
         T.pre = pre;
         T.post = post;
         T.coarse = coarse_sweeps;
-        const size_t smem = (size_t)T.words * 8;
-        if (smem > 48 * 1024) cudaFuncSetAttribute(k_axi_tail, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        launch_pdl(k_axi_tail, dim3(1), dim3(T.L[0].act), smem, s, T);
+        // at most 31 KB (256 x 4 cells): no opt-in needed
+        note(launch_pdl(k_axi_tail, dim3(1), dim3(T.L[0].act), (size_t)T.words * 8, s, T));
     } else {
-        launch_pdl(k_axi_coarse, dim3(1), dim3(1024), 0, s, e[top], (const double*)g[top], (const uint8_t*)m[top],
-                   (const double*)rd[top], lr[top], lz[top], coarse_sweeps);
+        note(launch_pdl(k_axi_coarse, dim3(1), dim3(1024), 0, s, e[top], (const double*)g[top], (const uint8_t*)m[top],
+                        (const double*)rd[top], lr[top], lz[top], coarse_sweeps));
     }
     for (int l = top - 1; l >= 0; --l) {
-        launch_pdl(k_axi_prolong_add, agrid(lr[l + 1], lz[l + 1]), kABlk, 0, s, (const double*)e[l + 1], e[l],
-                   (const uint8_t*)m[l], lr[l], lz[l]);
+        note(launch_pdl(k_axi_prolong_add, agrid(lr[l + 1], lz[l + 1]), kABlk, 0, s, (const double*)e[l + 1], e[l],
+                        (const uint8_t*)m[l], lr[l], lz[l]));
         for (int it = 0; it < post; ++it)
             for (int col = 1; col >= 0; --col)
-                launch_pdl(deep(lr[l], lz[l]) ? k_axi_smooth<kRows> : k_axi_smooth<1>, agrid_half(lr[l], lz[l]), kABlk, 0, s, e[l], (const double*)g[l],
-                           (const uint8_t*)m[l], (const double*)rd[l], lr[l], lz[l], col);
+                note(launch_pdl(deep(lr[l], lz[l]) ? k_axi_smooth<kRows> : k_axi_smooth<1>, agrid_half(lr[l], lz[l]), kABlk,
+                                0, s, e[l], (const double*)g[l], (const uint8_t*)m[l], (const double*)rd[l], lr[l], lz[l],
+                                col));
     }
     launches += (long long)top * (2 * pre - 1 + 2 * post + 2) + 1;
 }
@@ -747,10 +748,10 @@ void AxiMG::vcycle(cudaStream_t s) {
 void AxiMG::iteration(cudaStream_t s, double* phi, bool first) {
     const int nr = lr[0], nz = lz[0], n = nr * nz, f = first ? 1 : 0;
     vcycle(s);
-    launch_pdl(k_axi_apply, agrid_rows(nr, nz), kABlk, 0, s, (const double*)e[0], (const double*)r, (const double*)q,
-               (const uint8_t*)m[0], nr, nz, w, f, part, ctr + 1, norms);
-    launch_pdl(k_axi_step, grid_step(n), kABlk, 0, s, (const double*)e[0], (const double*)w, p, q, phi, r, g[0], n, f,
-               part, ctr + 2, norms);
+    note(launch_pdl(k_axi_apply, agrid_rows(nr, nz), kABlk, 0, s, (const double*)e[0], (const double*)r, (const double*)q,
+                    (const uint8_t*)m[0], nr, nz, w, f, part, ctr + 1, norms));
+    note(launch_pdl(k_axi_step, grid_step(n), kABlk, 0, s, (const double*)e[0], (const double*)w, p, q, phi, r, g[0], n,
+                    f, part, ctr + 2, norms));
     launches += 2;
 }
 
@@ -789,6 +790,7 @@ int AxiMG::solve(const AxiCharge& rho, const uint8_t* mask, double* phi, double 
         if (rn / bn <= rtol) break;
         if (cyc >= max_cycles) { rc = PIC_ERR_TIMEOUT; break; }
         iteration(s, phi, cyc == 0);
+        if (!launched()) return PIC_ERR_CUDA;
         ++cyc;
     }
     if (cycles_out) *cycles_out = cyc;
@@ -915,7 +917,7 @@ int AxiMG::capture_solve(cudaStream_t cs, const AxiCharge& rho, double* phi, dou
     }
     k_axi_report<<<1, 1, 0, cs>>>(loop, cycles_dst, rel_dst, err_dst, err_bit, kernels_dst, kb[0], kb[1]);
     if (fixed_kernels) *fixed_kernels = fixed;
-    return cudaGetLastError() == cudaSuccess ? PIC_OK : PIC_ERR_CUDA;
+    return launched() && cudaGetLastError() == cudaSuccess ? PIC_OK : PIC_ERR_CUDA;
 }
 
 }  // namespace pic

@@ -3,6 +3,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "graph_util.cuh"
+
 namespace pic {
 
 // Right-hand side of a solve: rho in C/m^3, or (rho null) the fixed-point
@@ -21,7 +23,7 @@ struct AxiLoop {
     double rel;
 };
 
-struct AxiMG {
+struct AxiMG : LaunchStatus {
     static constexpr int kMaxLevels = 14;
     int levels = 0;
     int lr[kMaxLevels], lz[kMaxLevels];

@@ -81,7 +81,7 @@ template <class T> cudaError_t PushLaunch<T>::resample(const PushArgs<T>& A, int
 template <class T> int BatchLaunch<T>::max_blocks_per_sm(int block) {
     constexpr bool FAST = sizeof(T) == 4;
     const size_t sm = smem(block);
-    cudaFuncSetAttribute(k_batch_collide<T, FAST, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    cudaFuncSetAttribute(k_batch_collide<T, FAST, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem(kBatchBlock));
     int b = 0;
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_batch_collide<T, FAST, false>, block, sm);
     return b > 0 ? b : 1;
@@ -96,20 +96,20 @@ template <class T> cudaError_t BatchLaunch<T>::init(const BatchArgs<T>& B, long 
     return cudaGetLastError();
 }
 
-template <class T> cudaError_t BatchLaunch<T>::prepare(int block) {
+template <class T> cudaError_t BatchLaunch<T>::prepare() {
     constexpr bool FAST = sizeof(T) == 4;
-    const size_t sm = smem(block);
-    cudaError_t e = cudaFuncSetAttribute(k_batch_collide<T, FAST, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)sm);
+    const int sm = (int)smem(kBatchBlock);
+    cudaError_t e = cudaFuncSetAttribute(k_batch_collide<T, FAST, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
     if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(k_batch_collide<T, FAST, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+        e = cudaFuncSetAttribute(k_batch_collide<T, FAST, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
     return e;
 }
 
 template <class T> int BatchLaunch<T>::persistent_blocks_per_sm(int block) {
     constexpr bool FAST = sizeof(T) == 4;
     const size_t sm = smem(block);
-    if (cudaFuncSetAttribute(k_batch_run<T, FAST>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm) != cudaSuccess)
+    if (cudaFuncSetAttribute(k_batch_run<T, FAST>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem(kBatchBlock)) !=
+        cudaSuccess)
         return 0;
     int b = 0;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_batch_run<T, FAST>, block, sm) != cudaSuccess) return 0;
@@ -120,7 +120,8 @@ template <class T>
 cudaError_t BatchLaunch<T>::run_persistent(const BatchArgs<T>& B, int n_steps, int block, int grid, cudaStream_t s) {
     constexpr bool FAST = sizeof(T) == 4;
     const size_t sm = smem(block);
-    cudaError_t e = cudaFuncSetAttribute(k_batch_run<T, FAST>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    cudaError_t e = cudaFuncSetAttribute(k_batch_run<T, FAST>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)smem(kBatchBlock));
     if (e != cudaSuccess) return e;
     // barrier arrivals, generation and abort flag start at zero
     e = cudaMemsetAsync(&B.bd->bar_count, 0, 3 * sizeof(unsigned), s);

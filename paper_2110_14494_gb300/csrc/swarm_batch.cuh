@@ -15,6 +15,7 @@
 namespace pic {
 
 constexpr int kMaxSwarms = 4096;
+constexpr int kBatchBlock = 256;  // largest block of the batched collision kernels
 constexpr int kBatchGenerations = 3;  // children generations per step inside the replayed graph
 constexpr int kMaxGenerations = 62;   // product generations per step of the persistent kernel
 
@@ -649,7 +650,7 @@ template <class T> __device__ __forceinline__ void stage_proc_batch(ProcSmem<T>&
 // Three float blocks an SM: 80 registers and a few spilled words; left to itself the compiler takes 108, two
 // blocks, 124 ms in place of 111 for 256 swarms.
 template <class T, bool FAST, bool CHILD>
-__global__ void __launch_bounds__(256, sizeof(T) == 4 ? 3 : 1) k_batch_collide(const BatchArgs<T> B) {
+__global__ void __launch_bounds__(kBatchBlock, sizeof(T) == 4 ? 3 : 1) k_batch_collide(const BatchArgs<T> B) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ ProcSmem<T> ps;
     stage_proc_batch(ps, B);
@@ -751,7 +752,7 @@ __device__ bool batch_run_step(const BatchArgs<T>& B, const ProcSmem<T>& ps, Bat
 // Every step of every swarm in one launch (cooperative: all blocks resident;
 // registers capped so that two blocks fit an SM in single precision).
 template <class T, bool FAST>
-__global__ void __launch_bounds__(256, sizeof(T) == 4 ? 2 : 1) k_batch_run(const BatchArgs<T> B, int n_steps) {
+__global__ void __launch_bounds__(kBatchBlock, sizeof(T) == 4 ? 2 : 1) k_batch_run(const BatchArgs<T> B, int n_steps) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ ProcSmem<T> ps;
     stage_proc_batch(ps, B);
@@ -771,7 +772,7 @@ template <class T> struct BatchLaunch {
     static size_t smem(int block) { return (size_t)(block / 32) * sizeof(BatchStage<T>); }
     static int max_blocks_per_sm(int block);
     static cudaError_t init(const BatchArgs<T>& B, long long n0, double sig, cudaStream_t s);
-    static cudaError_t prepare(int block);  // kernel attributes for this block size (outside any capture)
+    static cudaError_t prepare();  // kernel attributes, one limit for every block size (outside any capture)
     // One step: resampling, prefix sums, parents, kBatchGenerations children
     // generations, counts, step counter.  B.in / B.out are this step's buffers.
     static cudaError_t step(BatchArgs<T> B, int block, int grid, cudaStream_t s, long long* launches);

@@ -332,3 +332,66 @@ def test_batched_tables_of_odd_length(n_bins, prec, launch):
             assert np.all(np.abs(mom[s] - omom) <= 1e-9 * (np.abs(omom).max(axis=0) + 1e-300)), s
         else:
             assert np.all(np.abs(cnt[s] - ocnt) <= 2e-3 * ocnt + 2), s
+
+
+def _in_two_threads(jobs, reps):
+    """Runs each job reps times on a thread and stream of its own: lists of results, errors raised."""
+    import threading
+    out, errs = [[] for _ in jobs], []
+
+    def work(k):
+        with torch.cuda.stream(torch.cuda.Stream()):
+            for _ in range(reps):
+                try:
+                    out[k].append(jobs[k]())
+                except Exception as e:  # noqa: BLE001
+                    errs.append(e)
+
+    threads = [threading.Thread(target=work, args=(k,)) for k in range(len(jobs))]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    torch.cuda.synchronize()
+    return out, errs
+
+
+@pytest.mark.parametrize("prec", [64, 32])
+def test_solves_on_two_threads(prec):
+    """Small levels of 91 and 72 KB of shared memory in solves that run side by
+    side: the limit that a launch needs is not lowered by the other thread, and
+    both get the bits of a solve that runs alone (deterministic sums)."""
+    from paper_2110_14494_gb300 import poisson_solve
+
+    def job(nx, ny, nz):
+        rho = torch.as_tensor(np.random.default_rng(nx).uniform(-5e-2, 5e-2, (nz, ny, nx))).cuda()
+        torch.cuda.synchronize()
+
+        def solve():
+            phi = torch.zeros_like(rho)
+            poisson_solve(W.grid_spec(nx, ny, nz, 4e-5), rho, phi, v_hi=1500.0, rtol=1e-6, max_cycles=100, precision=prec)
+            return phi
+        return solve
+
+    jobs = [job(20, 20, 20), job(24, 16, 16)]
+    alone = [j() for j in jobs]
+    torch.cuda.synchronize()
+    out, errs = _in_two_threads(jobs, 200)
+    assert not errs, errs[0]
+    for got, want in zip(out, alone):
+        assert len(got) == 200 and all(torch.equal(g, want) for g in got)
+
+
+def test_batched_swarms_on_two_threads():
+    """Blocks of 256 and of 64 threads (106 and 27 KB of shared memory) side by
+    side: counts of every step as of a run alone."""
+    from paper_2110_14494_gb300 import swarm_run
+    gas = W.synthetic_air()
+    jobs = [lambda b=b: swarm_run(gas, [120.0, 200.0], precision=64, n0=300, n_steps=4, dt=1e-12, seed=3, n_lo=10,
+                                  n_hi=10000, want_moments=True, batched=True, block=b, blocks_per_sm=1, use_graph=1)[2]
+            for b in (256, 64)]
+    alone = [j() for j in jobs]
+    out, errs = _in_two_threads(jobs, 40)
+    assert not errs, errs[0]
+    for got, want in zip(out, alone):
+        assert len(got) == 40 and all(np.array_equal(g, want) for g in got)
