@@ -50,7 +50,8 @@ enum {
     PIC_ERR_CUDA = -2,     /* a CUDA runtime call failed */
     PIC_ERR_CAPACITY = -3, /* a particle buffer or queue ran full; the step's result is incomplete */
     PIC_ERR_OVERFLOW = -4, /* a fixed-point value left its range */
-    PIC_ERR_TIMEOUT = -5,  /* an iteration limit was reached before convergence */
+    PIC_ERR_TIMEOUT = -5,  /* an iteration limit was reached: a solve before it converged, an
+                              electron whose collisions did not end (see pic_step) */
     PIC_ERR_STATE = -6     /* call not valid in the context's current state */
 };
 
@@ -228,7 +229,10 @@ int pic_set_field_f64(pic_ctx *ctx, const double *Ex, const double *Ey, const do
  * and undo it when the counts call for a weight update or further product
  * generations: the results are those of the unspeculated order, bit for bit.
  * A field solve's own error flag (cycle limit) is reported by the next call
- * that reads the counters. */
+ * that reads the counters.  An electron makes about dt nu_max collision draws
+ * a step; float32 cannot subtract a flight of less than dt / 2^24 from the time
+ * left, so with a dt near 2^24 / nu_max and longer a step ends with
+ * PIC_ERR_TIMEOUT (and incomplete) after 2^25 draws of one electron. */
 int pic_step(pic_ctx *ctx, int n_steps, pic_step_stats *stats);
 
 /* Coupled solve settings of a live context (Sec. 2.5): the relative residual
@@ -485,7 +489,8 @@ int swarm_autotune(const swarm_config *sc, int n_swarms, const double *EN_Td, co
  * results: host [n_swarms]; moments (optional): host [n_swarms][n_steps][16];
  * counts (optional): host [n_swarms][n_steps].  Errors: PIC_ERR_CAPACITY when
  * a buffer or product queue ran full, PIC_ERR_TIMEOUT when a grid-wide
- * barrier of the persistent kernel gave up waiting (the launch ended early). */
+ * barrier of the persistent kernel gave up waiting (the launch ended early) or
+ * an electron's collisions did not end (see pic_step). */
 int swarm_run(const swarm_config *sc, int n_swarms, const double *EN_Td, const double *o2_frac,
               void *d_workspace, size_t workspace_bytes, swarm_result *results, double *moments,
               long long *counts, pic_stream_t stream);

@@ -50,7 +50,20 @@ enum : unsigned {
     kErrPhotoCapacity = 32u, // photoelectron queue full
     kErrPoissonLimit = 64u,  // a device-driven coupled solve reached its cycle limit
     kErrBarrier = 128u,      // a grid-wide barrier of a persistent kernel gave up waiting
+    kErrDraws = 256u,        // an electron drew without end within one step (trip_limit)
 };
+
+// Most trips that a warp of a collision loop makes without taking new work
+// items.  An electron needs about dt nu_max draws for a step (Poisson), and a
+// trip draws for every lane's electron (double precision: for at least half of
+// the electrons in flight, draws and collisions apart, so eight trips a draw at
+// most).  More means that flights no longer shorten the time left: single
+// precision cannot take a flight of dt / 2^24 off dt, so its limit ends there.
+// The launch then ends with kErrDraws instead of never.
+template <class T> int trip_limit(double dt, double nu_max) {
+    const double n = 1048576.0 + 16.0 * dt * nu_max, most = sizeof(T) == 4 ? 33554432.0 : 2147483646.0;
+    return n < most ? (int)n : (int)most;
+}
 
 // Global loads with acquire semantics at GPU scope (flags written by other
 // blocks of the same launch).

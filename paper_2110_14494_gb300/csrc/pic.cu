@@ -1409,6 +1409,7 @@ template <class T> static PushArgs<T> make_args(pic_ctx* c, int mode) {
     A.inv_dl2 = (T)(0.69314718055994530942 * c->inv_dl);
     A.l0t = (T)(c->l0 * c->inv_dl);
     A.dt = (T)c->dt_cur;
+    A.trip_limit = trip_limit<T>(c->dt_cur, c->nu_max);
     A.dt_kick = (T)c->dt_prev;
     A.K = c->K;
     A.step = c->step;
@@ -1460,10 +1461,12 @@ static int read_state(pic_ctx* c, DevState* h) {
 static int check_err(pic_ctx* c, const DevState& h) {
     if (!h.err) return PIC_OK;
     cudaMemsetAsync(&c->st()->err, 0, sizeof(unsigned), c->s);
-    char msg[192];
+    char msg[224];
     snprintf(msg, sizeof msg, "device error flags 0x%x (1 output full, 2 child queue full, 4 fixed-point overflow, "
-             "8 descendant stack, 16 split output full, 32 photoelectron queue full, 64 poisson cycle limit)", h.err);
+             "8 descendant stack, 16 split output full, 32 photoelectron queue full, 64 poisson cycle limit, "
+             "256 collision draws without end)", h.err);
     if (h.err & kErrOverflow) return c->fail(PIC_ERR_OVERFLOW, msg);
+    if (h.err & kErrDraws) return c->fail(PIC_ERR_TIMEOUT, "step: an electron's collisions did not end (dt too long?)");
     if (h.err == kErrPoissonLimit) return c->fail(PIC_ERR_TIMEOUT, "poisson solve: cycle limit reached");
     return c->fail(PIC_ERR_CAPACITY, msg);
 }
@@ -2634,10 +2637,12 @@ template <class T> struct BatchRunner {
         if (e == cudaSuccess) e = cudaStreamSynchronize(s);
         if (e != cudaSuccess) return PIC_ERR_CUDA;
         std::vector<T> numax((size_t)n), tau((size_t)n);
+        double most = 0.0;
         for (int i = 0; i < n; ++i) {
             double v;
             memcpy(&v, &bits[i], 8);
             if (!(v > 0.0)) return PIC_ERR_ARG;
+            most = v > most ? v : most;
             numax[i] = (T)v;
             tau[i] = flight_scale<T>(v);
         }
@@ -2645,6 +2650,7 @@ template <class T> struct BatchRunner {
         if (e == cudaSuccess) e = cudaMemcpyAsync(ws + L.tau, tau.data(), (size_t)n * sizeof(T), cudaMemcpyHostToDevice, s);
         if (e == cudaSuccess) e = cudaStreamSynchronize(s);
         if (e != cudaSuccess) return PIC_ERR_CUDA;
+        B.P.trip_limit = trip_limit<T>(sc->dt, most);
         B.tab_s = tabs;
         B.tab_stride = (long long)table_reals(nb);
         B.numax_s = (const T*)(ws + L.numax);
@@ -2867,7 +2873,7 @@ static int run_batched(const swarm_config* sc, int n, const double* EN, const do
     if (e == cudaSuccess) e = cudaMemcpyAsync(&hb, R.B.bd, sizeof hb, cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     if (e != cudaSuccess) return PIC_ERR_CUDA;
-    if (hb.err & kErrBarrier) return PIC_ERR_TIMEOUT;
+    if (hb.err & (kErrBarrier | kErrDraws)) return PIC_ERR_TIMEOUT;
     if (hb.err) return PIC_ERR_CAPACITY;
     // z moments back to the origin: z = dz + r
     for (size_t r = 0; r < (size_t)n * ns; ++r) {

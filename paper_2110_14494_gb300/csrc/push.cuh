@@ -40,6 +40,7 @@ template <class T> struct PushArgs {
     T tau_scale;               // flight-time factor (flight_scale)
     T inv_dl2, l0t;            // ln 2 * inv_dl and l0 * inv_dl: table coordinate from a base-2 logarithm
     T dt;                      // duration of this step
+    int trip_limit;            // of the collision loops (trip_limit)
     T dt_kick;                 // duration of the previous step (the half-kick completes its Eq. 2)
     Keys K;
     uint32_t step;
@@ -884,7 +885,6 @@ __global__ void k_resample(const PushArgs<T> A) {
 // CHILD = false: work item = one electron of the input buffer, kicked as it is
 // staged and flying dt.  CHILD = true: work item = one queued ionization
 // product, built when it is staged.
-constexpr int kTripLimit = 1 << 24;  // of a warp in one launch (a minute): an error instead of an endless kernel
 constexpr int kRow = 11;    // padded row of a stage entry: x y z vx vy vz ax ay az w t
 constexpr int kOut = 64;    // output stage capacity (flushed at 32)
 constexpr int kPQ = 40;     // warp queue of ionization products (built 32 at a time)
@@ -1042,7 +1042,7 @@ __device__ __forceinline__ void collide_loop(const PushArgs<T>& A, const ProcSme
     // queued products, buffered negative-ion events
     int in_head = 0, in_count = 0, n_out = 0, n_pq = 0, n_att = 0, trips = 0;
     for (;;) {
-        if (++trips > kTripLimit) { atomicOr(&A.st->err, kErrStack); break; }
+        if (++trips > A.trip_limit) { atomicOr(&A.st->err, kErrDraws); break; }
         // 1. idle lanes take staged work items
         const bool want = !active;
         const unsigned need = __ballot_sync(kFull, want);
@@ -1125,6 +1125,7 @@ __device__ __forceinline__ void collide_loop(const PushArgs<T>& A, const ProcSme
             }
             in_head = 0;
             in_count = cnt;
+            trips = 0;
             __syncwarp();
         }
         // 3. termination
@@ -1255,7 +1256,7 @@ __device__ __forceinline__ void collide_pool(const PushArgs<T>& A, const ProcSme
     bool dry = false;
     for (int q = lane; q < kPool; q += 32) sg->idle[q] = (uint8_t)q;
     for (;;) {
-        if (++trips > kTripLimit) { atomicOr(&A.st->err, kErrStack); break; }
+        if (++trips > A.trip_limit) { atomicOr(&A.st->err, kErrDraws); break; }
         __syncwarp();
         const bool products = n_pq >= 32 || (dry && n_pq > 0);
         // 1. places are filled while fewer than 32 electrons wait for a draw
@@ -1309,6 +1310,7 @@ __device__ __forceinline__ void collide_pool(const PushArgs<T>& A, const ProcSme
                 next += (unsigned)cnt;
             }
             nf -= cnt;
+            trips = 0;
             const bool alive = on && r[9] > (T)0;
             const unsigned am = __ballot_sync(kFull, alive), em = __ballot_sync(kFull, on && !alive);
             if (alive) {

@@ -465,7 +465,7 @@ __device__ void batch_phase(const BatchArgs<T>& B, const ProcSmem<T>& ps, BatchS
     bool active = false, dry = false;
     int in_head = 0, in_count = 0, n_out = 0, n_pq = 0, trips = 0;
     for (;;) {
-        if (++trips > kTripLimit) { atomicOr(&B.bd->err, kErrStack); break; }
+        if (++trips > B.P.trip_limit) { atomicOr(&B.bd->err, kErrDraws); break; }
         const bool want = !active;
         const unsigned need = __ballot_sync(kFull, want);
         const int avail = in_count - in_head;
@@ -513,6 +513,7 @@ __device__ void batch_phase(const BatchArgs<T>& B, const ProcSmem<T>& ps, BatchS
             n_pq -= cnt;
             in_head = 0;
             in_count = cnt;
+            trips = 0;
             __syncwarp();
         } else if (in_head >= in_count && !dry) {
             __syncwarp();
@@ -572,6 +573,7 @@ __device__ void batch_phase(const BatchArgs<T>& B, const ProcSmem<T>& ps, BatchS
                 }
                 in_head = 0;
                 in_count = cnt;
+                trips = 0;
             }
             __syncwarp();
         }

@@ -31,3 +31,32 @@ def test_tables_of_a_batch_begin_on_16_bytes(tmp_path):
     # the binary that runs lays its batches out by that rule
     used = "".join(open(os.path.join(B.CSRC, f)).read() for f in ("pic.cu", "swarm_batch.cuh"))
     assert "kTableStride" not in used
+
+
+def test_trip_limit_of_the_collision_loops(tmp_path):
+    """The limit leaves room for every step that ends: with mean dt nu_max, an
+    electron's draws exceed it by twelve standard deviations and 100 more with a
+    probability below 1e-30, in float32 up to the 2^24 draws that its time left
+    can count (a trip draws once for every lane), in float64 with the eight
+    trips a draw of a pool; and it is an int for any dt."""
+    means = [0.0, 1e-3, 1.0, 20.0, 1e3, 1e5, 1e6, 1e7, 1.6e7, 1e8, 1e300]
+    body = "".join(f'printf("%d %d\\n", trip_limit<float>({m}, 1.0), trip_limit<double>(1e-12, {m} * 1e12));' for m in means)
+    for m, (f32, f64) in zip(means, _run(tmp_path, body)):
+        draws = m + 12 * m ** 0.5 + 100
+        assert int(f32) >= min(draws, 2 ** 24) and int(f64) >= min(8 * draws, 2 ** 31 - 2), m
+        assert int(f32) <= 2 ** 25 and int(f64) <= 2 ** 31 - 2, m
+
+
+def test_error_flags_are_bits_of_their_own(tmp_path):
+    """Each error that a kernel raises has a bit to itself, the draw limit's
+    among them, and the context's message names every bit it can report."""
+    rows = _run(tmp_path, "".join(f'printf("{n} %u\\n", (unsigned){n});' for n in (
+        "kErrOutCapacity", "kErrChildCapacity", "kErrOverflow", "kErrStack", "kErrSplitCapacity", "kErrPhotoCapacity",
+        "kErrPoissonLimit", "kErrBarrier", "kErrDraws")))
+    bits = {n: int(v) for n, v in rows}
+    assert all(v and v & (v - 1) == 0 for v in bits.values()) and len(set(bits.values())) == len(bits)
+    text = open(os.path.join(B.CSRC, "pic.cu")).read().split("static int check_err")[1].split("\n}")[0]
+    for n, v in bits.items():
+        assert n == "kErrBarrier" or f"{v} " in text, n  # (a barrier only in batched swarms)
+    loops = "".join(open(os.path.join(B.CSRC, f)).read() for f in ("push.cuh", "swarm_batch.cuh"))
+    assert loops.count("trip_limit) { atomicOr(&") == loops.count("kErrDraws") == 3
