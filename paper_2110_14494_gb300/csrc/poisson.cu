@@ -635,19 +635,20 @@ bool MG::supported(int nx_, int ny_, int nz_) {
     return (long long)m.lx[L] * m.ly[L] * m.lz[L] <= kTailMaxCells;
 }
 
-size_t MG::bytes(int nx_, int ny_, int nz_, bool mixed_, bool pair_copy, bool lean) {
+size_t MG::bytes(int nx_, int ny_, int nz_, bool mixed_, bool pair_copy, Layout layout) {
     MG m;
-    return m.carve(nullptr, nx_, ny_, nz_, mixed_, pair_copy, lean);
+    return m.carve(nullptr, nx_, ny_, nz_, mixed_, pair_copy, layout);
 }
 
 // Bytes of the device array that poisson_solve_noalloc works in.
 constexpr size_t kNoAllocScratchBytes = 32u << 20;
 
 // Lays the buffers out from base (base null: sizes only); returns the bytes.
-// Float64: A z is kept between an iteration's two kernels (a solve on 64 x 48 x
-// 80 cells takes 1113 us, 1220 with A z formed again; 128^3 2184 and 2544),
-// but for grids whose workspace fits 32 MiB only without it (96^3: 1559 us).
-size_t MG::carve(void* base, int nx_, int ny_, int nz_, bool mixed_, bool pair_copy, bool lean) {
+// Float64: A z is kept between an iteration's two kernels wherever the
+// workspace has room (a solve on 64 x 48 x 80 cells takes 1113 us, 1220 with
+// A z formed again; 96^3 1338 and 1511; 128^3 2184 and 2544).
+size_t MG::carve(void* base, int nx_, int ny_, int nz_, bool mixed_, bool pair_copy, Layout layout) {
+    const bool lean = layout == kLean;
     plan(nx_, ny_, nz_);
     mixed = mixed_;
     uintptr_t p = (uintptr_t)base;
@@ -687,13 +688,14 @@ size_t MG::carve(void* base, int nx_, int ny_, int nz_, bool mixed_, bool pair_c
         g[l] = (float*)take(n * sizeof(float));
         m[l] = (uint8_t*)take(n);
     }
-    // lean: the partial sums share the second level's e and g (8 bytes a coarse cell, at least twice their size),
-    // which only the V-cycle uses
+    // lean: the partial sums share the second level's e and g, which only the V-cycle uses: 8 bytes a coarse cell
+    // against 24 a block of up to 32 x 4 x 4 fine ones, 1.5 times their size at least (4 x 6 x 6 cells)
     if (!mixed_ && lean && levels > 1) part = (double*)e[1];
     tail_tab = tail_tables() && !lean ? (uint4*)take((size_t)tail_plan(*this).cells * sizeof(uint4)) : nullptr;
     const size_t used = (size_t)(p - p0);
     w64 = nullptr;
-    if (!mixed_ && !lean && (used > kNoAllocScratchBytes || used + align256(n0 * 8) <= kNoAllocScratchBytes))
+    if (!mixed_ && (layout == kFull || (layout == kStated && (used > kNoAllocScratchBytes ||
+                                                              used + align256(n0 * 8) <= kNoAllocScratchBytes))))
         w64 = (double*)take(n0 * 8);
     return (size_t)(p - p0);
 }
@@ -1193,16 +1195,17 @@ bool poisson_args_ok(const poisson_config* pc, const double* rho, const double* 
     return MG::supported(pc->nx, pc->ny, pc->nz);
 }
 
-size_t poisson_bytes(const poisson_config* pc, bool lean) {
-    return MG::bytes(pc->nx, pc->ny, pc->nz, pc->precision == 32, true, lean);
+size_t poisson_bytes(const poisson_config* pc, MG::Layout layout) {
+    return MG::bytes(pc->nx, pc->ny, pc->nz, pc->precision == 32, true, layout);
 }
 
-// The solve behind both entry points, on a workspace of poisson_bytes(pc, lean).
+// The solve behind both entry points, on a workspace of poisson_bytes(pc, layout).
 int poisson_run(const poisson_config* pc, const double* rho, const uint8_t* mask, double* phi, float* Ex, float* Ey,
-                float* Ez, double rtol, int max_cycles, void* ws, bool lean, poisson_stats* st, cudaStream_t s) {
+                float* Ez, double rtol, int max_cycles, void* ws, MG::Layout layout, poisson_stats* st,
+                cudaStream_t s) {
     MG mg;
     const bool mixed = pc->precision == 32;
-    mg.carve(ws, pc->nx, pc->ny, pc->nz, mixed, true, lean);
+    mg.carve(ws, pc->nx, pc->ny, pc->nz, mixed, true, layout);
     double hn[2];
     int cycles = 0;
     double rel = 0.0;
@@ -1229,15 +1232,16 @@ extern "C" size_t poisson_workspace_bytes(const poisson_config* pc) {
     if (!pc || (pc->precision != 0 && pc->precision != 32 && pc->precision != 64) ||
         !MG::supported(pc->nx, pc->ny, pc->nz))
         return 0;
-    return poisson_bytes(pc, false);
+    return poisson_bytes(pc, MG::kStated);
 }
 
 extern "C" int poisson_solve(const poisson_config* pc, const double* rho, const uint8_t* mask, double* phi, float* Ex,
                              float* Ey, float* Ez, double rtol, int max_cycles, void* ws, size_t ws_bytes,
                              poisson_stats* st, pic_stream_t stream) {
     if (!ws || !poisson_args_ok(pc, rho, phi, Ex, Ey, Ez, rtol, max_cycles)) return PIC_ERR_ARG;
-    if (ws_bytes < poisson_bytes(pc, false) || ((uintptr_t)ws & 255)) return PIC_ERR_ARG;
-    return poisson_run(pc, rho, mask, phi, Ex, Ey, Ez, rtol, max_cycles, ws, false, st, (cudaStream_t)stream);
+    if (ws_bytes < poisson_bytes(pc, MG::kStated) || ((uintptr_t)ws & 255)) return PIC_ERR_ARG;
+    const MG::Layout layout = ws_bytes < poisson_bytes(pc, MG::kFull) ? MG::kStated : MG::kFull;
+    return poisson_run(pc, rho, mask, phi, Ex, Ey, Ez, rtol, max_cycles, ws, layout, st, (cudaStream_t)stream);
 }
 
 // ------------------------------------------------------------------ no-allocation variant
@@ -1278,9 +1282,9 @@ extern "C" int poisson_solve_noalloc(const poisson_config* pc, const double* rho
                                      float* Ex, float* Ey, float* Ez, double rtol, int max_cycles, poisson_stats* st,
                                      pic_stream_t stream) {
     if (!poisson_args_ok(pc, rho, phi, Ex, Ey, Ez, rtol, max_cycles)) return PIC_ERR_ARG;
-    if (poisson_bytes(pc, true) > kNoAllocScratchBytes) return PIC_ERR_CAPACITY;
+    if (poisson_bytes(pc, MG::kLean) > kNoAllocScratchBytes) return PIC_ERR_CAPACITY;
     void* ws = nullptr;
     int rc = noalloc_scratch(&ws);
     if (rc) return rc;
-    return poisson_run(pc, rho, mask, phi, Ex, Ey, Ez, rtol, max_cycles, ws, true, st, (cudaStream_t)stream);
+    return poisson_run(pc, rho, mask, phi, Ex, Ey, Ez, rtol, max_cycles, ws, MG::kLean, st, (cudaStream_t)stream);
 }

@@ -457,12 +457,21 @@ class PicContext:
         _check(lib().pic_load(self.h, buf, len(blob)), self.h, "pic_load")
 
 
+def _poisson_bytes(pc) -> int:
+    """Workspace of a solve with room for the array that poisson_workspace_bytes
+    leaves out of some float64 sizes of at most 32 MiB (see there)."""
+    nb = lib().poisson_workspace_bytes(C.byref(pc))
+    if pc.precision != 32 and 0 < nb <= 32 << 20:
+        nb += (8 * pc.nx * pc.ny * pc.nz + 255) // 256 * 256
+    return nb
+
+
 def poisson_solve(grid: dict, rho, phi, mask=None, E=None, v_lo=0.0, v_hi=0.0, v_mask=0.0, rtol=1e-6,
                   max_cycles=100, stream=None, precision=64):
     """rho, phi: float64 CUDA tensors [nz][ny][nx]; E: optional tuple of three float32 tensors.
     precision 64: CG in float64; 32: float-pair potential with float32 CG and refinement."""
     pc = poisson_config(grid["nx"], grid["ny"], grid["nz"], grid["dx"], v_lo, v_hi, v_mask, precision)
-    nb = lib().poisson_workspace_bytes(C.byref(pc))
+    nb = _poisson_bytes(pc)
     ws, ptr = _workspace(nb)
     st = poisson_stats()
     Ex, Ey, Ez = E if E is not None else (None, None, None)

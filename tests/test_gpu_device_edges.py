@@ -395,3 +395,39 @@ def test_batched_swarms_on_two_threads():
     assert not errs, errs[0]
     for got, want in zip(out, alone):
         assert len(got) == 40 and all(np.array_equal(g, want) for g in got)
+
+
+@pytest.mark.parametrize("n,in_stated", [(88, True), (96, False), (100, True)])
+def test_float64_solve_uses_the_room_it_is_given(n, in_stated):
+    """A z is kept in the last n^3 doubles of a workspace that has room for
+    them (which 96^3 is stated without), formed again in one that has not, and
+    in the fixed scratch (up to 96^3): the same bits."""
+    import ctypes as C
+    from paper_2110_14494_gb300 import picmcc as P
+    rho = torch.as_tensor(np.random.default_rng(n).uniform(-5e-2, 5e-2, (n, n, n))).cuda()
+    pc = P.poisson_config(n, n, n, 4e-5, 0.0, 1500.0, 0.0, 64)
+    stated = P.lib().poisson_workspace_bytes(C.byref(pc))
+    az = (8 * n ** 3 + 255) // 256 * 256
+    full = stated if in_stated else stated + az
+    assert P._poisson_bytes(pc) >= full
+
+    def solve(nb):
+        ws, ptr = P._workspace(full)
+        ws.fill_(0xA5)
+        phi, st = torch.zeros_like(rho), P.poisson_stats()
+        rc = P.lib().poisson_solve(C.byref(pc), C.c_void_p(rho.data_ptr()), None, C.c_void_p(phi.data_ptr()), None, None,
+                                   None, 1e-10, 100, C.c_void_p(ptr), nb, C.byref(st), P._stream())
+        torch.cuda.synchronize()
+        assert rc == P.PIC_OK
+        off = ptr - ws.data_ptr() + full - az
+        return phi, bool((ws[off:off + 8 * n ** 3] != 0xA5).any())
+
+    phi, kept = solve(full)
+    assert kept
+    if not in_stated:
+        less, kept = solve(stated)
+        assert not kept and torch.equal(less, phi)
+    phi2 = torch.zeros_like(rho)
+    rc, _ = _solve_noalloc(P, pc, rho, phi2, torch.zeros((n, n, n), dtype=torch.uint8, device="cuda"), 1e-10, 100)
+    assert rc == (P.PIC_OK if n <= 96 else P.PIC_ERR_CAPACITY)
+    assert n > 96 or torch.equal(phi2, phi)
