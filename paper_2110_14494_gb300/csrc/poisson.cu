@@ -605,6 +605,27 @@ cudaError_t sweep_first(float* e, const float* g, const uint8_t* m, int nx, int 
     return launch_pdl(k_sweep_first<1>, grid_pair(nx, ny, nz, 1), kPairBlk, 0, s, e, g, m, nx, ny, nz);
 }
 dim3 grid_mx3(int nx, int ny, int nz) { return dim3((nx + BX - 1) / BX, (ny + BY - 1) / BY, (nz + ZC - 1) / ZC); }
+// The float64 CG kernels' blocks walk several slabs of ZC planes on larger
+// grids: a block's sums cost a third of one slab's double operations, and the
+// last block adds those of all.  One slab while the grid is about one wave of
+// blocks (five an SM), two or three while that makes it one, from there three
+// and more the larger it is (a single wave of long blocks is bound by latency
+// and leaves SMs idle at its end: 512 x 256 x 256 cells 36842 us).  A solve to
+// 1e-6 with one slab a block everywhere, with the separate kernels on bounded
+// grids that came before, and now: 96^3 cells 2388, 2467 and 2024 us, 192^3
+// 8530, 8372 and 7928, 256^3 19333, 17755 and 17286, 512 x 256 x 256 37401, 33856
+// and 32891.
+dim3 grid_cg64(int nx, int ny, int nz) {
+    dim3 g = grid_mx3(nx, ny, nz);
+    const unsigned blocks = g.x * g.y * g.z, wave = 5u * (unsigned)device_sms();
+    unsigned each = (blocks + wave - 1) / wave;
+    if (each > 3) {
+        each = blocks / 3500;
+        each = each < 3 ? 3 : (each > 8 ? 8 : each);
+    }
+    g.z = (g.z + each - 1) / each;
+    return g;
+}
 
 }  // namespace
 
@@ -693,9 +714,9 @@ size_t MG::carve(void* base, int nx_, int ny_, int nz_, bool mixed_, bool pair_c
     if (!mixed_ && lean && levels > 1) part = (double*)e[1];
     tail_tab = tail_tables() && !lean ? (uint4*)take((size_t)tail_plan(*this).cells * sizeof(uint4)) : nullptr;
     const size_t used = (size_t)(p - p0);
+    const bool room = used + align256(n0 * 8) <= kNoAllocScratchBytes;
     w64 = nullptr;
-    if (!mixed_ && (layout == kFull || (layout == kStated && (used > kNoAllocScratchBytes ||
-                                                              used + align256(n0 * 8) <= kNoAllocScratchBytes))))
+    if (!mixed_ && (layout == kFull || room || (layout == kStated && used > kNoAllocScratchBytes)))
         w64 = (double*)take(n0 * 8);
     return (size_t)(p - p0);
 }
@@ -846,10 +867,12 @@ void MG::iteration(cudaStream_t s, double* phi, const uint8_t* mk, bool first) {
     const int nx = lx[0], ny = ly[0], nz = lz[0];
     const int f = first ? 1 : 0;
     vcycle(s, false);
-    note(launch_pdl(k_apply64, grid_mx3(nx, ny, nz), kBlk, 0, s, (const float*)e[0], (const double*)r64,
+    const dim3 g3 = grid_cg64(nx, ny, nz);
+    const bool many = (int)g3.z * ZC < nz;
+    note(launch_pdl(many ? k_apply64<true> : k_apply64<false>, g3, kBlk, 0, s, (const float*)e[0], (const double*)r64,
                     (const double*)q64, w64, mk, nx, ny, nz, f, part, ctr + 1, norms));
-    note(launch_pdl(k_step64, grid_mx3(nx, ny, nz), kBlk, 0, s, (const float*)e[0], (const double*)w64, mk, p64, q64, phi,
-                    r64, g[0], nx, ny, nz, f, part, ctr + 2, norms));
+    note(launch_pdl(many ? k_step64<true> : k_step64<false>, g3, kBlk, 0, s, (const float*)e[0], (const double*)w64, mk,
+                    p64, q64, phi, r64, g[0], nx, ny, nz, f, part, ctr + 2, norms));
     launches += 2;
 }
 
@@ -880,8 +903,11 @@ int MG::solve(const double* rho, const uint8_t* mask, double* phi, double h, dou
         g_key[0] = phi; g_key[1] = rho; g_key[2] = mask;
     }
     if (cudaMemsetAsync(ctr, 0, 8 * sizeof(unsigned), s) != cudaSuccess) return PIC_ERR_CUDA;
-    k_resid64<<<grid_mx3(nx, ny, nz), kBlk, 0, s>>>(phi, rho, mk, nx, ny, nz, h2e, v_lo, v_hi, v_mask, r64, g[0], part,
-                                                    ctr, norms);
+    const dim3 g3 = grid_cg64(nx, ny, nz);
+    if ((int)g3.z * ZC < nz)
+        k_resid64<true><<<g3, kBlk, 0, s>>>(phi, rho, mk, nx, ny, nz, h2e, v_lo, v_hi, v_mask, r64, g[0], part, ctr, norms);
+    else
+        k_resid64<false><<<g3, kBlk, 0, s>>>(phi, rho, mk, nx, ny, nz, h2e, v_lo, v_hi, v_mask, r64, g[0], part, ctr, norms);
     launches += 1;
     int cyc = 0, rc = PIC_OK;
     double bn = 1.0, rn = 0.0;

@@ -111,9 +111,9 @@ struct MG : LaunchStatus {
     static bool supported(int nx, int ny, int nz);
     // Workspace of the float64 solve (mixed false) or of the mixed one
     // (pair_copy: with room for the pair copy of a float64 potential).
-    // kLean: no more than the solve cannot do without (no stored A z, no tail tables), for the fixed scratch
-    // of poisson_solve_noalloc; kStated: what poisson_workspace_bytes states, A z unless that alone would take a
-    // float64 workspace above 32 MiB; kFull: with A z.
+    // kLean: for the fixed scratch of poisson_solve_noalloc, without the tail's tables and with A z only within
+    // its 32 MiB; kStated: what poisson_workspace_bytes states, A z unless that alone would take a float64
+    // workspace above 32 MiB; kFull: with A z.
     enum Layout { kLean, kStated, kFull };
     static size_t bytes(int nx, int ny, int nz, bool mixed = false, bool pair_copy = false, Layout layout = kFull);
     size_t carve(void* base, int nx, int ny, int nz, bool mixed = false, bool pair_copy = false, Layout layout = kFull);

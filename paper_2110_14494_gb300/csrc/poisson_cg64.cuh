@@ -73,15 +73,18 @@ template <int NV> __device__ bool grid_sums64(const double (&v)[NV], double* par
 // preconditioner; ||b||^2 with b = h^2 rho / eps0 + plate and electrode terms,
 // ||r||^2; electrode cells get phi = v_mask (their neighbours use v_mask, not
 // the value they may still hold).
+// MANY: the block walks several slabs of planes (grid_cg64).
+template <bool MANY>
 __global__ void __launch_bounds__(BX * BY) k_resid64(double* __restrict__ phi, const double* __restrict__ rho,
                                                      const uint8_t* __restrict__ mask, int nx, int ny, int nz, double h2e,
                                                      double v_lo, double v_hi, double v_mask, double* __restrict__ r,
                                                      float* __restrict__ g0, double* part, unsigned* ctr, double* sc) {
-    const int i = blockIdx.x * BX + threadIdx.x, j = blockIdx.y * BY + threadIdx.y, k0 = blockIdx.z * ZC;
+    const int i = blockIdx.x * BX + threadIdx.x, j = blockIdx.y * BY + threadIdx.y;
     const bool in = i < nx && j < ny;
     const int pl = nx * ny, c0 = in ? lin(i, j, 0, nx, ny) : 0;
     double acc[2] = {0.0, 0.0};
-    if (in) {
+    int k0 = blockIdx.z * ZC;
+    if (in) do {
         double col[ZC + 2], xm[ZC], xp[ZC], ym[ZC], yp[ZC], rh[ZC];
         uint8_t cm[ZC + 2], mx[ZC], mp[ZC], my[ZC], mq[ZC];
 #pragma unroll
@@ -131,7 +134,7 @@ __global__ void __launch_bounds__(BX * BY) k_resid64(double* __restrict__ phi, c
             acc[0] += b * b;
             acc[1] += rr * rr;
         }
-    }
+    } while (MANY && (k0 += gridDim.z * ZC) < nz);
     double tot[2];
     if (grid_sums64<2>(acc, part, ctr, tot)) {
         sc[S_B2] = tot[0];
@@ -188,31 +191,36 @@ __device__ __forceinline__ void apply64(const float* __restrict__ z, const uint8
 
 // The sums z.r, z.q_prev and z.w with w = A z (stored if w is given), then the
 // iteration's scalars (last block).
+template <bool MANY>
 __global__ void __launch_bounds__(BX * BY) k_apply64(const float* __restrict__ z, const double* __restrict__ r,
                                                      const double* __restrict__ q_prev, double* __restrict__ w,
                                                      const uint8_t* __restrict__ mask, int nx, int ny, int nz, int first,
                                                      double* part, unsigned* ctr, double* sc) {
     pdl_wait();
-    const int i = blockIdx.x * BX + threadIdx.x, j = blockIdx.y * BY + threadIdx.y, k0 = blockIdx.z * ZC;
+    const int i = blockIdx.x * BX + threadIdx.x, j = blockIdx.y * BY + threadIdx.y;
     const bool in = i < nx && j < ny;
     const int pl = nx * ny, c0 = in ? lin(i, j, 0, nx, ny) : 0;
-    double rv[ZC], qv[ZC], acc[3] = {0.0, 0.0, 0.0};
+    double acc[3] = {0.0, 0.0, 0.0};
+    int k0 = blockIdx.z * ZC;
+    do {
+        double rv[ZC], qv[ZC];
 #pragma unroll
-    for (int d = 0; d < ZC; ++d) {
-        const bool ok = in && k0 + d < nz;
-        rv[d] = ok ? r[c0 + (k0 + d) * pl] : 0.0;
-        qv[d] = ok && !first ? q_prev[c0 + (k0 + d) * pl] : 0.0;
-    }
-    Apply64 o;
-    apply64(z, mask, i, j, k0, nx, ny, nz, o);
+        for (int d = 0; d < ZC; ++d) {
+            const bool ok = in && k0 + d < nz;
+            rv[d] = ok ? r[c0 + (k0 + d) * pl] : 0.0;
+            qv[d] = ok && !first ? q_prev[c0 + (k0 + d) * pl] : 0.0;
+        }
+        Apply64 o;
+        apply64(z, mask, i, j, k0, nx, ny, nz, o);
 #pragma unroll
-    for (int d = 0; d < ZC; ++d) {
-        if (!in || k0 + d >= nz) break;
-        if (w) w[c0 + (k0 + d) * pl] = o.w[d];
-        acc[0] += o.z[d] * rv[d];
-        if (!first) acc[1] += o.z[d] * qv[d];
-        acc[2] += o.z[d] * o.w[d];
-    }
+        for (int d = 0; d < ZC; ++d) {
+            if (!in || k0 + d >= nz) break;
+            if (w) w[c0 + (k0 + d) * pl] = o.w[d];
+            acc[0] += o.z[d] * rv[d];
+            if (!first) acc[1] += o.z[d] * qv[d];
+            acc[2] += o.z[d] * o.w[d];
+        }
+    } while (MANY && (k0 += gridDim.z * ZC) < nz);
     double tot[3];
     if (grid_sums64<3>(acc, part, ctr, tot)) cg_scalars(tot, first, sc);
 }
@@ -220,49 +228,55 @@ __global__ void __launch_bounds__(BX * BY) k_apply64(const float* __restrict__ z
 // p = z + beta p, q = w + beta q, phi += alpha p, r -= alpha q with its
 // float32 copy, ||r||^2.  Without a stored w (MG::carve) w = A z is formed again: the same values, 13 double
 // operations a cell more (16 us in place of 7 on 64 x 48 x 80 cells).
+template <bool MANY>
 __global__ void __launch_bounds__(BX * BY) k_step64(const float* __restrict__ z, const double* __restrict__ w,
                                                     const uint8_t* __restrict__ mask, double* __restrict__ p,
                                                     double* __restrict__ q, double* __restrict__ phi,
                                                     double* __restrict__ r, float* __restrict__ g0, int nx, int ny, int nz,
                                                     int first, double* part, unsigned* ctr, double* sc) {
     pdl_wait();
-    const int i = blockIdx.x * BX + threadIdx.x, j = blockIdx.y * BY + threadIdx.y, k0 = blockIdx.z * ZC;
+    const int i = blockIdx.x * BX + threadIdx.x, j = blockIdx.y * BY + threadIdx.y;
     const double a = sc[S_ALPHA], b = first ? 0.0 : sc[S_BETA];
     const bool in = i < nx && j < ny, prev = b != 0.0;
-    const int pl = nx * ny, c0 = in ? lin(i, j, k0, nx, ny) : 0;
-    double pv[ZC], qv[ZC], fv[ZC], rv[ZC], acc[1] = {0.0};
-#pragma unroll
-    for (int d = 0; d < ZC; ++d) {
-        const bool ok = in && k0 + d < nz;
-        pv[d] = ok && prev ? p[c0 + d * pl] : 0.0;
-        qv[d] = ok && prev ? q[c0 + d * pl] : 0.0;
-        fv[d] = ok ? phi[c0 + d * pl] : 0.0;
-        rv[d] = ok ? r[c0 + d * pl] : 0.0;
-    }
-    Apply64 o;
-    if (w) {
+    const int pl = nx * ny;
+    double acc[1] = {0.0};
+    int k0 = blockIdx.z * ZC;
+    do {
+        const int c0 = in ? lin(i, j, k0, nx, ny) : 0;
+        double pv[ZC], qv[ZC], fv[ZC], rv[ZC];
 #pragma unroll
         for (int d = 0; d < ZC; ++d) {
             const bool ok = in && k0 + d < nz;
-            o.z[d] = ok ? (double)z[c0 + d * pl] : 0.0;
-            o.w[d] = ok ? w[c0 + d * pl] : 0.0;
+            pv[d] = ok && prev ? p[c0 + d * pl] : 0.0;
+            qv[d] = ok && prev ? q[c0 + d * pl] : 0.0;
+            fv[d] = ok ? phi[c0 + d * pl] : 0.0;
+            rv[d] = ok ? r[c0 + d * pl] : 0.0;
         }
-    } else {
-        apply64(z, mask, i, j, k0, nx, ny, nz, o);
-    }
+        Apply64 o;
+        if (w) {
 #pragma unroll
-    for (int d = 0; d < ZC; ++d) {
-        if (!in || k0 + d >= nz) break;
-        const int c = c0 + d * pl;
-        const double pp = prev ? o.z[d] + b * pv[d] : o.z[d], qq = prev ? o.w[d] + b * qv[d] : o.w[d];
-        p[c] = pp;
-        q[c] = qq;
-        phi[c] = fv[d] + a * pp;
-        const double rr = rv[d] - a * qq;
-        r[c] = rr;
-        g0[c] = (float)rr;
-        acc[0] += rr * rr;
-    }
+            for (int d = 0; d < ZC; ++d) {
+                const bool ok = in && k0 + d < nz;
+                o.z[d] = ok ? (double)z[c0 + d * pl] : 0.0;
+                o.w[d] = ok ? w[c0 + d * pl] : 0.0;
+            }
+        } else {
+            apply64(z, mask, i, j, k0, nx, ny, nz, o);
+        }
+#pragma unroll
+        for (int d = 0; d < ZC; ++d) {
+            if (!in || k0 + d >= nz) break;
+            const int c = c0 + d * pl;
+            const double pp = prev ? o.z[d] + b * pv[d] : o.z[d], qq = prev ? o.w[d] + b * qv[d] : o.w[d];
+            p[c] = pp;
+            q[c] = qq;
+            phi[c] = fv[d] + a * pp;
+            const double rr = rv[d] - a * qq;
+            r[c] = rr;
+            g0[c] = (float)rr;
+            acc[0] += rr * rr;
+        }
+    } while (MANY && (k0 += gridDim.z * ZC) < nz);
     double tot[1];
     if (grid_sums64<1>(acc, part, ctr, tot)) sc[S_R2] = tot[0];
 }

@@ -400,8 +400,8 @@ def test_batched_swarms_on_two_threads():
 @pytest.mark.parametrize("n,in_stated", [(88, True), (96, False), (100, True)])
 def test_float64_solve_uses_the_room_it_is_given(n, in_stated):
     """A z is kept in the last n^3 doubles of a workspace that has room for
-    them (which 96^3 is stated without), formed again in one that has not, and
-    in the fixed scratch (up to 96^3): the same bits."""
+    them (which 96^3 is stated without) and formed again in one that has not;
+    the fixed scratch has room at 88^3, none at 96^3: the same bits."""
     import ctypes as C
     from paper_2110_14494_gb300 import picmcc as P
     rho = torch.as_tensor(np.random.default_rng(n).uniform(-5e-2, 5e-2, (n, n, n))).cuda()
@@ -431,3 +431,41 @@ def test_float64_solve_uses_the_room_it_is_given(n, in_stated):
     rc, _ = _solve_noalloc(P, pc, rho, phi2, torch.zeros((n, n, n), dtype=torch.uint8, device="cuda"), 1e-10, 100)
     assert rc == (P.PIC_OK if n <= 96 else P.PIC_ERR_CAPACITY)
     assert n > 96 or torch.equal(phi2, phi)
+
+
+@pytest.mark.parametrize("shape", [(96, 64, 100), (96, 96, 96), (160, 144, 72), (512, 128, 240)])
+def test_float64_solve_with_several_slabs_a_block(shape):
+    """Blocks of the CG kernels that walk 2, 3, 3 and 8 slabs of planes, the
+    last ones fewer: the residual that the solve reports (its sums over all
+    slabs) is the one of the potential it returns, formed here.  Its rounding,
+    2e-16 of seven terms a cell, is below 1e-13 of the right-hand side."""
+    from paper_2110_14494_gb300 import poisson_solve
+    nx, ny, nz = shape
+    h, lo, hi, vm = 4e-5, -100.0, 1500.0, 700.0
+    g = torch.Generator(device="cuda").manual_seed(nx)
+    rho = 1e-1 * torch.rand((nz, ny, nx), generator=g, device="cuda", dtype=torch.float64) - 5e-2
+    mask = torch.rand((nz, ny, nx), generator=g, device="cuda") < 0.002
+    phi = torch.zeros_like(rho)
+    cyc, rel = poisson_solve(W.grid_spec(nx, ny, nz, h), rho, phi, mask=mask.to(torch.uint8), v_lo=lo, v_hi=hi, v_mask=vm,
+                             rtol=1e-9, max_cycles=40, precision=64)
+    f = torch.where(mask, torch.full_like(phi, vm), phi)
+    assert torch.equal(f, phi)
+
+    def neighbours(u, low, high, mirror):
+        s = torch.zeros_like(u)
+        for d in (2, 1, 0):
+            n = u.shape[d]
+            s.narrow(d, 1, n - 1).add_(u.narrow(d, 0, n - 1))
+            s.narrow(d, 0, n - 1).add_(u.narrow(d, 1, n - 1))
+            if d and mirror:
+                s.narrow(d, 0, 1).add_(u.narrow(d, 0, 1))
+                s.narrow(d, n - 1, 1).add_(u.narrow(d, n - 1, 1))
+        s[0] += low
+        s[-1] += high
+        return s
+
+    h2r = h * h / 8.8541878128e-12 * rho
+    b = h2r + neighbours(torch.where(mask, torch.full_like(phi, vm), torch.zeros_like(phi)), 2 * lo, 2 * hi, False)
+    r = h2r + neighbours(f, 2 * lo - f[0], 2 * hi - f[-1], True) - 6.0 * f
+    res = (r[~mask].norm() / b[~mask].norm()).item()
+    assert rel <= 1e-9 and abs(res - rel) <= 1e-3 * rel + 1e-13, (cyc, rel, res)
