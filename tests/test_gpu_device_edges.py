@@ -469,3 +469,30 @@ def test_float64_solve_with_several_slabs_a_block(shape):
     r = h2r + neighbours(f, 2 * lo - f[0], 2 * hi - f[-1], True) - 6.0 * f
     res = (r[~mask].norm() / b[~mask].norm()).item()
     assert rel <= 1e-9 and abs(res - rel) <= 1e-3 * rel + 1e-13, (cyc, rel, res)
+
+
+@pytest.mark.parametrize("prec", [64, 32])
+def test_weight_update_around_the_electrons_of_a_warp(prec):
+    """Cells of 1 to 300 electrons, 31, 32, 33, 128 and 129 among them (one
+    electron a lane, four, and more), beside empty ones: the merged and split
+    set is the oracle's, bit for bit."""
+    from paper_2110_14494_gb300 import PicContext
+    from tests.gpu_common import by_id
+    grid = W.grid_spec(9, 7, 8, 1e-4)
+    counts = [1, 2, 31, 32, 33, 63, 64, 65, 96, 127, 128, 129, 161, 256, 257, 300]
+    p0 = W.random_particles(sum(counts), grid, 61, w_range=(1.0, 40.0))
+    cells = np.repeat(5 + 17 * np.arange(len(counts)), counts)  # every 17th cell
+    for k, i in (("x", cells % 9), ("y", cells // 9 % 7), ("z", cells // 63)):
+        p0[k][:] = (1e-4 * (i + 0.25 + 0.5 * (p0[k] / (1e-4 * grid["n" + k])))).astype(np.float32)
+    gas = W.synthetic_air()
+    ctx = PicContext(gas, grid, precision=prec, capacity=20000, seed=SEED, dt=1e-12, n_ppc=40, w_min=1.0, particle_cap=0)
+    ctx.set_particles(p0)
+    ctx.weight_update()
+    gpu = by_id(ctx.get_particles())
+    P = O.Particles(20000, p0)
+    rc, _ = O.merge_split(O.Model(gas, 1e-12, SEED, prec, grid), P, 0, n_ppc=40, w_min=1.0, cap=0)
+    ref = by_id(P.view())
+    assert rc == 0 and len(ref["id"]) != len(p0["id"])
+    assert np.array_equal(gpu["id"], ref["id"])
+    for k in ("x", "y", "z", "vx", "vy", "vz", "w"):
+        assert np.array_equal(gpu[k], ref[k]), k
