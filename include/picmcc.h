@@ -232,7 +232,7 @@ int pic_set_field_f64(pic_ctx *ctx, const double *Ex, const double *Ey, const do
  * that reads the counters.  An electron makes about dt nu_max collision draws
  * a step; float32 cannot subtract a flight of less than dt / 2^24 from the time
  * left, so with a dt near 2^24 / nu_max and longer a step ends with
- * PIC_ERR_TIMEOUT (and incomplete) after 2^25 draws of one electron. */
+ * PIC_ERR_TIMEOUT (and incomplete) after some 2^25 draws of one electron. */
 int pic_step(pic_ctx *ctx, int n_steps, pic_step_stats *stats);
 
 /* Coupled solve settings of a live context (Sec. 2.5): the relative residual

@@ -54,15 +54,17 @@ enum : unsigned {
 };
 
 // Most trips that a warp of a collision loop makes without taking new work
-// items.  An electron needs about dt nu_max draws for a step (Poisson), and a
-// trip draws for every lane's electron (double precision: for at least half of
-// the electrons in flight, draws and collisions apart, so eight trips a draw at
-// most).  More means that flights no longer shorten the time left: single
-// precision cannot take a flight of dt / 2^24 off dt, so its limit ends there.
-// The launch then ends with kErrDraws instead of never.
-template <class T> int trip_limit(double dt, double nu_max) {
-    const double n = 1048576.0 + 16.0 * dt * nu_max, most = sizeof(T) == 4 ? 33554432.0 : 2147483646.0;
-    return n < most ? (int)n : (int)most;
+// items; the launch then ends with kErrDraws instead of never.  An electron
+// needs about dt nu_max draws for a step (Poisson).  Single precision: a trip
+// draws for every lane, and the time left less a flight of its 2^-25 is the
+// time left again, so an electron that needs more than 2^24 draws hardly gets
+// on (a constant: as a kernel argument it costs a step up to 3 %).  Double
+// precision: at least half of the electrons in flight advance by a draw or a
+// collision, eight trips a draw at most.
+constexpr int kTripsF32 = 1 << 25;
+inline int trip_limit(double dt, double nu_max) {
+    const double n = 1048576.0 + 16.0 * dt * nu_max;
+    return n < 2147483647.0 ? (int)n : 2147483647;
 }
 
 // Global loads with acquire semantics at GPU scope (flags written by other

@@ -1415,7 +1415,7 @@ template <class T> static PushArgs<T> make_args(pic_ctx* c, int mode) {
     A.inv_dl2 = (T)(0.69314718055994530942 * c->inv_dl);
     A.l0t = (T)(c->l0 * c->inv_dl);
     A.dt = (T)c->dt_cur;
-    A.trip_limit = trip_limit<T>(c->dt_cur, c->nu_max);
+    A.trip_limit = trip_limit(c->dt_cur, c->nu_max);
     A.dt_kick = (T)c->dt_prev;
     A.K = c->K;
     A.step = c->step;
@@ -2656,7 +2656,7 @@ template <class T> struct BatchRunner {
         if (e == cudaSuccess) e = cudaMemcpyAsync(ws + L.tau, tau.data(), (size_t)n * sizeof(T), cudaMemcpyHostToDevice, s);
         if (e == cudaSuccess) e = cudaStreamSynchronize(s);
         if (e != cudaSuccess) return PIC_ERR_CUDA;
-        B.P.trip_limit = trip_limit<T>(sc->dt, most);
+        B.P.trip_limit = trip_limit(sc->dt, most);
         B.tab_s = tabs;
         B.tab_stride = (long long)table_reals(nb);
         B.numax_s = (const T*)(ws + L.numax);

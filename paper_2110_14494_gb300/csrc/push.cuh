@@ -40,7 +40,7 @@ template <class T> struct PushArgs {
     T tau_scale;               // flight-time factor (flight_scale)
     T inv_dl2, l0t;            // ln 2 * inv_dl and l0 * inv_dl: table coordinate from a base-2 logarithm
     T dt;                      // duration of this step
-    int trip_limit;            // of the collision loops (trip_limit)
+    int trip_limit;            // of the collision loops in double precision (trip_limit)
     T dt_kick;                 // duration of the previous step (the half-kick completes its Eq. 2)
     Keys K;
     uint32_t step;
@@ -885,6 +885,9 @@ __global__ void k_resample(const PushArgs<T> A) {
 // CHILD = false: work item = one electron of the input buffer, kicked as it is
 // staged and flying dt.  CHILD = true: work item = one queued ionization
 // product, built when it is staged.
+template <class T> __device__ __forceinline__ int most_trips(const PushArgs<T>& A) {
+    return sizeof(T) == 4 ? kTripsF32 : A.trip_limit;
+}
 constexpr int kRow = 11;    // padded row of a stage entry: x y z vx vy vz ax ay az w t
 constexpr int kOut = 64;    // output stage capacity (flushed at 32)
 constexpr int kPQ = 40;     // warp queue of ionization products (built 32 at a time)
@@ -1040,9 +1043,9 @@ __device__ __forceinline__ void collide_loop(const PushArgs<T>& A, const ProcSme
     bool active = false, dry = false, first = true;
     // warp-uniform counters: input stage head and size, output stage size,
     // queued products, buffered negative-ion events
-    int in_head = 0, in_count = 0, n_out = 0, n_pq = 0, n_att = 0, trips = 0;
+    int in_head = 0, in_count = 0, n_out = 0, n_pq = 0, n_att = 0, trips_left = most_trips(A);
     for (;;) {
-        if (++trips > A.trip_limit) { atomicOr(&A.st->err, kErrDraws); break; }
+        if (--trips_left < 0) { atomicOr(&A.st->err, kErrDraws); break; }
         // 1. idle lanes take staged work items
         const bool want = !active;
         const unsigned need = __ballot_sync(kFull, want);
@@ -1125,7 +1128,7 @@ __device__ __forceinline__ void collide_loop(const PushArgs<T>& A, const ProcSme
             }
             in_head = 0;
             in_count = cnt;
-            trips = 0;
+            trips_left = most_trips(A);
             __syncwarp();
         }
         // 3. termination
@@ -1252,11 +1255,11 @@ __device__ __forceinline__ void collide_pool(const PushArgs<T>& A, const ProcSme
     unsigned end = next < n_items ? (n_items - next < chunk ? n_items : next + chunk) : 0u;
     if (end == 0u) next = 0u;
     // warp-uniform: sizes of the lists, of the output stage, queued products, buffered negative-ion events
-    int nd = 0, nh = 0, nf = kPool, n_out = 0, n_pq = 0, n_att = 0, trips = 0;
+    int nd = 0, nh = 0, nf = kPool, n_out = 0, n_pq = 0, n_att = 0, trips_left = most_trips(A);
     bool dry = false;
     for (int q = lane; q < kPool; q += 32) sg->idle[q] = (uint8_t)q;
     for (;;) {
-        if (++trips > A.trip_limit) { atomicOr(&A.st->err, kErrDraws); break; }
+        if (--trips_left < 0) { atomicOr(&A.st->err, kErrDraws); break; }
         __syncwarp();
         const bool products = n_pq >= 32 || (dry && n_pq > 0);
         // 1. places are filled while fewer than 32 electrons wait for a draw
@@ -1310,7 +1313,7 @@ __device__ __forceinline__ void collide_pool(const PushArgs<T>& A, const ProcSme
                 next += (unsigned)cnt;
             }
             nf -= cnt;
-            trips = 0;
+            trips_left = most_trips(A);
             const bool alive = on && r[9] > (T)0;
             const unsigned am = __ballot_sync(kFull, alive), em = __ballot_sync(kFull, on && !alive);
             if (alive) {

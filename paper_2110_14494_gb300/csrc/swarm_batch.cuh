@@ -463,9 +463,9 @@ __device__ void batch_phase(const BatchArgs<T>& B, const ProcSmem<T>& ps, BatchS
     int s_cur = -1, s_cache = -1;
     long long w_next = 0, w_end = 0;
     bool active = false, dry = false;
-    int in_head = 0, in_count = 0, n_out = 0, n_pq = 0, trips = 0;
+    int in_head = 0, in_count = 0, n_out = 0, n_pq = 0, trips_left = most_trips(B.P);
     for (;;) {
-        if (++trips > B.P.trip_limit) { atomicOr(&B.bd->err, kErrDraws); break; }
+        if (--trips_left < 0) { atomicOr(&B.bd->err, kErrDraws); break; }
         const bool want = !active;
         const unsigned need = __ballot_sync(kFull, want);
         const int avail = in_count - in_head;
@@ -513,7 +513,7 @@ __device__ void batch_phase(const BatchArgs<T>& B, const ProcSmem<T>& ps, BatchS
             n_pq -= cnt;
             in_head = 0;
             in_count = cnt;
-            trips = 0;
+            trips_left = most_trips(B.P);
             __syncwarp();
         } else if (in_head >= in_count && !dry) {
             __syncwarp();
@@ -573,7 +573,7 @@ __device__ void batch_phase(const BatchArgs<T>& B, const ProcSmem<T>& ps, BatchS
                 }
                 in_head = 0;
                 in_count = cnt;
-                trips = 0;
+                trips_left = most_trips(B.P);
             }
             __syncwarp();
         }
