@@ -1420,7 +1420,6 @@ template <class T> static PushArgs<T> make_args(pic_ctx* c, int mode) {
     A.K = c->K;
     A.step = c->step;
     A.first = c->a_valid ? 0 : 1;
-    A.kick_on_load = 0;
     A.cap_out = c->cfg.capacity;
     A.cap_child = c->cfg.capacity;
     A.nx = c->g.nx; A.ny = c->g.ny; A.nz = c->g.nz;
@@ -2149,7 +2148,6 @@ template <class T> static int one_step(pic_ctx* c, bool stats, bool* solved) {
     c->mark(0);
     c->launches += 3;
     // the gather and half-kick of Eq. 2 are done as the collision kernel loads each parent
-    A.kick_on_load = 1;
     cudaError_t e = PushLaunch<T>::parents(A, MODE_PIC, stats, c->grid_push, c->s);
     c->mark(1);
     if (e == cudaSuccess) e = PushLaunch<T>::children(A, MODE_PIC, stats, c->grid_push, c->s);

@@ -6,11 +6,15 @@
 // sections.  Sec. 2.1.3: the field is interpolated to the particle and the
 // particle mapped to the grid with trilinear (cloud-in-cell) weights.
 //
-// One thread owns one electron for the whole step: gather, half-kick, the
-// chain of free flights and collisions, reflection at the domain faces,
-// electrode absorption, append of the survivor to the other buffer with a
-// warp-aggregated cursor, and its deposit.  Ionization products are queued
-// with their remaining time and finished by k_children in the same step.
+// A step of an electron: gather, half-kick, the chain of free flights and
+// collisions, reflection at the domain faces, electrode absorption, append of
+// the survivor to the other buffer with a warp-aggregated cursor, and its
+// deposit.  Single precision (collide_loop): one lane owns the electron through
+// its flights and collisions.  Double precision (collide_pool): the electron
+// stands in its warp's shared memory, and whichever lanes come next do its
+// draws and collisions.  Ionization products wait in the warp's queue and fly
+// their remaining time as its next work items; k_children finishes those that
+// the queue could not take.
 // Instantiated for T = float and T = double in separate translation units.
 #pragma once
 #include <type_traits>
@@ -45,7 +49,6 @@ template <class T> struct PushArgs {
     Keys K;
     uint32_t step;
     int first;                 // previous acceleration unknown: no half-kick
-    int kick_on_load;          // parents get the gather and half-kick when the collision kernel loads them
     long long cap_out, cap_child;
     // grid (PIC mode)
     int nx, ny, nz;
@@ -866,11 +869,12 @@ __global__ void k_resample(const PushArgs<T> A) {
 }
 
 // ------------------------------------------------------------------ collisions
-// Lanes refill from per-warp shared-memory stages.  Every lane owns one
-// electron at a time and advances it by up to two draws and a collision per
-// loop iteration (advance); a lane whose electron has finished the step takes
-// the next electron from the warp's input stage at once, so the warp stays
-// converged while electrons need different numbers of events.  All
+// Single precision (collide_loop; double precision: collide_pool, which has the
+// output stage and the product queue in common): lanes refill from per-warp
+// shared-memory stages.  Every lane owns one electron at a time and advances it by up to two draws and a
+// collision per loop iteration (advance); a lane whose electron has finished
+// the step takes the next electron from the warp's input stage at once, so the
+// warp stays converged while electrons need different numbers of events.  All
 // per-electron memory work is done by the whole warp, 32 electrons at a time:
 // the input stage is filled with one coalesced load of consecutive work items,
 // finished electrons wait in the output stage until 32 are there and are then
@@ -885,14 +889,14 @@ __global__ void k_resample(const PushArgs<T> A) {
 // CHILD = false: work item = one electron of the input buffer, kicked as it is
 // staged and flying dt.  CHILD = true: work item = one queued ionization
 // product, built when it is staged.
-template <class T> __device__ __forceinline__ int most_trips(const PushArgs<T>& A) {
-    return sizeof(T) == 4 ? kTripsF32 : A.trip_limit;
-}
 constexpr int kRow = 11;    // padded row of a stage entry: x y z vx vy vz ax ay az w t
 constexpr int kOut = 64;    // output stage capacity (flushed at 32)
 constexpr int kPQ = 40;     // warp queue of ionization products (built 32 at a time)
 constexpr int kPQRow = 9;   // x y z, product speed, ax ay az of the ionizing electron, w, remaining time
 constexpr int kAtt = 32;    // warp buffer of attachment events awaiting their deposit
+template <class T> __device__ __forceinline__ int most_trips(const PushArgs<T>& A) {
+    return sizeof(T) == 4 ? kTripsF32 : A.trip_limit;
+}
 
 template <class T> struct Stage {
     T in[32 * kRow];
@@ -1118,7 +1122,7 @@ __device__ __forceinline__ void collide_loop(const PushArgs<T>& A, const ProcSme
                             T f[10];
                             for (int q = 0; q < 10; ++q) f[q] = A.in.r[q][it];
                             if (MODE == MODE_SWARM) uniform_accel(A, f);
-                            else if (A.kick_on_load) half_kick(A, f);
+                            else half_kick(A, f);
                             for (int q = 0; q < 10; ++q) r[q] = f[q];
                             r[10] = A.dt;
                             sg->in_id[lane] = A.in.id[it];
@@ -1300,7 +1304,7 @@ __device__ __forceinline__ void collide_pool(const PushArgs<T>& A, const ProcSme
                     } else {
                         for (int q = 0; q < 10; ++q) r[q] = A.in.r[q][it];
                         if (MODE == MODE_SWARM) uniform_accel(A, r);
-                        else if (A.kick_on_load) half_kick(A, r);
+                        else half_kick(A, r);
                         r[10] = A.dt;
                         id = A.in.id[it];
                     }
