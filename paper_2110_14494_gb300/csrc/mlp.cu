@@ -1207,7 +1207,7 @@ extern "C" int mlp_train(float* params, float* m, float* v, int step0, const flo
         e = backprop(params, x, t, n, w, s);
         if (e == cudaSuccess)
             e = pic::launch_pdl(k_adam, dim3(kParamBlocks), dim3(kParamThreads), 0, s, parts_of(w), params, m, v,
-                            step0 + k + 1, lr, beta1, beta2, eps, w.w2b, loss, inv6n);
+                                step0 + k + 1, lr, beta1, beta2, eps, w.w2b, loss, inv6n);
     }
     return e == cudaSuccess && cudaGetLastError() == cudaSuccess ? PIC_OK : PIC_ERR_CUDA;
 }
