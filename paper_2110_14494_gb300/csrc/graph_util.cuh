@@ -29,7 +29,8 @@ cudaError_t launch_pdl(void (*k)(P...), dim3 g, dim3 b, size_t smem, cudaStream_
     return cudaLaunchKernelEx(&cfg, k, args...);
 }
 
-// First error of a sequence of launches; launched() reports and clears it.
+// First error of a sequence of launches; launched() reports and clears it.  A
+// solve clears it at its start: one that gave up earlier may have left one.
 struct LaunchStatus {
     cudaError_t launch_err = cudaSuccess;
     void note(cudaError_t e) {

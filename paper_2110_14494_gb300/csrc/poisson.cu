@@ -889,6 +889,7 @@ void MG::release() {
 int MG::solve(const double* rho, const uint8_t* mask, double* phi, double h, double v_lo, double v_hi, double v_mask,
               double rtol, int max_cycles, int packed_prec, void* E4, float* Ex, float* Ey, float* Ez,
               cudaStream_t s, int* cycles_out, double* rel_out, double* host_norms) {
+    launch_err = cudaSuccess;
     const int nx = lx[0], ny = ly[0], nz = lz[0];
     const double h2e = h * h / kEps0;
     if (!persistent || !masks_ready) {
@@ -1013,6 +1014,7 @@ int MG::solve_mixed(const void* rho, bool rho64, const uint8_t* mask, float* phi
                     float* E4, float* Ex, float* Ey, float* Ez, cudaStream_t s, int* cycles_out, double* rel_out,
                     double* host_norms) {
     if (!mixed) return PIC_ERR_STATE;
+    launch_err = cudaSuccess;
     const int nx = lx[0], ny = ly[0], nz = lz[0], n = nx * ny * nz;
     if (!persistent || !masks_ready) {
         if (build_masks(mask, s) != cudaSuccess) return PIC_ERR_CUDA;
@@ -1127,6 +1129,7 @@ int MG::capture_solve_mixed(cudaStream_t cs, const float* rho, float* phi_hi, fl
                             int max_cycles, float* E4, int* cycles_dst, double* rel_dst, unsigned* err_dst,
                             unsigned err_bit, unsigned long long* kernels_dst, long long* fixed_kernels) {
     if (!mixed || !loop || !out_hi || !masks_ready) return PIC_ERR_STATE;
+    launch_err = cudaSuccess;
     const int nx = lx[0], ny = ly[0], nz = lz[0], n = nx * ny * nz;
     const MxBoundary bc{pair_of(v_lo), pair_of(v_hi), pair_of(v_mask)};
     const dim3 g3 = grid_mx3(nx, ny, nz), gf = grid_mxf(n);

@@ -772,6 +772,7 @@ void launch_resid(const AxiMG& a, cudaStream_t s, double* phi, const AxiCharge& 
 int AxiMG::solve(const AxiCharge& rho, const uint8_t* mask, double* phi, double h, double v_lo, double v_hi,
                  double v_mask, double rtol, int max_cycles, int packed_prec, void* E4, float* Er, float* Ez,
                  cudaStream_t s, int* cycles_out, double* rel_out, double* host_norms) {
+    launch_err = cudaSuccess;
     const int nr = lr[0], nz = lz[0];
     if (!persistent || !masks_ready) {
         if (build_masks(mask, s) != cudaSuccess) return PIC_ERR_CUDA;
@@ -868,6 +869,7 @@ int AxiMG::capture_solve(cudaStream_t cs, const AxiCharge& rho, double* phi, dou
                          double* rel_dst, unsigned* err_dst, unsigned err_bit, unsigned long long* kernels_dst,
                          long long* fixed_kernels) {
     if (!loop || !masks_ready || !cap_body[0] || !cap_body[1] || !cap_body[2]) return PIC_ERR_STATE;
+    launch_err = cudaSuccess;
     const int nr = lr[0], nz = lz[0];
     cudaGraph_t top = capturing_graph(cs), first = nullptr, more = nullptr, body = nullptr;
     if (!top) return PIC_ERR_CUDA;
